@@ -578,13 +578,13 @@ void fwd_t(const void* qkv, void* out, float* lse, int B, int S, int H, int Hkv,
 }
 
 // dK, dV of each KV head = fixed-order sums of its query heads' partials.
-__global__ void reduce_dkv_k(const float* __restrict__ part, bf16* __restrict__ dqkv, int NS, int H, int Hkv, int hd,
-                             float scale) {
+__global__ void reduce_dkv_k(const float* __restrict__ part, bf16* __restrict__ dqkv, int NS, int H, int Hkv, int rep,
+                             int hd, float scale) {
   pdl_wait();
   pdl_trigger();
-  const int rep = H / Hkv, ld = (H + 2 * Hkv) * hd;
+  const int ld = (H + 2 * Hkv) * hd;
   const size_t total = (size_t)NS * Hkv * (hd / 2);
-  const size_t HNS = (size_t)H * NS * hd;
+  const size_t HNS = (size_t)Hkv * rep * NS * hd;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
     const int dd = (int)(i % (hd / 2)) * 2;
     const int kvh = (int)((i / (hd / 2)) % Hkv);
@@ -630,7 +630,7 @@ void bwd_t(const void* qkv, const void* out, const void* dout, const float* lse,
   if (part) {
     const size_t total = (size_t)B * S * Hkv * (hd / 2);
     const int blocks = (int)std::min<size_t>((total + 255) / 256, 152 * 16);
-    launch_pdl(reduce_dkv_k, blocks, 256, 0, s, part, (bf16*)dqkv, B * S, H, Hkv, hd, scale);
+    launch_pdl(reduce_dkv_k, blocks, 256, 0, s, part, (bf16*)dqkv, B * S, H, Hkv, H / Hkv, hd, scale);
     cudaFreeAsync(part, s);
   }
 }
@@ -645,10 +645,11 @@ bool attn_fwd_tc(const void* qkv, void* out, float* lse, int B, int S, int H, in
   return true;
 }
 
-void launch_reduce_dkv(const float* part, void* dqkv, int NS, int H, int Hkv, int hd, float scale, cudaStream_t s) {
+void launch_reduce_dkv(const float* part, void* dqkv, int NS, int H, int Hkv, int rep, int hd, float scale,
+                       cudaStream_t s) {
   const size_t total = (size_t)NS * Hkv * (hd / 2);
   const int blocks = (int)std::min<size_t>((total + 255) / 256, 152 * 16);
-  launch_pdl(fa::reduce_dkv_k, blocks, 256, 0, s, part, (bf16*)dqkv, NS, H, Hkv, hd, scale);
+  launch_pdl(fa::reduce_dkv_k, blocks, 256, 0, s, part, (bf16*)dqkv, NS, H, Hkv, rep, hd, scale);
 }
 
 bool attn_bwd_tc(const void* qkv, const void* out, const void* dout, const float* lse, float* D, void* dqkv, int B, int S,

@@ -1,13 +1,15 @@
-// Causal attention on the 5th-generation tensor cores (sm_103a), head dims 64 and 128: a persistent
-// one-pass forward with lazy rescaling and a two-kernel backward (dQ; dK and dV) with 64-row (head dim
-// 128) or 128-row (head dim 64) inner blocks.
+// Causal attention on the 5th-generation tensor cores (sm_103a), head dims 64 and 128: a one-pass forward
+// with lazy rescaling and a two-kernel backward (dQ; dK and dV).
 //
-// A tile is 128 rows of one (batch, head): the forward runs at most one CTA per SM over a deal of the
-// tiles, the backward kernels one CTA per tile. TMA brings a tile's fixed operands once and the streamed
-// tiles through a stage ring (128-byte swizzle; a 3-D tensor map over [batch, token, feature] reads rows past
-// the sequence end as zeros); one elected lane of the MMA warp issues tcgen05.mma with fp32
-// accumulators in TMEM; the elementwise warps own TMEM lane quadrants (one row per thread). Every
-// mbarrier wait is bounded (about 2 s); on expiry the kernel raises ZL_DEVERR_TIMEOUT and unwinds.
+// A tile is 128 rows of one (batch, head), one CTA per tile, the longest tiles first. TMA brings a tile's
+// fixed operands once and streams the 128-row blocks of the other side (128-byte swizzle; a 3-D tensor map
+// over [batch, token, feature] reads rows past the sequence end as zeros); one elected lane of the MMA warp
+// issues tcgen05.mma with fp32 accumulators in TMEM; the elementwise warps own TMEM lane quadrants (one row
+// per thread). What the elementwise warps hand back to the tensor cores (P, dS) goes into TMEM as the A
+// operand, over the scores that it was made from, so it never passes through shared memory. The products
+// are issued in the order in which they depend on each other's TMEM columns, and the tensor pipe runs them
+// in that order. Every mbarrier wait is bounded (about 2 s); on expiry the kernel raises ZL_DEVERR_TIMEOUT
+// and unwinds.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <math.h>
@@ -22,10 +24,7 @@ namespace zl {
 namespace tg {
 using namespace tc;
 
-constexpr int QB = 128;     // query rows per CTA
-constexpr int KB = 128;     // keys per block
-constexpr int NSM = 8;      // softmax warps: two per TMEM lane quadrant, one 64-key half of a block each
-constexpr int NTHR = 64 + 32 * NSM;   // warp 0: TMA; warp 1: MMA and TMEM; warps 2-9: softmax and output
+constexpr int QB = 128;     // rows of a tile and of a streamed block
 constexpr float kL2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
 
 __device__ __forceinline__ float ex2(float x) {
@@ -34,105 +33,162 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
+__device__ __forceinline__ uint32_t pack2(float a, float b) {
+  __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<uint32_t*>(&h);
+}
+
+// Bounded wait of a producer that unwinds: lets a copy it issued land before the CTA exits.
+__device__ __forceinline__ void drain1(uint64_t* bar, int parity) {
+  if (parity < 0) return;
+  const unsigned long long t0 = gtimer();
+  while (!mbar_test(bar, (uint32_t)parity) && gtimer() - t0 < 100000000ull) {
+  }
+}
+
+__device__ __forceinline__ void tmem_alloc(uint32_t* dst, uint32_t cols) {
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(dst)), "r"(cols)
+               : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+
+// Warp 1 after the final __syncthreads: waits (bounded) for the last MMAs, frees the TMEM.
+__device__ __forceinline__ void tmem_release(uint64_t* fin, uint32_t tmem, uint32_t cols) {
+  if ((threadIdx.x & 31) == 0) drain1(fin, 0);
+  __syncwarp();
+  fence_after();
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols) : "memory");
+}
+
+// 128 rows x HD columns of one head from `m` into a tile of HD / 64 blocks of [128 rows][64 columns].
+template <int HD>
+__device__ __forceinline__ void load_tile(uint8_t* dst, const CUtensorMap* m, uint64_t* bar, int col, int row, int b) {
+#pragma unroll
+  for (int c = 0; c < HD / 64; ++c) tma3d(dst + c * 16384, m, bar, col + 64 * c, row, b);
+}
+
+// D[128 x 128] = A[128 x HD] B[128 x HD]^T, both K-major tiles of load_tile.
+template <int HD>
+__device__ __forceinline__ void mma_nt(uint32_t d, uint32_t a, uint32_t b) {
+  constexpr uint32_t id = idesc_f16(128, 128, false, false);
+#pragma unroll
+  for (int ks = 0; ks < HD / 16; ++ks) {
+    const uint32_t o = (ks / 4) * 16384 + (ks % 4) * 32;
+    mma_bf16(d, sdesc(a + o, 16, 1024), sdesc(b + o, 16, 1024), id, ks > 0 ? 1u : 0u);
+  }
+}
+
+// D[128 x HD] (+)= A[128 x 128] B[128 x HD]: A in TMEM, each group of CW score columns holding its bf16
+// pairs in the group's first CW / 2 columns; B a tile of load_tile read MN-major (16-row steps 2 KB apart).
+template <int HD, int CW>
+__device__ __forceinline__ void mma_ta(uint32_t d, uint32_t a, uint32_t b, bool acc) {
+  constexpr uint32_t id = idesc_f16(128, HD, false, true);
+#pragma unroll
+  for (int ks = 0; ks < 8; ++ks)
+    mma_bf16_ta(d, a + (ks * 16 / CW) * CW + (ks * 16 % CW) / 2, sdesc(b + ks * 2048, 16384, 1024), id,
+                (acc || ks > 0) ? 1u : 0u);
+}
+
+// This warp's 32 rows x HD fp32 columns at TMEM address `t` (this lane's row), times `f`, as bf16 through the
+// staging area `st` (HD / 64 boxes of 32 rows x 128 bytes, 128-byte swizzle) to rows row0 .. of `m`; box c0
+// .. c1 - 1 only. Rows past the sequence end are clipped by the map (a box with none inside is skipped).
+__device__ __forceinline__ void store_rows(uint32_t t, float f, uint8_t* st, const CUtensorMap* m, int col, int row0,
+                                           int b, int S, int c0, int c1, int lane) {
+  for (int c = c0; c < c1; ++c) {
+    uint8_t* box = st + c * 4096;
+    uint32_t u[64];
+    tmem_ld64u(t + (uint32_t)(64 * c), u);
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+      uint32_t w[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        w[e] = pack2(__uint_as_float(u[8 * p + 2 * e]) * f, __uint_as_float(u[8 * p + 2 * e + 1]) * f);
+      *reinterpret_cast<uint4*>(box + lane * 128 + ((p ^ (lane & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    fence_async_smem();
+    __syncwarp();
+    if (lane == 0 && row0 < S) tma_store3d(m, box, col + 64 * c, row0, b);
+  }
+  if (lane == 0) {   // the staging area outlives the copies' reads of it; the writes land by the kernel's end
+    bulk_commit();
+    bulk_wait_read0();
+  }
+}
+
 // ==============================================================================================
-// Forward, one pass with lazy rescaling, persistent. Each CTA takes its share of the tiles (128 query
-// rows of one batch and head; snake_tile's deal of a longest-first order), so the next tile's Q and K/V
-// loads and first S product overlap the current tile's last softmax block and its output; the output
-// accumulator O is double-buffered in TMEM by tile parity. Per 128-key block j: S_j = Q K_j^T (TMEM,
-// double-buffered), then O += P_{j-1} V_{j-1} (across a tile boundary: the previous tile's last block).
-// The softmax warps (two per lane quadrant, one 64-key half each) exchange the half-row maxima of S_j
-// through shared memory, so both take the same decisions, and keep a running maximum m that moves only
-// when the block maximum exceeds it by more than 8 (log2 units): P = 2^(s - m) then stays at most 256
-// (exact in fp32 sums, the usual bf16 rounding), and O and the row sum l are rescaled (in TMEM /
-// registers) only on such a move. The rescale happens after the wait that P's buffer is free, which is
-// also the completion of the previous P V product, so no product touches O meanwhile. At the end O / l
-// is the softmax-weighted sum and m + log2 l the row's log-sum-exp. Barrier phases follow global block
-// and tile counters, so they run on across tiles.
+// Forward, one pass with lazy rescaling. Per 128-key block j: S = Q K_j^T (TMEM), the softmax warps (half
+// a query row per thread, the two halves' maxima exchanged through shared memory) turn S into P =
+// 2^(s - m) in place, O += P V_j. The running maximum m moves only
+// when the block maximum exceeds it by more than 8 (log2 units): P then stays at most 256 (exact in fp32
+// sums, the usual bf16 rounding), and O and the row sum l are rescaled (in TMEM / registers) only on such
+// a move. At the end O / l is the softmax-weighted sum and m + log2 l the row's log-sum-exp.
+//
+// One block's chain S -> softmax -> P V is serial (S, P and O share 256 TMEM columns), and two CTAs per SM
+// (256 columns and at most 113 KB of shared memory each) fill each other's gaps: while one is in its
+// softmax, the other's products run. What bounds it: the softmax phase (about 1,450 cycles a block with its
+// hand-offs, of which 512 are the exponentials) against 1,024 cycles of products at head dim 128. Measured
+// against one persistent CTA per SM with P in shared memory: B 2, S 1024, 32 heads of 128 36.8 -> 22.7 us
+// (755 TFLOP/s); B 1, S 4096 1,250 TFLOP/s; B 4, S 2048, 32 / 4 heads of 64 103 us (665 TFLOP/s). Four
+// softmax warps with whole rows (no exchange) measured 1-3% slower.
 // ==============================================================================================
 template <int HD>
-struct F1Cfg {
-  static constexpr int QBYTES = QB * HD * 2;
-  static constexpr int KBYTES = KB * HD * 2;
-  static constexpr int VBYTES = KB * HD * 2;
-  static constexpr int STAGES = HD == 64 ? 4 : 2;
-  static constexpr int STAGE = KBYTES + VBYTES;
-  static constexpr int PBYTES = QB * KB * 2;
-  static constexpr int XBYTES = (2 * 2 * QB + 2 * QB) * 4;   // maxima [2 buffers][2 halves][rows], sums [2][rows]
-  static constexpr int SMEM = QBYTES + STAGES * STAGE + PBYTES + XBYTES + 256 + 1024;
-  static constexpr uint32_t OCOL = 256;                        // O of even tiles; odd tiles at OCOL + HD
-  static_assert(SMEM <= 232448, "shared memory per CTA");
-  static_assert(OCOL + 2 * HD <= 512, "TMEM columns");
+struct FCfg {
+  static constexpr int T = 128 * HD * 2;                // one tile
+  static constexpr int NST = HD == 64 ? 2 : 1;          // K and V buffers
+  static constexpr int XBYTES = (2 * 2 * 128 + 2 * 128) * 4;   // maxima [2 buffers][2 halves][rows], sums [2][rows]
+  static constexpr int SMEM = T + NST * 2 * T + XBYTES + 256 + 1024;
+  static constexpr int NSW = 8;                         // softmax warps: two per lane quadrant, 64 keys each
+  static constexpr int NTHR = 64 + 32 * NSW;            // TMA warp, MMA warp, softmax warps
+  static constexpr uint32_t OCOL = 128, COLS = 256;
+  static_assert(SMEM + 1024 <= 233472 / 2, "two CTAs per SM");
+  static_assert(OCOL + HD <= COLS, "TMEM columns");
 };
 
-// The it-th tile of CTA c among G: the tiles are sorted longest first and dealt out G at a time, the
-// direction alternating between deals (deal 0: c, deal 1: 2G - 1 - c, ...), so every CTA's long and short
-// tiles even out; past the last tile it returns a value >= every tile count (every later deal is past it
-// too).
-__device__ __forceinline__ int snake_tile(int it, int c, int G) {
-  return (it & 1) ? (it + 1) * G - 1 - c : it * G + c;
-}
-
-// Tile t of the longest-first order: query block (longest first), then batch, then head (heads that share
-// a K/V head are adjacent, so their K/V tiles come from L2).
-__device__ __forceinline__ void fwd_tile(int t, int H, int B, int nqb, int& h, int& b, int& qb) {
-  const int hb = H * B;
-  qb = nqb - 1 - t / hb;
-  const int r = t % hb;
-  h = r % H;
-  b = r / H;
-}
-
 template <int HD>
-__global__ void __launch_bounds__(NTHR, 1)
-    attn_fwd1_tg_k(const __grid_constant__ CUtensorMap tqk, const __grid_constant__ CUtensorMap tvv,
-                   bf16* __restrict__ out, float* __restrict__ lse, int S, int B, int H, int Hkv, float scale,
-                   unsigned* err) {
-  using C_ = F1Cfg<HD>;
+__global__ void __launch_bounds__(FCfg<HD>::NTHR, 2)
+    attn_fwd_k(const __grid_constant__ CUtensorMap tqkv, const __grid_constant__ CUtensorMap tout,
+               float* __restrict__ lse, int S, int H, int Hkv, float scale, unsigned* err) {
+  using C_ = FCfg<HD>;
+  constexpr int NST = C_::NST;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t* sq = smem;
-  uint8_t* sst = sq + C_::QBYTES;                      // stages: K tile, then V tile
-  uint8_t* sp = sst + C_::STAGES * C_::STAGE;          // P
-  float* xmax = (float*)(sp + C_::PBYTES);             // [2][2][QB]
-  float* xsum = xmax + 4 * QB;                         // [2][QB]
-  uint64_t* full = (uint64_t*)(xsum + 2 * QB);
-  uint64_t* empty = full + C_::STAGES;
-  uint64_t* qfull = empty + C_::STAGES;
-  uint64_t* qempty = qfull + 1;
-  uint64_t* sfull = qempty + 1;                        // [2]
-  uint64_t* sempty = sfull + 2;                        // [2]
-  uint64_t* pfull = sempty + 2;
-  uint64_t* pempty = pfull + 1;
-  uint64_t* ofull = pempty + 1;                        // [2]
-  uint64_t* oempty = ofull + 2;                        // [2]
-  uint64_t* fin = oempty + 2;
+  uint8_t* sq = smem;                       // Q, at the end the staging of the output
+  uint8_t* sk = sq + C_::T;                 // [NST] K
+  uint8_t* sv = sk + NST * C_::T;           // [NST] V
+  float* xmax = (float*)(sv + NST * C_::T);   // [2][2][128]
+  float* xsum = xmax + 512;                   // [2][128]
+  uint64_t* kfull = (uint64_t*)(xsum + 256);
+  uint64_t* kempty = kfull + NST;
+  uint64_t* vfull = kempty + NST;
+  uint64_t* vempty = vfull + NST;
+  uint64_t* qfull = vempty + NST;
+  uint64_t* sfull = qfull + 1;
+  uint64_t* pfull = sfull + 1;
+  uint64_t* ofull = pfull + 1;
+  uint64_t* fin = ofull + 1;
   uint32_t* tbase = (uint32_t*)(fin + 1);
   volatile int* abort_flag = (volatile int*)(tbase + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nqb = (S + QB - 1) / QB, ntiles = nqb * B * H;
-  const int group = H / Hkv;
+  const int h = blockIdx.x, b = blockIdx.y, qb = gridDim.z - 1 - blockIdx.z;   // longest first
+  const int kvh = h / (H / Hkv), q0 = qb * QB, nkb = qb + 1;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < C_::STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-    mbar_init(qfull, 1);
-    mbar_init(qempty, 1);
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&sfull[i], 1);
-      mbar_init(&sempty[i], NSM);
-      mbar_init(&ofull[i], 1);
-      mbar_init(&oempty[i], NSM);
+    for (int s = 0; s < NST; ++s) {
+      mbar_init(&kfull[s], 1);
+      mbar_init(&kempty[s], 1);
+      mbar_init(&vfull[s], 1);
+      mbar_init(&vempty[s], 1);
     }
-    mbar_init(pfull, NSM);
-    mbar_init(pempty, 1);
+    mbar_init(qfull, 1);
+    mbar_init(sfull, 1);
+    mbar_init(pfull, C_::NSW);
+    mbar_init(ofull, 1);
     mbar_init(fin, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tbase)), "r"(512u)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
+  if (warp == 1) tmem_alloc(tbase, C_::COLS);
   fence_before();
   __syncthreads();
   fence_after();
@@ -142,1369 +198,674 @@ __global__ void __launch_bounds__(NTHR, 1)
 
   if (warp == 0) {
     // ---------------- TMA producer (whole warp, one elected lane issues) ----------------
+    const int xk = (H + kvh) * HD, xv = (H + Hkv + kvh) * HD;
     const bool leader = elect_one();
+    if (leader) {
+      mbar_expect_tx(qfull, C_::T);
+      load_tile<HD>(sq, &tqkv, qfull, h * HD, q0, b);
+    }
     bool ok = true;
-    int qlast = -1;   // tile count of the last Q load issued
-    int issued[C_::STAGES];
+    int kp[NST], vp[NST];   // parity of the last fill of each buffer, -1 if none
 #pragma unroll
-    for (int s = 0; s < C_::STAGES; ++s) issued[s] = -1;
-    int stage = 0, it = 0;
-    uint32_t phase = 0;
-    for (; ok; ++it) {
-      const int t = snake_tile(it, blockIdx.x, gridDim.x);
-      if (t >= ntiles) break;
-      int h, b, qb;
-      fwd_tile(t, H, B, nqb, h, b, qb);
-      const int kvh = h / group, nkb = qb + 1;
-      const int xq = h * HD, xk = (H + kvh) * HD, xv = (H + Hkv + kvh) * HD;
-      // Q's buffer is free once the previous tile's S products have completed
-      if (!uwait(qempty, ((uint32_t)it & 1u) ^ 1u, abort_flag, err)) { ok = false; break; }
-      qlast = it;
+    for (int s = 0; s < NST; ++s) kp[s] = vp[s] = -1;
+    for (int j = 0; ok && j < nkb; ++j) {
+      const int st = j % NST;
+      const uint32_t ph = (uint32_t)(j / NST) & 1u;
+      if (!uwait(&kempty[st], ph ^ 1u, abort_flag, err)) { ok = false; break; }
+      kp[st] = (int)ph;
       if (leader) {
-        mbar_expect_tx(qfull, C_::QBYTES);
-#pragma unroll
-        for (int c = 0; c < HD / 64; ++c) tma3d(sq + c * 16384, &tqk, qfull, xq + 64 * c, qb * QB, b);
+        mbar_expect_tx(&kfull[st], C_::T);
+        load_tile<HD>(sk + st * C_::T, &tqkv, &kfull[st], xk, j * QB, b);
       }
       __syncwarp();
-      for (int j = 0; j < nkb; ++j) {
-        if (!uwait(&empty[stage], phase ^ 1u, abort_flag, err)) { ok = false; break; }
-        issued[stage] = (int)phase;
-        if (leader) {
-          mbar_expect_tx(&full[stage], C_::STAGE);
-          uint8_t* sk = sst + stage * C_::STAGE;
-          uint8_t* sv = sk + C_::KBYTES;
-#pragma unroll
-          for (int c = 0; c < HD / 64; ++c) tma3d(sk + c * 16384, &tqk, &full[stage], xk + 64 * c, j * KB, b);
-#pragma unroll
-          for (int kh = 0; kh < 2; ++kh)
-#pragma unroll
-            for (int nb = 0; nb < HD / 64; ++nb)
-              tma3d(sv + (kh * (HD / 64) + nb) * 8192, &tvv, &full[stage], xv + 64 * nb, j * KB + 64 * kh, b);
-        }
-        __syncwarp();
-        if (++stage == C_::STAGES) { stage = 0; phase ^= 1u; }
+      if (!uwait(&vempty[st], ph ^ 1u, abort_flag, err)) { ok = false; break; }
+      vp[st] = (int)ph;
+      if (leader) {
+        mbar_expect_tx(&vfull[st], C_::T);
+        load_tile<HD>(sv + st * C_::T, &tqkv, &vfull[st], xv, j * QB, b);
       }
+      __syncwarp();
     }
     if (!ok && lane == 0) {   // unwinding: let the copies in flight land before the CTA exits
-      for (int s = 0; s < C_::STAGES; ++s) {
-        if (issued[s] < 0) continue;
-        const unsigned long long t0 = gtimer();
-        while (!mbar_test(&full[s], (uint32_t)issued[s]) && gtimer() - t0 < 100000000ull) {
-        }
+#pragma unroll
+      for (int s = 0; s < NST; ++s) {
+        drain1(&kfull[s], kp[s]);
+        drain1(&vfull[s], vp[s]);
       }
-      if (qlast >= 0) {   // the last Q load (phase parity = its tile count)
-        const unsigned long long t0 = gtimer();
-        while (!mbar_test(qfull, (uint32_t)qlast & 1u) && gtimer() - t0 < 100000000ull) {
-        }
-      }
+      drain1(qfull, 0);
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer (whole warp, one elected lane issues and commits) ----------------
-    constexpr uint32_t id_s = idesc_f16(QB, KB, false, false);
-    constexpr uint32_t id_o = idesc_f16(QB, HD, false, true);
+    const uint32_t q_addr = su32(sq), k_addr = su32(sk), v_addr = su32(sv);
     const bool leader = elect_one();
-    bool ok = true;
-    int stage = 0, jg = 0, it = 0;
-    uint32_t phase = 0;
-    const uint32_t q_addr = su32(sq), p_addr = su32(sp);
-    // the P V product still to issue: block jl (of its tile) with global index pg, in stage pst, of tile pit
-    struct Pending { bool on; int jl, pg, pst, pit; bool last; } pend{false, 0, 0, 0, 0, false};
-    // O[tile parity] += P V: waits for P (and, on a tile's first block, for O's buffer to be read out);
-    // then the stage and P are free, and after a tile's last block O is complete
-    auto pv = [&](const Pending& p) -> bool {
-      if (!uwait(pfull, (uint32_t)p.pg & 1u, abort_flag, err)) return false;
-      const int ob = p.pit & 1;
-      if (p.jl == 0 && !uwait(&oempty[ob], ((uint32_t)(p.pit >> 1) & 1u) ^ 1u, abort_flag, err)) return false;
+    bool ok = uwait(qfull, 0, abort_flag, err);
+    for (int j = 0; ok && j < nkb; ++j) {
+      const int st = j % NST;
+      const uint32_t ph = (uint32_t)(j / NST) & 1u;
+      if (!uwait(&kfull[st], ph, abort_flag, err)) { ok = false; break; }
       fence_after();
-      if (leader) {
-        const uint32_t tso = tmem + C_::OCOL + (uint32_t)(ob * HD);
-        const uint32_t v_addr = su32(sst + p.pst * C_::STAGE + C_::KBYTES);
-#pragma unroll
-        for (int ks = 0; ks < KB / 16; ++ks) {
-          const int kh = ks / 4, kr = ks % 4;
-          const uint64_t ad = sdesc(p_addr + kh * 16384 + kr * 32, 16, 1024);
-          const uint64_t bd = sdesc(v_addr + kh * (HD / 64) * 8192 + kr * 2048, 8192, 1024);
-          mma_bf16(tso, ad, bd, id_o, (p.jl > 0 || ks > 0) ? 1u : 0u);
-        }
-        mma_commit(&empty[p.pst]);
-        mma_commit(pempty);
-        if (p.last) mma_commit(&ofull[ob]);
+      if (leader) {   // over P of block j - 1, which its P V product (issued before) reads first
+        mma_nt<HD>(tmem, q_addr, k_addr + st * C_::T);
+        mma_commit(sfull);
+        mma_commit(&kempty[st]);
       }
       __syncwarp();
-      return true;
-    };
-    for (; ok; ++it) {
-      const int t = snake_tile(it, blockIdx.x, gridDim.x);
-      if (t >= ntiles) break;
-      int h, b, qb;
-      fwd_tile(t, H, B, nqb, h, b, qb);
-      const int nkb = qb + 1;
-      if (!uwait(qfull, (uint32_t)it & 1u, abort_flag, err)) { ok = false; break; }
-      for (int j = 0; j < nkb; ++j, ++jg) {
-        const int sb = jg & 1;
-        if (!uwait(&sempty[sb], ((uint32_t)(jg >> 1) & 1u) ^ 1u, abort_flag, err) ||
-            !uwait(&full[stage], phase, abort_flag, err)) {
-          ok = false;
-          break;
-        }
-        fence_after();
-        if (leader) {
-          const uint32_t k_addr = su32(sst + stage * C_::STAGE);
-#pragma unroll
-          for (int ks = 0; ks < HD / 16; ++ks) {
-            const int kq = ks / 4, kr = ks % 4;
-            mma_bf16(tmem + sb * 128, sdesc(q_addr + kq * 16384 + kr * 32, 16, 1024),
-                     sdesc(k_addr + kq * 16384 + kr * 32, 16, 1024), id_s, ks > 0 ? 1u : 0u);
-          }
-          mma_commit(&sfull[sb]);
-          if (j == nkb - 1) mma_commit(qempty);   // Q is free once the tile's last S product completes
-        }
-        __syncwarp();
-        if (pend.on && !pv(pend)) { ok = false; break; }
-        pend = Pending{true, j, jg, stage, it, j == nkb - 1};
-        if (++stage == C_::STAGES) { stage = 0; phase ^= 1u; }
+      if (!uwait(&vfull[st], ph, abort_flag, err) || !uwait(pfull, (uint32_t)j & 1u, abort_flag, err)) {
+        ok = false;
+        break;
       }
+      fence_after();
+      if (leader) {
+        mma_ta<HD, 32>(tmem + C_::OCOL, tmem, v_addr + st * C_::T, j > 0);
+        mma_commit(&vempty[st]);
+        if (j == nkb - 1) mma_commit(ofull);
+      }
+      __syncwarp();
     }
-    if (ok && pend.on && !pv(pend)) ok = false;
     if (leader) mma_commit(fin);   // every MMA of the leader completes before TMEM is released
     __syncwarp();
   } else {
-    // ---------------- softmax and output: warps 2..9, one query row per thread ----------------
-    const int quad = warp & 3, half = (warp - 2) / 4;    // TMEM lane quadrant; key half of every block
-    const int r = quad * 32 + lane;                       // row within the block = TMEM lane
+    // ---------------- softmax and output: warps 2..9, half a query row per thread ----------------
+    const int quad = warp & 3, half = (warp - 2) >> 2;    // TMEM lane quadrant; key half of every block
+    const int r = quad * 32 + lane, q = q0 + r;
     const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
+    const uint32_t ts = trow + (uint32_t)(64 * half);
     const float sl2 = scale * kL2e;
-    // A failed wait only skips work: both warps of a quadrant still pass every named barrier (the same
-    // tiles and blocks on both).
+    const uint64_t SL2 = f2(sl2, sl2);
+    // After a failed wait the loop only runs on over whatever TMEM holds (both warps of a quadrant pass every
+    // named barrier); nothing is stored.
     bool ok = true;
-    int jg = 0, it = 0;
-    for (;; ++it) {
-      const int t = snake_tile(it, blockIdx.x, gridDim.x);
-      if (t >= ntiles) break;
-      int h, b, qb;
-      fwd_tile(t, H, B, nqb, h, b, qb);
-      const int nkb = qb + 1, q = qb * QB + r;
-      const uint32_t ocol = C_::OCOL + (uint32_t)((it & 1) * HD);
-      float m = -INFINITY, l = 0.f;                       // running maximum (log2 units), this half's sum
-      for (int j = 0; j < nkb; ++j, ++jg) {
-        const int sb = jg & 1;
-        if (ok && !uwait(&sfull[sb], (uint32_t)(jg >> 1) & 1u, abort_flag, err)) ok = false;
-        float v[64];
-        float mh = -INFINITY;
-        if (ok) {
-          fence_after();
-          const int kmax = min(q, S - 1) - j * KB - half * 64;   // last visible key offset in the half
-          const uint32_t tcol = trow + (uint32_t)(sb * 128 + half * 64);
-          tmem_ld32(tcol, v);
-          tmem_ld32(tcol + 32u, v + 32);
-          fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&sempty[sb]);
-#pragma unroll
-          for (int e = 0; e < 64; ++e) {
-            v[e] = e <= kmax ? v[e] * sl2 : -INFINITY;
-            mh = fmaxf(mh, v[e]);
-          }
-        }
-        // the partner half's maximum (double-buffered by block parity; one barrier per block)
-        float* xm = xmax + (jg & 1) * 2 * QB;
-        xm[half * QB + r] = mh;
-        asm volatile("bar.sync %0, 64;" ::"r"(1 + quad) : "memory");
-        if (!ok) continue;
-        const float mblk = fmaxf(mh, xm[(1 - half) * QB + r]);
-        const float mnew = fmaxf(m, mblk);
-        const bool move = mnew > m + 8.f;   // also true on the first block (m = -inf)
-        // P's buffer is free once the previous P V product has completed; O then holds blocks < j
-        if (!uwait(pempty, ((uint32_t)jg & 1u) ^ 1u, abort_flag, err)) { ok = false; continue; }
-        if (j > 0 && __any_sync(0xffffffffu, move)) {   // rescale this half of the O row (warp-wide TMEM access)
-          const float a = move ? ex2(m - mnew) : 1.f;
-          l *= a;
-          fence_after();
-#pragma unroll 1
-          for (int c = half * (HD / 2); c < (half + 1) * (HD / 2); c += 32) {
-            float o[32];
-            tmem_ld32(trow + ocol + (uint32_t)c, o);
-#pragma unroll
-            for (int e = 0; e < 32; ++e) o[e] *= a;
-            tmem_st32(trow + ocol + (uint32_t)c, o);
-          }
-        }
-        if (move) m = mnew;
-        uint8_t* prow = sp + half * 16384 + r * 128;   // this half's P block, row r (128-byte swizzle)
-        float sum = 0.f;
-#pragma unroll
-        for (int c = 0; c < 64; c += 32) {
-          uint32_t pk[16];
-#pragma unroll
-          for (int e = 0; e < 32; e += 2) {
-            const float p0 = ex2(v[c + e] - m), p1 = ex2(v[c + e + 1] - m);   // masked scores are -inf: 0
-            sum += p0 + p1;
-            __nv_bfloat162 hv = __floats2bfloat162_rn(p0, p1);
-            pk[e / 2] = *reinterpret_cast<uint32_t*>(&hv);
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int piece = c / 8 + u;
-            *reinterpret_cast<uint4*>(prow + ((piece ^ (r & 7)) << 4)) =
-                make_uint4(pk[4 * u], pk[4 * u + 1], pk[4 * u + 2], pk[4 * u + 3]);
-          }
-        }
-        l += sum;
-        fence_before();
-        fence_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(pfull);
-      }
-      // output: both halves use the same m; O / (l_0 + l_1), log-sum-exp m + log2(l_0 + l_1)
-      xsum[half * QB + r] = l;
-      asm volatile("bar.sync %0, 64;" ::"r"(1 + quad) : "memory");
-      if (!ok) continue;
-      const float lt = l + xsum[(1 - half) * QB + r];
-      const float inv = lt > 0.f ? 1.f / lt : 0.f;
-      if (!uwait(&ofull[it & 1], (uint32_t)(it >> 1) & 1u, abort_flag, err)) { ok = false; continue; }
+    float m = -INFINITY;                                  // running maximum (log2 units)
+    uint64_t la = f2(0.f, 0.f), lb = la;                  // this half's row sum, in four parts
+    for (int j = 0; j < nkb; ++j) {
+      if (ok && !uwait(sfull, (uint32_t)j & 1u, abort_flag, err)) ok = false;
+      uint32_t v[64];
+      float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
       fence_after();
-      bf16* orow = out + ((size_t)b * S + min(q, S - 1)) * ((size_t)H * HD) + (size_t)h * HD;
+      tmem_ld64u(ts, v);
+      if (j == nkb - 1) {   // the diagonal block: keys after the query (and past the end) are masked
+        const int kmax = min(q, S - 1) - j * QB - 64 * half;
+#pragma unroll
+        for (int e = 0; e < 64; ++e)
+          if (e > kmax) v[e] = 0xff800000u;
+      }
+#pragma unroll
+      for (int e = 0; e < 64; e += 4) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) mx[u] = fmaxf(mx[u], __uint_as_float(v[e + u]));
+      }
+      const float mh = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sl2;
+      // the partner half's maximum (double-buffered by block parity; one barrier per block)
+      float* xm = xmax + (j & 1) * 256;
+      xm[half * 128 + r] = mh;
+      asm volatile("bar.sync %0, 64;" ::"r"(1 + quad) : "memory");
+      const float mnew = fmaxf(m, fmaxf(mh, xm[(1 - half) * 128 + r]));
+      const bool move = mnew > m + 8.f;   // also true on the first block (m = -inf)
+      // the previous P V product completed before this S, which was issued after it
+      if (j > 0 && __any_sync(0xffffffffu, move)) {   // rescale this half of the O row (warp-wide TMEM access)
+        const float a = move ? ex2(m - mnew) : 1.f;
+        la = mul2(la, f2(a, a));
+        lb = mul2(lb, f2(a, a));
 #pragma unroll 1
-      for (int c = half * (HD / 2); c < (half + 1) * (HD / 2); c += 32) {   // every lane loads (tcgen05.ld is
-        float o[32];                                                        // warp-wide); rows >= S store nothing
-        tmem_ld32(trow + ocol + (uint32_t)c, o);
-        if (q < S) {
+        for (int c = half * (HD / 2); c < (half + 1) * (HD / 2); c += 32) {
+          float o[32];
+          tmem_ld32(trow + C_::OCOL + (uint32_t)c, o);
 #pragma unroll
-          for (int e = 0; e < 32; ++e) o[e] *= inv;
-#pragma unroll
-          for (int u = 0; u < 4; ++u) Vec8<bf16>::store(orow + c + 8 * u, o + 8 * u);
+          for (int e = 0; e < 32; ++e) o[e] *= a;
+          tmem_st32(trow + C_::OCOL + (uint32_t)c, o);
         }
       }
-      // this warp's half of O has been read: the buffer may take the tile after next
+      if (move) m = mnew;
+      const uint64_t NM = f2(-m, -m);
+#pragma unroll
+      for (int c = 0; c < 64; c += 32) {   // P of 32 keys into the first 16 of their 32 columns
+        uint32_t pk[16];
+#pragma unroll
+        for (int e = 0; e < 32; e += 4) {
+          const float2 x = uf2(fma2(f2(__uint_as_float(v[c + e]), __uint_as_float(v[c + e + 1])), SL2, NM));
+          const float2 y = uf2(fma2(f2(__uint_as_float(v[c + e + 2]), __uint_as_float(v[c + e + 3])), SL2, NM));
+          const float p0 = ex2(x.x), p1 = ex2(x.y), p2 = ex2(y.x), p3 = ex2(y.y);   // masked scores are -inf: 0
+          la = add2(la, f2(p0, p1));
+          lb = add2(lb, f2(p2, p3));
+          pk[e / 2] = pack2(p0, p1);
+          pk[e / 2 + 1] = pack2(p2, p3);
+        }
+        tmem_st16u(ts + (uint32_t)c, pk);
+      }
+      tmem_st_wait();
       fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&oempty[it & 1]);
+      if (lane == 0) mbar_arrive(pfull);
+    }
+    // output: both halves use the same m; O / (l_0 + l_1), log-sum-exp m + log2(l_0 + l_1)
+    const float2 ls = uf2(add2(la, lb));
+    xsum[half * 128 + r] = ls.x + ls.y;
+    asm volatile("bar.sync %0, 64;" ::"r"(1 + quad) : "memory");
+    const float lt = xsum[r] + xsum[128 + r];
+    const float inv = lt > 0.f ? 1.f / lt : 0.f;
+    if (ok && uwait(ofull, 0, abort_flag, err)) {
+      fence_after();
+      // one 64-column box per warp (head dim 64: the first warp of a quadrant has the only one)
+      if (half < HD / 64)
+        store_rows(trow + C_::OCOL, inv, sq + quad * (HD / 64) * 4096, &tout, h * HD, q0 + quad * 32, b, S, half,
+                   half + 1, lane);
       if (q < S && half == 0) lse[((size_t)b * H + h) * S + q] = (lt > 0.f ? m + log2f(lt) : INFINITY) * kLn2;
     }
   }
 
   fence_before();
   __syncthreads();
-  if (warp == 1) {
-    if (lane == 0) {
-      const unsigned long long t0 = gtimer();
-      while (!mbar_test(fin, 0) && gtimer() - t0 < 100000000ull) {
-      }
-    }
-    __syncwarp();
-    fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
-  }
+  if (warp == 1) tmem_release(fin, tmem, C_::COLS);
 }
 
 // ==============================================================================================
-// Backward: two kernels, each a fixed-order sum per output row (no atomics). Head dim 128 runs the
-// kernels of this section (64-row inner blocks); head dim 64 the 128-row variant that follows them.
-//   dQ kernel: one CTA per 128 queries; 64-key inner blocks j: S = Q K_j^T, dP = dO V_j^T (TMEM),
-//              dS = P * (dP - D) (shared memory, bf16), dQ += dS K_j (TMEM); also writes D = rowsum(dO * O).
-//   dK/dV kernel: one CTA per 128 keys; 64-query inner blocks i: S^T = K Q_i^T, dP^T = V dO_i^T,
-//              P^T and dS^T (shared memory), dV += P^T dO_i, dK += dS^T Q_i.
-// The 128 x 64 S / dP blocks are double-buffered in TMEM (columns 0 and 128, dP 64 columns after S); the
-// accumulators start at column 256. A 64-row tile of Q / dO / K / V is one K-major [64 x 64] block per 64
-// head-dim columns (8 KB each); the same bytes are the MN-major B operand of the accumulating product
-// (16-row steps 2 KB apart, head-dim blocks 8 KB apart).
+// Backward: two kernels, each a fixed-order sum per output row (no atomics), 128-row blocks.
+//   dQ kernel: one CTA per 128 queries; per key block j: S = Q K_j^T, dP = dO V_j^T,
+//              dS = P * (dP - D), dQ += dS K_j; also writes D = rowsum(dO * O).
+//   dK/dV kernel: one CTA per 128 keys of one KV head (and a share of its query heads); per query block i:
+//              S^T = K Q_i^T, dP^T = V dO_i^T, dV += P^T dO_i, dK += dS^T Q_i.
+// Sixteen elementwise warps, four per TMEM lane quadrant, 32 score columns each. P and dS go back into TMEM as
+// bf16, over the scores they come from (each warp over its own columns), as the A operands of the
+// accumulating products: nothing but the TMA tiles is in shared memory. The elementwise warps alternate
+// between the P and the dS phase of a block, and the products of the other operand run under each phase.
+// What bounds it: the P phase (about 1,100-1,400 cycles a block: TMEM reads, 512 cycles of exponentials, the
+// conversion and the TMEM writes), the hand-offs (about 280 cycles from the last warp's arrival to the next
+// product, 400-550 from the last product to the warps) and, at short sequences, each tile's first loads and
+// its output. Measured against P and dS in shared memory (64-row blocks at head dim 128), both kernels
+// together: B 2, S 1024, 32 heads of 128 127 -> 86 us; B 8, S 512, 12 heads of 64 46 -> 34.6 us; B 4, S 2048,
+// 32 / 4 heads of 64 540 -> 300 us. Eight elementwise warps with 64 columns each measured 10-15% slower.
 // ==============================================================================================
-constexpr int IB = 64;   // inner block rows
-constexpr int NEW = 16;  // elementwise warps: two groups of eight (two per TMEM lane quadrant, one
-                         // 32-column half each); group g takes the inner blocks of parity g
+constexpr int NEW = 16;
 constexpr int NTHR_B = 64 + 32 * NEW;
 
 template <int HD>
 struct BCfg {
-  static constexpr int T128 = 128 * HD * 2;
-  static constexpr int T64 = IB * HD * 2;
-  static constexpr int NST = HD == 64 ? 4 : 3;   // pipeline stages of (Q_i, dO_i) or (K_j, V_j)
-  static constexpr int OPB = 128 * IB * 2;       // one bf16 [128 x 64] operand (P^T, dS^T or dS)
-  // K, V | stages | P^T, dS^T double-buffered | stats (-lse2, D) per stage | barriers | alignment
-  static constexpr int SMEM_DKV = 2 * T128 + NST * 2 * T64 + 4 * OPB + NST * 2 * IB * 4 + 256 + 1024;
-  // Q, dO | stages | dS double-buffered | D quarters | barriers | alignment
-  static constexpr int SMEM_DQ = 2 * T128 + NST * 2 * T64 + 2 * OPB + 4 * 128 * 4 + 256 + 1024;
-  static_assert(SMEM_DKV <= 232448 && SMEM_DQ <= 232448, "shared memory per CTA");
+  static constexpr int T = 128 * HD * 2;
+  // dQ kernel: K_j is held until its dQ product, V_j only until its dP product
+  static constexpr int NK = HD == 64 ? 4 : 3, NV = HD == 64 ? 4 : 2;
+  static constexpr int SMEM_DQ = (2 + NK + NV) * T + 128 * 4 + 256 + 1024;   // Q, dO | K | V | D | barriers | align
+  // dK/dV kernel: stages of (Q_i, dO_i) with their statistics (-lse2, D), and score buffers
+  static constexpr int NST = HD == 64 ? 4 : 2, NSB = HD == 64 ? 2 : 1;
+  static constexpr int SMEM_DKV = (2 + NST * 2) * T + NST * 2 * 128 * 4 + 256 + 1024;
+  static_assert(SMEM_DQ <= 232448 && SMEM_DKV <= 232448, "shared memory per CTA");
+  static_assert((NSB + 1) * 128 + 2 * HD <= 512, "TMEM columns");
 };
 
-// Stores 16 bf16 values (32 bytes: 16-byte chunks 2 qu and 2 qu + 1) into row r of a swizzled
-// [128 x 64] K-major operand.
-__device__ __forceinline__ void put_row16(uint8_t* g, int qu, int r, const uint32_t* pk) {
-  uint8_t* row = g + r * 128;
-#pragma unroll
-  for (int u = 0; u < 2; ++u)
-    *reinterpret_cast<uint4*>(row + (((2 * qu + u) ^ (r & 7)) << 4)) =
-        make_uint4(pk[4 * u], pk[4 * u + 1], pk[4 * u + 2], pk[4 * u + 3]);
-}
-
-__device__ __forceinline__ uint32_t pack2(float a, float b) {
-  __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<uint32_t*>(&h);
-}
-
-// Lane 0 of the producer, after a failed wait: lets the copies it issued land (bounded) before exit.
-template <int N>
-__device__ __forceinline__ void drain(uint64_t* full, const int* issued, uint64_t* first) {
-  for (int s = 0; s < N; ++s) {
-    if (issued[s] < 0) continue;
-    const unsigned long long t0 = gtimer();
-    while (!mbar_test(&full[s], (uint32_t)issued[s]) && gtimer() - t0 < 100000000ull) {
-    }
-  }
-  const unsigned long long t0 = gtimer();
-  while (!mbar_test(first, 0) && gtimer() - t0 < 100000000ull) {
-  }
-}
-
-__device__ __forceinline__ void tmem_alloc512(uint32_t* dst) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(dst)), "r"(512u)
-               : "memory");
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-
-// Warp 1 after the final __syncthreads: waits (bounded) for the last MMAs, frees the TMEM.
-__device__ __forceinline__ void tmem_release(uint64_t* fin, uint32_t tmem) {
-  if ((threadIdx.x & 31) == 0) {
-    const unsigned long long t0 = gtimer();
-    while (!mbar_test(fin, 0) && gtimer() - t0 < 100000000ull) {
-    }
-  }
-  __syncwarp();
-  fence_after();
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
-}
-
-// The TMA and MMA warps run their loops with the whole warp (uniform control flow, so addresses and
-// descriptors stay in uniform registers); one elected lane issues each group of copies or products.
-
-// dQ (and D) kernel. Maps: tq = qkv in 128-row boxes, tdo = dO in 128-row boxes, tkv = qkv in 64-row boxes.
+// dQ (and D) kernel. TMEM: S 0-127, dP two buffers 128-383, dQ 384 .. 384 + HD.
 template <int HD>
 __global__ void __launch_bounds__(NTHR_B, 1)
-    attn_bwd_dq_tg_k(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CUtensorMap tdo,
-                     const __grid_constant__ CUtensorMap tkv, const bf16* __restrict__ outp,
-                     const bf16* __restrict__ dout, const float* __restrict__ lse, float* __restrict__ Dv,
-                     bf16* __restrict__ dqkv, int S, int H, int Hkv, float scale, unsigned* err) {
+    attn_bwd_dq_k(const __grid_constant__ CUtensorMap tqkv, const __grid_constant__ CUtensorMap tdo,
+                  const __grid_constant__ CUtensorMap tdq, const bf16* __restrict__ outp,
+                  const bf16* __restrict__ dout, const float* __restrict__ lse, float* __restrict__ Dv, int S, int H,
+                  int Hkv, float scale, unsigned* err) {
   using C_ = BCfg<HD>;
-  constexpr int NST = C_::NST;
+  constexpr int NK = C_::NK, NV = C_::NV;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t* sq = smem;
-  uint8_t* sdo = sq + C_::T128;
-  uint8_t* sst = sdo + C_::T128;                  // stage s: K_j at s * 2 T64, V_j after it
-  uint8_t* sds = sst + NST * 2 * C_::T64;         // dS, two buffers
-  float* dpart = (float*)(sds + 2 * C_::OPB);     // [4][128] quarters of D
-  uint64_t* full = (uint64_t*)(dpart + 512);
-  uint64_t* empty = full + NST;
-  uint64_t* qfull = empty + NST;
-  uint64_t* sfull = qfull + 1;                    // [2]
-  uint64_t* sempty = sfull + 2;                   // [2]
-  uint64_t* dsfull = sempty + 2;                  // [2]
-  uint64_t* dsempty = dsfull + 2;                 // [2]
-  uint64_t* ofull = dsempty + 2;
-  uint64_t* fin = ofull + 1;
-  uint32_t* tbase = (uint32_t*)(fin + 1);
-  volatile int* abort_flag = (volatile int*)(tbase + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int h = blockIdx.x, b = blockIdx.y, qb = gridDim.z - 1 - blockIdx.z;   // longest first
-  const int kvh = h / (H / Hkv);
-  const int q0 = qb * 128;
-  const int nkb = min(2 * qb + 2, (S + IB - 1) / IB);
-  const int ld = (H + 2 * Hkv) * HD, HDall = H * HD;
-  const int xq = h * HD, xk = (H + kvh) * HD, xv = (H + Hkv + kvh) * HD;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < NST; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-    mbar_init(qfull, 1);
-    for (int u = 0; u < 2; ++u) {   // buffer u is used by elementwise group u only
-      mbar_init(&sfull[u], 1);
-      mbar_init(&sempty[u], NEW / 2);
-      mbar_init(&dsfull[u], NEW / 2);
-      mbar_init(&dsempty[u], 1);
-    }
-    mbar_init(ofull, 1);
-    mbar_init(fin, 1);
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 1) tmem_alloc512(tbase);
-  fence_before();
-  __syncthreads();
-  fence_after();
-  const uint32_t tmem = *tbase;
-  pdl_wait();
-  pdl_trigger();
-
-  if (warp == 0) {
-    int issued[NST];
-#pragma unroll
-    for (int s = 0; s < NST; ++s) issued[s] = -1;
-    const bool leader = elect_one();
-    if (leader) {
-      mbar_expect_tx(qfull, 2 * C_::T128);
-#pragma unroll
-      for (int c = 0; c < HD / 64; ++c) {
-        tma3d(sq + c * 16384, &tq, qfull, xq + 64 * c, q0, b);
-        tma3d(sdo + c * 16384, &tdo, qfull, h * HD + 64 * c, q0, b);
-      }
-    }
-    int stage = 0;
-    uint32_t phase = 0;
-    bool ok = true;
-    for (int j = 0; j < nkb; ++j) {
-      if (!uwait(&empty[stage], phase ^ 1u, abort_flag, err)) { ok = false; break; }
-      issued[stage] = (int)phase;
-      if (leader) {
-        mbar_expect_tx(&full[stage], 2 * C_::T64);
-        uint8_t* st = sst + stage * 2 * C_::T64;
-#pragma unroll
-        for (int c = 0; c < HD / 64; ++c) {
-          tma3d(st + c * 8192, &tkv, &full[stage], xk + 64 * c, j * IB, b);
-          tma3d(st + C_::T64 + c * 8192, &tkv, &full[stage], xv + 64 * c, j * IB, b);
-        }
-      }
-      __syncwarp();
-      if (++stage == NST) { stage = 0; phase ^= 1u; }
-    }
-    if (!ok && lane == 0) drain<NST>(full, issued, qfull);
-  } else if (warp == 1) {
-    constexpr uint32_t id_s = idesc_f16(128, IB, false, false);
-    constexpr uint32_t id_q = idesc_f16(128, HD, false, true);
-    const uint32_t q_addr = su32(sq), do_addr = su32(sdo), ds_addr = su32(sds);
-    const bool leader = elect_one();   // issues every product and every commit that tracks them
-    bool ok = uwait(qfull, 0, abort_flag, err);
-    fence_after();
-    int stage = 0, pstage = 0;
-    uint32_t phase = 0;
-    auto dq = [&](int jb, int st) -> bool {   // dQ += dS_jb K_jb
-      const int db = jb & 1;
-      if (!uwait(&dsfull[db], (uint32_t)(jb >> 1) & 1u, abort_flag, err)) return false;
-      fence_after();
-      if (leader) {
-        const uint32_t k_addr = su32(sst + st * 2 * C_::T64), a_addr = ds_addr + db * C_::OPB;
-#pragma unroll
-        for (int ks = 0; ks < IB / 16; ++ks)
-          mma_bf16(tmem + 256, sdesc(a_addr + ks * 32, 16, 1024), sdesc(k_addr + ks * 2048, 8192, 1024), id_q,
-                   (jb > 0 || ks > 0) ? 1u : 0u);
-        mma_commit(&empty[st]);
-        mma_commit(&dsempty[db]);
-      }
-      __syncwarp();
-      return true;
-    };
-    for (int j = 0; ok && j < nkb; ++j) {
-      const int buf = j & 1;
-      if (!uwait(&sempty[buf], ((uint32_t)(j >> 1) & 1u) ^ 1u, abort_flag, err) ||
-          !uwait(&full[stage], phase, abort_flag, err)) {
-        ok = false;
-        break;
-      }
-      fence_after();
-      if (leader) {
-        const uint32_t k_addr = su32(sst + stage * 2 * C_::T64), v_addr = k_addr + C_::T64;
-        const uint32_t ts = tmem + (uint32_t)(buf * 128);
-#pragma unroll
-        for (int ks = 0; ks < HD / 16; ++ks) {
-          const int kq = ks / 4, kr = ks % 4;
-          mma_bf16(ts, sdesc(q_addr + kq * 16384 + kr * 32, 16, 1024), sdesc(k_addr + kq * 8192 + kr * 32, 16, 1024),
-                   id_s, ks > 0 ? 1u : 0u);
-          mma_bf16(ts + IB, sdesc(do_addr + kq * 16384 + kr * 32, 16, 1024),
-                   sdesc(v_addr + kq * 8192 + kr * 32, 16, 1024), id_s, ks > 0 ? 1u : 0u);
-        }
-        mma_commit(&sfull[buf]);
-      }
-      __syncwarp();
-      if (j > 0 && !dq(j - 1, pstage)) { ok = false; break; }
-      pstage = stage;
-      if (++stage == NST) { stage = 0; phase ^= 1u; }
-    }
-    if (ok && !dq(nkb - 1, pstage)) ok = false;
-    if (leader) {
-      if (ok) mma_commit(ofull);
-      mma_commit(fin);
-    }
-    __syncwarp();
-  } else {
-    const int quad = warp & 3, qu = (warp - 2) / 4;   // TMEM lane quadrant, 16-column quarter
-    const int r = quad * 32 + lane;
-    const int q = q0 + r, qc = min(q, S - 1);
-    const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
-    const size_t si = ((size_t)b * H + h) * S + qc;
-    const float nlse2 = q < S ? -lse[si] * kL2e : -INFINITY;
-    {   // D = rowsum(dO * O): each quarter sums a quarter of the row, fixed-order combination
-      const bf16* orow = outp + ((size_t)b * S + qc) * HDall + (size_t)h * HD + qu * (HD / 4);
-      const bf16* grow = dout + ((size_t)b * S + qc) * HDall + (size_t)h * HD + qu * (HD / 4);
-      float acc = 0.f;
-#pragma unroll
-      for (int c = 0; c < HD / 4; c += 8) {
-        float o8[8], g8[8];
-        Vec8<bf16>::load(orow + c, o8);
-        Vec8<bf16>::load(grow + c, g8);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc = fmaf(o8[e], g8[e], acc);
-      }
-      dpart[qu * 128 + r] = acc;
-    }
-    asm volatile("bar.sync 1, %0;" ::"n"(32 * NEW) : "memory");
-    const float Dq = (dpart[r] + dpart[128 + r]) + (dpart[256 + r] + dpart[384 + r]);
-    if (q < S && qu == 0) Dv[si] = Dq;
-    const uint64_t SL2 = f2(scale * kL2e, scale * kL2e), NL = f2(nlse2, nlse2), DD = f2(Dq, Dq);
-    const int qmin = q0 + quad * 32;   // smallest query row of this warp
-    // inner blocks alternate between the two groups, so each group's chain of waits, TMEM loads,
-    // arithmetic and stores has two blocks' time; a thread takes 32 columns in two 16-column passes
-    const int grp = (warp - 2) >> 3, half = ((warp - 2) >> 2) & 1;
-    bool ok = true;
-    for (int j = grp; j < nkb; j += 2) {
-      const int buf = j & 1;
-      if (!uwait(&sfull[buf], (uint32_t)(j >> 1) & 1u, abort_flag, err)) { ok = false; break; }
-      fence_after();
-      for (int sub = 0; sub < 2; ++sub) {
-        const int c0 = half * 32 + sub * 16;
-        float sv[16], dp[16];
-        tmem_ld16(trow + (uint32_t)(buf * 128 + c0), sv);
-        tmem_ld16(trow + (uint32_t)(buf * 128 + IB + c0), dp);
-        if (sub == 1) {
-          fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&sempty[buf]);
-        }
-        const int kbase = j * IB + c0;
-        const bool diag = kbase + 15 > qmin;   // warp-uniform: some column may lie above the diagonal
-        const int kmax = q - kbase;            // causal: columns e <= kmax
-        uint32_t pk[8];
-#pragma unroll
-        for (int e = 0; e < 16; e += 2) {
-          float2 x = uf2(fma2(f2(sv[e], sv[e + 1]), SL2, NL));
-          if (diag) {
-            if (e > kmax) x.x = -INFINITY;
-            if (e + 1 > kmax) x.y = -INFINITY;
-          }
-          const float p0 = ex2(x.x), p1 = ex2(x.y);
-          const float2 ds = uf2(mul2(f2(p0, p1), sub2(f2(dp[e], dp[e + 1]), DD)));
-          pk[e / 2] = pack2(ds.x, ds.y);
-        }
-        if (sub == 0 && !uwait(&dsempty[buf], ((uint32_t)(j >> 1) & 1u) ^ 1u, abort_flag, err)) { ok = false; break; }
-        put_row16(sds + buf * C_::OPB, c0 >> 4, r, pk);
-      }
-      if (!ok) break;
-      fence_async_smem();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&dsfull[buf]);
-    }
-    if (ok && uwait(ofull, 0, abort_flag, err)) {
-      fence_after();
-      bf16* drow = dqkv + ((size_t)b * S + qc) * ld + (size_t)h * HD;
-#pragma unroll
-      for (int c = qu * (HD / 4); c < (qu + 1) * (HD / 4); c += 16) {
-        float v[16];
-        tmem_ld16(trow + 256 + (uint32_t)c, v);
-        if (q < S) {
-#pragma unroll
-          for (int e = 0; e < 16; ++e) v[e] *= scale;
-          Vec8<bf16>::store(drow + c, v);
-          Vec8<bf16>::store(drow + c + 8, v + 8);
-        }
-      }
-    }
-  }
-  fence_before();
-  __syncthreads();
-  if (warp == 1) tmem_release(fin, tmem);
-}
-
-// dK / dV kernel. One CTA per 128 keys of one query head (grouped heads: fp32 partials
-// part[2][H][B*S][HD], dK unscaled, summed per group afterwards) or of one KV head (H == Hkv: bf16 straight
-// into dqkv). Maps: tkv = qkv in 128-row boxes, tq = qkv in 64-row boxes, tdo = dO in 64-row boxes.
-template <int HD>
-__global__ void __launch_bounds__(NTHR_B, 1)
-    attn_bwd_dkv_tg_k(const __grid_constant__ CUtensorMap tkv, const __grid_constant__ CUtensorMap tq,
-                      const __grid_constant__ CUtensorMap tdo, const float* __restrict__ lse,
-                      const float* __restrict__ Dv, bf16* __restrict__ dqkv, int S, int H, int Hkv, float scale,
-                      float* __restrict__ part, unsigned* err) {
-  using C_ = BCfg<HD>;
-  constexpr int NST = C_::NST;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t* sk = smem;
-  uint8_t* sv = sk + C_::T128;
-  uint8_t* sst = sv + C_::T128;                   // stage s: Q_i at s * 2 T64, dO_i after it
-  uint8_t* sp = sst + NST * 2 * C_::T64;          // buffer u: P^T at sp + 2 u OPB, dS^T after it
-  float* stats = (float*)(sp + 4 * C_::OPB);      // stage s: -lse2[64], D[64]
-  uint64_t* full = (uint64_t*)(stats + NST * 2 * IB);
-  uint64_t* empty = full + NST;
-  uint64_t* kvfull = empty + NST;
-  uint64_t* sfull = kvfull + 1;                   // [2]
-  uint64_t* sempty = sfull + 2;                   // [2]
-  uint64_t* pfull = sempty + 2;                   // [2]
-  uint64_t* pempty = pfull + 2;                   // [2]
-  uint64_t* ofull = pempty + 2;
-  uint64_t* fin = ofull + 1;
-  uint32_t* tbase = (uint32_t*)(fin + 1);
-  volatile int* abort_flag = (volatile int*)(tbase + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int h = blockIdx.x, b = blockIdx.y, kb = blockIdx.z;   // key block 0 (the longest) first
-  const int kvh = part ? h / (H / Hkv) : h;
-  const int k0 = kb * 128, i0 = 2 * kb;
-  const int nit = (S + IB - 1) / IB - i0;
-  const int ld = (H + 2 * Hkv) * HD;
-  const int xq = h * HD, xk = (H + kvh) * HD, xv = (H + Hkv + kvh) * HD;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < NST; ++s) { mbar_init(&full[s], 2); mbar_init(&empty[s], 1); }
-    mbar_init(kvfull, 1);
-    for (int u = 0; u < 2; ++u) {   // buffer u is used by elementwise group u only
-      mbar_init(&sfull[u], 1);
-      mbar_init(&sempty[u], NEW / 2);
-      mbar_init(&pfull[u], NEW / 2);
-      mbar_init(&pempty[u], 1);
-    }
-    mbar_init(ofull, 1);
-    mbar_init(fin, 1);
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 1) tmem_alloc512(tbase);
-  fence_before();
-  __syncthreads();
-  fence_after();
-  const uint32_t tmem = *tbase;
-  pdl_wait();
-  pdl_trigger();
-
-  if (warp == 0) {
-    // one elected lane: TMA of K, V once and of (Q_i, dO_i) per block; every lane: two of the block's
-    // -lse2 and D
-    int issued[NST];
-#pragma unroll
-    for (int s = 0; s < NST; ++s) issued[s] = -1;
-    const bool leader = elect_one();
-    if (leader) {
-      mbar_expect_tx(kvfull, 2 * C_::T128);
-#pragma unroll
-      for (int c = 0; c < HD / 64; ++c) {
-        tma3d(sk + c * 16384, &tkv, kvfull, xk + 64 * c, k0, b);
-        tma3d(sv + c * 16384, &tkv, kvfull, xv + 64 * c, k0, b);
-      }
-    }
-    int stage = 0;
-    uint32_t phase = 0;
-    bool ok = true;
-    // this lane's two statistics of the next block, loaded one block ahead
-    float nl[2], dd[2];
-    auto fetch = [&](int it) {
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int qq = (i0 + it) * IB + lane * 2 + u;
-        const size_t si = ((size_t)b * H + h) * S + (qq < S ? qq : 0);
-        nl[u] = qq < S ? -lse[si] * kL2e : -INFINITY;
-        dd[u] = qq < S ? Dv[si] : 0.f;
-      }
-    };
-    fetch(0);
-    for (int it = 0; it < nit; ++it) {
-      const int qi0 = (i0 + it) * IB;
-      if (!uwait(&empty[stage], phase ^ 1u, abort_flag, err)) { ok = false; break; }
-      issued[stage] = (int)phase;
-      if (leader) {
-        mbar_expect_tx(&full[stage], 2 * C_::T64);
-        uint8_t* st = sst + stage * 2 * C_::T64;
-#pragma unroll
-        for (int c = 0; c < HD / 64; ++c) {
-          tma3d(st + c * 8192, &tq, &full[stage], xq + 64 * c, qi0, b);
-          tma3d(st + C_::T64 + c * 8192, &tdo, &full[stage], h * HD + 64 * c, qi0, b);
-        }
-      }
-      float* sl = stats + stage * 2 * IB;
-      *reinterpret_cast<float2*>(sl + lane * 2) = make_float2(nl[0], nl[1]);
-      *reinterpret_cast<float2*>(sl + IB + lane * 2) = make_float2(dd[0], dd[1]);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&full[stage]);
-      if (it + 1 < nit) fetch(it + 1);
-      if (++stage == NST) { stage = 0; phase ^= 1u; }
-    }
-    if (!ok && lane == 0) drain<NST>(full, issued, kvfull);
-  } else if (warp == 1) {
-    constexpr uint32_t id_s = idesc_f16(128, IB, false, false);
-    constexpr uint32_t id_g = idesc_f16(128, HD, false, true);
-    const uint32_t k_addr = su32(sk), v_addr = su32(sv), p_addr = su32(sp);
-    const bool leader = elect_one();   // issues every product and every commit that tracks them
-    bool ok = uwait(kvfull, 0, abort_flag, err);
-    fence_after();
-    int stage = 0, pstage = 0;
-    uint32_t phase = 0;
-    auto grads = [&](int ib, int st) -> bool {   // dV += P^T dO_ib, dK += dS^T Q_ib
-      const int pb = ib & 1;
-      if (!uwait(&pfull[pb], (uint32_t)(ib >> 1) & 1u, abort_flag, err)) return false;
-      fence_after();
-      if (leader) {
-        const uint32_t qa = su32(sst + st * 2 * C_::T64), da = qa + C_::T64;
-        const uint32_t pa = p_addr + pb * 2 * C_::OPB, dsa = pa + C_::OPB;
-#pragma unroll
-        for (int ks = 0; ks < IB / 16; ++ks) {
-          const uint32_t acc = (ib > 0 || ks > 0) ? 1u : 0u;
-          mma_bf16(tmem + 256, sdesc(pa + ks * 32, 16, 1024), sdesc(da + ks * 2048, 8192, 1024), id_g, acc);
-          mma_bf16(tmem + 256 + HD, sdesc(dsa + ks * 32, 16, 1024), sdesc(qa + ks * 2048, 8192, 1024), id_g, acc);
-        }
-        mma_commit(&empty[st]);
-        mma_commit(&pempty[pb]);
-      }
-      __syncwarp();
-      return true;
-    };
-    for (int it = 0; ok && it < nit; ++it) {
-      const int buf = it & 1;
-      if (!uwait(&sempty[buf], ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag, err) ||
-          !uwait(&full[stage], phase, abort_flag, err)) {
-        ok = false;
-        break;
-      }
-      fence_after();
-      if (leader) {
-        const uint32_t qa = su32(sst + stage * 2 * C_::T64), da = qa + C_::T64;
-        const uint32_t ts = tmem + (uint32_t)(buf * 128);
-#pragma unroll
-        for (int ks = 0; ks < HD / 16; ++ks) {
-          const int kq = ks / 4, kr = ks % 4;
-          mma_bf16(ts, sdesc(k_addr + kq * 16384 + kr * 32, 16, 1024), sdesc(qa + kq * 8192 + kr * 32, 16, 1024),
-                   id_s, ks > 0 ? 1u : 0u);
-          mma_bf16(ts + IB, sdesc(v_addr + kq * 16384 + kr * 32, 16, 1024),
-                   sdesc(da + kq * 8192 + kr * 32, 16, 1024), id_s, ks > 0 ? 1u : 0u);
-        }
-        mma_commit(&sfull[buf]);
-      }
-      __syncwarp();
-      if (it > 0 && !grads(it - 1, pstage)) { ok = false; break; }
-      pstage = stage;
-      if (++stage == NST) { stage = 0; phase ^= 1u; }
-    }
-    if (ok && !grads(nit - 1, pstage)) ok = false;
-    if (leader) {
-      if (ok) mma_commit(ofull);
-      mma_commit(fin);
-    }
-    __syncwarp();
-  } else {
-    const int quad = warp & 3, qu = (warp - 2) / 4;   // TMEM lane quadrant, 16-column quarter
-    const int r = quad * 32 + lane;                    // key row = TMEM lane
-    const int key = k0 + r;
-    const int kmaxw = k0 + quad * 32 + 31;             // largest key of this warp
-    const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
-    const uint64_t SL2 = f2(scale * kL2e, scale * kL2e);
-    // Only the causal mask is applied: queries >= S have -lse2 = -inf (P = 0) and D = 0, and rows of
-    // keys >= S are never stored. Inner blocks alternate between the two groups (as in the dQ kernel).
-    const int grp = (warp - 2) >> 3, half = ((warp - 2) >> 2) & 1;
-    bool ok = true;
-    for (int it = grp; it < nit; it += 2) {
-      const int buf = it & 1, stage = it % NST;
-      const uint32_t phase = (uint32_t)(it / NST) & 1u;
-      if (!uwait(&sfull[buf], (uint32_t)(it >> 1) & 1u, abort_flag, err)) { ok = false; break; }
-      fence_after();
-      // this stage's statistics: its full phase has completed (the S MMA waited on it); the wait orders
-      // the producer's stores before these loads
-      if (!uwait(&full[stage], phase, abort_flag, err)) { ok = false; break; }
-      for (int sub = 0; sub < 2; ++sub) {
-        const int c0 = half * 32 + sub * 16;
-        float sv[16], dp[16];
-        tmem_ld16(trow + (uint32_t)(buf * 128 + c0), sv);
-        tmem_ld16(trow + (uint32_t)(buf * 128 + IB + c0), dp);
-        if (sub == 1) {
-          fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&sempty[buf]);
-        }
-        const float4* sl4 = reinterpret_cast<const float4*>(stats + stage * 2 * IB + c0);
-        const float4* sd4 = reinterpret_cast<const float4*>(stats + stage * 2 * IB + IB + c0);
-        float4 l[4], d[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) { l[u] = sl4[u]; d[u] = sd4[u]; }
-        const int qbase = (i0 + it) * IB + c0;   // query of column 0 of these 16
-        const bool diag = qbase < kmaxw;          // warp-uniform: some column may precede its key
-        const int qlo = key - qbase;              // causal: columns e >= qlo
-        uint32_t pk[8], dk[8];
-#pragma unroll
-        for (int e4 = 0; e4 < 4; ++e4) {
-          const int e = 4 * e4;
-          float2 xa = uf2(fma2(f2(sv[e], sv[e + 1]), SL2, f2(l[e4].x, l[e4].y)));
-          float2 xb = uf2(fma2(f2(sv[e + 2], sv[e + 3]), SL2, f2(l[e4].z, l[e4].w)));
-          if (diag) {
-            if (e < qlo) xa.x = -INFINITY;
-            if (e + 1 < qlo) xa.y = -INFINITY;
-            if (e + 2 < qlo) xb.x = -INFINITY;
-            if (e + 3 < qlo) xb.y = -INFINITY;
-          }
-          const float p0 = ex2(xa.x), p1 = ex2(xa.y), p2 = ex2(xb.x), p3 = ex2(xb.y);
-          const float2 da = uf2(mul2(f2(p0, p1), sub2(f2(dp[e], dp[e + 1]), f2(d[e4].x, d[e4].y))));
-          const float2 db = uf2(mul2(f2(p2, p3), sub2(f2(dp[e + 2], dp[e + 3]), f2(d[e4].z, d[e4].w))));
-          pk[2 * e4] = pack2(p0, p1);
-          pk[2 * e4 + 1] = pack2(p2, p3);
-          dk[2 * e4] = pack2(da.x, da.y);
-          dk[2 * e4 + 1] = pack2(db.x, db.y);
-        }
-        if (sub == 0 && !uwait(&pempty[buf], ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag, err)) { ok = false; break; }
-        put_row16(sp + buf * 2 * C_::OPB, c0 >> 4, r, pk);
-        put_row16(sp + buf * 2 * C_::OPB + C_::OPB, c0 >> 4, r, dk);
-      }
-      if (!ok) break;
-      fence_async_smem();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&pfull[buf]);
-    }
-    if (ok && uwait(ofull, 0, abort_flag, err)) {
-      fence_after();
-      const int kc = min(key, S - 1);
-      const size_t NS = (size_t)gridDim.y * S;
-#pragma unroll
-      for (int c = qu * (HD / 4); c < (qu + 1) * (HD / 4); c += 16) {
-        float gv[16], gk[16];
-        tmem_ld16(trow + 256 + (uint32_t)c, gv);
-        tmem_ld16(trow + 256 + HD + (uint32_t)c, gk);
-        if (key < S) {
-          if (part) {
-            float* pk2 = part + ((size_t)h * NS + (size_t)b * S + kc) * HD + c;
-            float* pv2 = pk2 + (size_t)H * NS * HD;
-#pragma unroll
-            for (int e = 0; e < 16; e += 4) {
-              *reinterpret_cast<float4*>(pk2 + e) = make_float4(gk[e], gk[e + 1], gk[e + 2], gk[e + 3]);
-              *reinterpret_cast<float4*>(pv2 + e) = make_float4(gv[e], gv[e + 1], gv[e + 2], gv[e + 3]);
-            }
-          } else {
-            bf16* dkr = dqkv + ((size_t)b * S + kc) * ld + (size_t)xk + c;
-            bf16* dvr = dqkv + ((size_t)b * S + kc) * ld + (size_t)xv + c;
-#pragma unroll
-            for (int e = 0; e < 16; ++e) gk[e] *= scale;
-            Vec8<bf16>::store(dkr, gk);
-            Vec8<bf16>::store(dkr + 8, gk + 8);
-            Vec8<bf16>::store(dvr, gv);
-            Vec8<bf16>::store(dvr + 8, gv + 8);
-          }
-        }
-      }
-    }
-  }
-  fence_before();
-  __syncthreads();
-  if (warp == 1) tmem_release(fin, tmem);
-}
-
-// ----------------------------------------------------------------------------------------------
-// Backward with 128-wide inner blocks (head dim 64): per 128 keys (dQ) or 128 queries (dK / dV), one
-// round of hand-offs and 24 products instead of two rounds and 32. S / dP are single-buffered in TMEM
-// (columns 0 and 128): the elementwise warps read them into registers in two 16-column passes and
-// release them after the second, so the next block's products still overlap the arithmetic. Sixteen
-// elementwise warps, four per lane quadrant, 32 columns each. A 128-row tile of Q / dO / K / V is one
-// K-major [128 x 64] block per 64 head-dim columns (16 KB); as the MN-major B operand of the
-// accumulating product its 16-row steps are 2 KB apart.
-// ----------------------------------------------------------------------------------------------
-constexpr int WB = 128;   // inner block rows
-
-template <int HD>
-struct WCfg {
-  static constexpr int T128 = 128 * HD * 2;
-  static constexpr int NST = 3;             // stages of (Q_i, dO_i) or (K_j, V_j), 128 rows each
-  static constexpr int OPB = 128 * WB * 2;  // one bf16 [128 x 128] operand: two 64-column halves of 16 KB
-  // K, V | stages | P^T, dS^T | statistics (-lse2, D) per stage | barriers | alignment
-  static constexpr int SMEM_DKV = 2 * T128 + NST * 2 * T128 + 2 * OPB + NST * 2 * WB * 4 + 256 + 1024;
-  // Q, dO | stages | dS | D quarters | barriers | alignment
-  static constexpr int SMEM_DQ = 2 * T128 + NST * 2 * T128 + OPB + 4 * 128 * 4 + 256 + 1024;
-  static_assert(SMEM_DKV <= 232448 && SMEM_DQ <= 232448, "shared memory per CTA");
-};
-
-// 16 bf16 values (columns 16 s .. 16 s + 15 of a thread's 32, qq the 32-column quarter) into row r of a
-// swizzled [128 x 128] K-major operand (two 64-column halves of 16 KB).
-__device__ __forceinline__ void put_row16w(uint8_t* g, int qq, int sub, int r, const uint32_t* pk) {
-  uint8_t* row = g + (qq >> 1) * 16384 + r * 128;
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int chunk = ((qq & 1) * 4 + sub * 2 + u) ^ (r & 7);
-    *reinterpret_cast<uint4*>(row + (chunk << 4)) = make_uint4(pk[4 * u], pk[4 * u + 1], pk[4 * u + 2], pk[4 * u + 3]);
-  }
-}
-
-// dQ (and D) kernel, 128-key inner blocks. Maps: tq, tdo, tkv, all in 128-row boxes.
-template <int HD>
-__global__ void __launch_bounds__(NTHR_B, 1)
-    attn_bwd_dq_w_k(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CUtensorMap tdo,
-                    const __grid_constant__ CUtensorMap tkv, const bf16* __restrict__ outp,
-                    const bf16* __restrict__ dout, const float* __restrict__ lse, float* __restrict__ Dv,
-                    bf16* __restrict__ dqkv, int S, int H, int Hkv, float scale, unsigned* err) {
-  using C_ = WCfg<HD>;
-  constexpr int NST = C_::NST;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t* sq = smem;
-  uint8_t* sdo = sq + C_::T128;
-  uint8_t* sst = sdo + C_::T128;                  // stage s: K_j at s * 2 T128, V_j after it
-  uint8_t* sds = sst + NST * 2 * C_::T128;        // dS
-  float* dpart = (float*)(sds + C_::OPB);         // [4][128] quarters of D
-  uint64_t* full = (uint64_t*)(dpart + 512);
-  uint64_t* empty = full + NST;
-  uint64_t* qfull = empty + NST;
+  uint8_t* sq = smem;                             // Q, at the end the staging of dQ
+  uint8_t* sdo = sq + C_::T;
+  uint8_t* sk = sdo + C_::T;                      // [NK] K
+  uint8_t* sv = sk + NK * C_::T;                  // [NV] V
+  float* sD = (float*)(sv + NV * C_::T);          // [128] D
+  uint64_t* kfull = (uint64_t*)(sD + 128);
+  uint64_t* kempty = kfull + NK;
+  uint64_t* vfull = kempty + NK;
+  uint64_t* vempty = vfull + NV;
+  uint64_t* qfull = vempty + NV;
   uint64_t* sfull = qfull + 1;
-  uint64_t* sempty = sfull + 1;
-  uint64_t* dsfull = sempty + 1;
-  uint64_t* dsempty = dsfull + 1;
-  uint64_t* ofull = dsempty + 1;
+  uint64_t* sread = sfull + 1;                    // the elementwise warps have S in registers
+  uint64_t* dpfull = sread + 1;                   // [2]
+  uint64_t* dsfull = dpfull + 2;
+  uint64_t* ofull = dsfull + 1;
   uint64_t* fin = ofull + 1;
   uint32_t* tbase = (uint32_t*)(fin + 1);
   volatile int* abort_flag = (volatile int*)(tbase + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int h = blockIdx.x, b = blockIdx.y, qb = gridDim.z - 1 - blockIdx.z;   // longest first
-  const int kvh = h / (H / Hkv);
-  const int q0 = qb * 128;
-  const int nkb = min(qb + 1, (S + WB - 1) / WB);
-  const int ld = (H + 2 * Hkv) * HD, HDall = H * HD;
-  const int xq = h * HD, xk = (H + kvh) * HD, xv = (H + Hkv + kvh) * HD;
+  const int kvh = h / (H / Hkv), q0 = qb * QB, nkb = qb + 1;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < NST; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+    for (int s = 0; s < NK; ++s) { mbar_init(&kfull[s], 1); mbar_init(&kempty[s], 1); }
+    for (int s = 0; s < NV; ++s) { mbar_init(&vfull[s], 1); mbar_init(&vempty[s], 1); }
     mbar_init(qfull, 1);
     mbar_init(sfull, 1);
-    mbar_init(sempty, NEW);
+    mbar_init(sread, NEW);
+    mbar_init(&dpfull[0], 1);
+    mbar_init(&dpfull[1], 1);
     mbar_init(dsfull, NEW);
-    mbar_init(dsempty, 1);
     mbar_init(ofull, 1);
     mbar_init(fin, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) tmem_alloc512(tbase);
+  if (warp == 1) tmem_alloc(tbase, 512);
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tbase;   // S: columns 0-127, dP: 128-255, dQ: 256 + HD
+  const uint32_t tmem = *tbase;
+  constexpr uint32_t DP = 128, DQ = 384;
   pdl_wait();
   pdl_trigger();
 
   if (warp == 0) {
-    int issued[NST];
-#pragma unroll
-    for (int s = 0; s < NST; ++s) issued[s] = -1;
+    const int xk = (H + kvh) * HD, xv = (H + Hkv + kvh) * HD;
     const bool leader = elect_one();
     if (leader) {
-      mbar_expect_tx(qfull, 2 * C_::T128);
-#pragma unroll
-      for (int c = 0; c < HD / 64; ++c) {
-        tma3d(sq + c * 16384, &tq, qfull, xq + 64 * c, q0, b);
-        tma3d(sdo + c * 16384, &tdo, qfull, h * HD + 64 * c, q0, b);
-      }
+      mbar_expect_tx(qfull, 2 * C_::T);
+      load_tile<HD>(sq, &tqkv, qfull, h * HD, q0, b);
+      load_tile<HD>(sdo, &tdo, qfull, h * HD, q0, b);
     }
-    int stage = 0;
-    uint32_t phase = 0;
     bool ok = true;
-    for (int j = 0; j < nkb; ++j) {
-      if (!uwait(&empty[stage], phase ^ 1u, abort_flag, err)) { ok = false; break; }
-      issued[stage] = (int)phase;
-      if (leader) {
-        mbar_expect_tx(&full[stage], 2 * C_::T128);
-        uint8_t* st = sst + stage * 2 * C_::T128;
+    int kp[NK], vp[NV];   // parity of the last fill of each buffer, -1 if none
 #pragma unroll
-        for (int c = 0; c < HD / 64; ++c) {
-          tma3d(st + c * 16384, &tkv, &full[stage], xk + 64 * c, j * WB, b);
-          tma3d(st + C_::T128 + c * 16384, &tkv, &full[stage], xv + 64 * c, j * WB, b);
-        }
+    for (int s = 0; s < NK; ++s) kp[s] = -1;
+#pragma unroll
+    for (int s = 0; s < NV; ++s) vp[s] = -1;
+    for (int j = 0; j < nkb; ++j) {
+      const int ks = j % NK, vs = j % NV;
+      const uint32_t kph = (uint32_t)(j / NK) & 1u, vph = (uint32_t)(j / NV) & 1u;
+      if (!uwait(&kempty[ks], kph ^ 1u, abort_flag, err)) { ok = false; break; }
+      kp[ks] = (int)kph;
+      if (leader) {
+        mbar_expect_tx(&kfull[ks], C_::T);
+        load_tile<HD>(sk + ks * C_::T, &tqkv, &kfull[ks], xk, j * QB, b);
       }
       __syncwarp();
-      if (++stage == NST) { stage = 0; phase ^= 1u; }
+      if (!uwait(&vempty[vs], vph ^ 1u, abort_flag, err)) { ok = false; break; }
+      vp[vs] = (int)vph;
+      if (leader) {
+        mbar_expect_tx(&vfull[vs], C_::T);
+        load_tile<HD>(sv + vs * C_::T, &tqkv, &vfull[vs], xv, j * QB, b);
+      }
+      __syncwarp();
     }
-    if (!ok && lane == 0) drain<NST>(full, issued, qfull);
+    if (!ok && lane == 0) {   // unwinding: let the copies in flight land before the CTA exits
+#pragma unroll
+      for (int s = 0; s < NK; ++s) drain1(&kfull[s], kp[s]);
+#pragma unroll
+      for (int s = 0; s < NV; ++s) drain1(&vfull[s], vp[s]);
+      drain1(qfull, 0);
+    }
   } else if (warp == 1) {
-    constexpr uint32_t id_s = idesc_f16(128, WB, false, false);
-    constexpr uint32_t id_q = idesc_f16(128, HD, false, true);
-    const uint32_t q_addr = su32(sq), do_addr = su32(sdo), ds_addr = su32(sds);
+    // S_{j+1} and dP_{j+1} are issued as soon as S_j has been read into registers, ahead of dQ += dS_j K_j, so
+    // they run under the dS phase of block j. dP_{j+1} overwrites dS_{j-1}, whose product was issued before.
+    const uint32_t q_addr = su32(sq), do_addr = su32(sdo), k_addr = su32(sk), v_addr = su32(sv);
     const bool leader = elect_one();   // issues every product and every commit that tracks them
     bool ok = uwait(qfull, 0, abort_flag, err);
-    fence_after();
-    int stage = 0, pstage = 0;
-    uint32_t phase = 0;
-    auto dq = [&](int jb, int st) -> bool {   // dQ += dS_jb K_jb
-      if (!uwait(dsfull, (uint32_t)(jb & 1), abort_flag, err)) return false;
+    auto scores = [&](int j) -> bool {   // S_j, then dP_j
+      const int ks = j % NK, vs = j % NV;
+      if (!uwait(&kfull[ks], (uint32_t)(j / NK) & 1u, abort_flag, err)) return false;
       fence_after();
       if (leader) {
-        const uint32_t k_addr = su32(sst + st * 2 * C_::T128);
-#pragma unroll
-        for (int ks = 0; ks < WB / 16; ++ks)
-          mma_bf16(tmem + 256, sdesc(ds_addr + (ks / 4) * 16384 + (ks % 4) * 32, 16, 1024),
-                   sdesc(k_addr + ks * 2048, 16384, 1024), id_q, (jb > 0 || ks > 0) ? 1u : 0u);
-        mma_commit(&empty[st]);
-        mma_commit(dsempty);
-      }
-      __syncwarp();
-      return true;
-    };
-    for (int j = 0; ok && j < nkb; ++j) {
-      if (!uwait(sempty, ((uint32_t)j & 1u) ^ 1u, abort_flag, err) || !uwait(&full[stage], phase, abort_flag, err)) {
-        ok = false;
-        break;
-      }
-      fence_after();
-      if (leader) {
-        const uint32_t k_addr = su32(sst + stage * 2 * C_::T128), v_addr = k_addr + C_::T128;
-#pragma unroll
-        for (int ks = 0; ks < HD / 16; ++ks) {
-          const int kq = ks / 4, kr = ks % 4;
-          mma_bf16(tmem, sdesc(q_addr + kq * 16384 + kr * 32, 16, 1024), sdesc(k_addr + kq * 16384 + kr * 32, 16, 1024),
-                   id_s, ks > 0 ? 1u : 0u);
-          mma_bf16(tmem + 128, sdesc(do_addr + kq * 16384 + kr * 32, 16, 1024),
-                   sdesc(v_addr + kq * 16384 + kr * 32, 16, 1024), id_s, ks > 0 ? 1u : 0u);
-        }
+        mma_nt<HD>(tmem, q_addr, k_addr + ks * C_::T);
         mma_commit(sfull);
       }
       __syncwarp();
-      if (j > 0 && !dq(j - 1, pstage)) { ok = false; break; }
-      pstage = stage;
-      if (++stage == NST) { stage = 0; phase ^= 1u; }
+      if (!uwait(&vfull[vs], (uint32_t)(j / NV) & 1u, abort_flag, err)) return false;
+      fence_after();
+      if (leader) {
+        mma_nt<HD>(tmem + DP + 128 * (j & 1), do_addr, v_addr + vs * C_::T);
+        mma_commit(&dpfull[j & 1]);
+        mma_commit(&vempty[vs]);
+      }
+      __syncwarp();
+      return true;
+    };
+    ok = ok && scores(0);
+    for (int j = 0; ok && j < nkb; ++j) {
+      if (j + 1 < nkb && (!uwait(sread, (uint32_t)j & 1u, abort_flag, err) || !scores(j + 1))) { ok = false; break; }
+      if (!uwait(dsfull, (uint32_t)j & 1u, abort_flag, err)) { ok = false; break; }
+      fence_after();
+      if (leader) {
+        const int ks = j % NK;
+        mma_ta<HD, 32>(tmem + DQ, tmem + DP + 128 * (j & 1), k_addr + ks * C_::T, j > 0);
+        mma_commit(&kempty[ks]);
+      }
+      __syncwarp();
     }
-    if (ok && !dq(nkb - 1, pstage)) ok = false;
     if (leader) {
       if (ok) mma_commit(ofull);
       mma_commit(fin);
     }
     __syncwarp();
   } else {
-    const int quad = warp & 3, qq = (warp - 2) / 4;   // TMEM lane quadrant, 32-column quarter
+    const int quad = warp & 3, qq = (warp - 2) >> 2;   // TMEM lane quadrant, 32-column quarter
     const int r = quad * 32 + lane;
-    const int q = q0 + r, qc = min(q, S - 1);
-    const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
-    const size_t si = ((size_t)b * H + h) * S + qc;
+    const int q = q0 + r;
+    const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(32 * qq);
+    const size_t si = ((size_t)b * H + h) * S + min(q, S - 1);
     const float nlse2 = q < S ? -lse[si] * kL2e : -INFINITY;
-    {   // D = rowsum(dO * O): each quarter sums a quarter of the row, fixed-order combination
-      const bf16* orow = outp + ((size_t)b * S + qc) * HDall + (size_t)h * HD + qq * (HD / 4);
-      const bf16* grow = dout + ((size_t)b * S + qc) * HDall + (size_t)h * HD + qq * (HD / 4);
-      float acc = 0.f;
+    {   // D = rowsum(dO * O), eight rows per warp: LR lanes per row, 16 bytes of O and dO each
+      constexpr int LR = HD / 8, RPL = 32 / LR;
+      const int w = warp - 2, sub = lane / LR;
+      uint4 o4[8 / RPL], g4[8 / RPL];
 #pragma unroll
-      for (int c = 0; c < HD / 4; c += 8) {
-        float o8[8], g8[8];
-        Vec8<bf16>::load(orow + c, o8);
-        Vec8<bf16>::load(grow + c, g8);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc = fmaf(o8[e], g8[e], acc);
+      for (int u = 0; u < 8 / RPL; ++u) {
+        const int row = min(q0 + 8 * w + u * RPL + sub, S - 1);
+        const size_t o = ((size_t)b * S + row) * ((size_t)H * HD) + (size_t)h * HD + (lane % LR) * 8;
+        o4[u] = *reinterpret_cast<const uint4*>(outp + o);
+        g4[u] = *reinterpret_cast<const uint4*>(dout + o);
       }
-      dpart[qq * 128 + r] = acc;
+#pragma unroll
+      for (int u = 0; u < 8 / RPL; ++u) {
+        const uint32_t ow[4] = {o4[u].x, o4[u].y, o4[u].z, o4[u].w}, gw[4] = {g4[u].x, g4[u].y, g4[u].z, g4[u].w};
+        uint64_t acc = f2(0.f, 0.f);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc = fma2(bf2_to_f2(ow[e]), bf2_to_f2(gw[e]), acc);
+        const float2 a2 = uf2(acc);
+        float a = a2.x + a2.y;
+#pragma unroll
+        for (int x = LR / 2; x > 0; x >>= 1) a += __shfl_xor_sync(0xffffffffu, a, x);
+        const int lr = 8 * w + u * RPL + sub;
+        if (lane % LR == 0) {
+          sD[lr] = a;
+          if (q0 + lr < S) Dv[((size_t)b * H + h) * S + q0 + lr] = a;
+        }
+      }
     }
     asm volatile("bar.sync 1, %0;" ::"n"(32 * NEW) : "memory");
-    const float Dq = (dpart[r] + dpart[128 + r]) + (dpart[256 + r] + dpart[384 + r]);
-    if (q < S && qq == 0) Dv[si] = Dq;
+    const float Dq = sD[r];
     const uint64_t SL2 = f2(scale * kL2e, scale * kL2e), NL = f2(nlse2, nlse2), DD = f2(Dq, Dq);
-    const int qmin = q0 + quad * 32;   // smallest query row of this warp
     bool ok = true;
     for (int j = 0; j < nkb; ++j) {
       if (!uwait(sfull, (uint32_t)j & 1u, abort_flag, err)) { ok = false; break; }
       fence_after();
-      for (int sub = 0; sub < 2; ++sub) {
-        const int c0 = qq * 32 + sub * 16;
-        float sv[16], dp[16];
-        tmem_ld16(trow + (uint32_t)c0, sv);
-        tmem_ld16(trow + 128u + (uint32_t)c0, dp);
-        if (sub == 1) {
-          fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(sempty);
-        }
-        const int kbase = j * WB + c0;
-        const bool diag = kbase + 15 > qmin;   // warp-uniform: some column may lie above the diagonal
-        const int kmax = q - kbase;            // causal: columns e <= kmax
-        uint32_t pk[8];
+      uint32_t p[32];   // S, then P (fp32 bits)
+      tmem_ld32u(trow, p);
+      fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(sread);
+      if (j == nkb - 1) {   // the diagonal block: keys after the query are masked
+        const int kmax = r - 32 * qq;
 #pragma unroll
-        for (int e = 0; e < 16; e += 2) {
-          float2 x = uf2(fma2(f2(sv[e], sv[e + 1]), SL2, NL));
-          if (diag) {
-            if (e > kmax) x.x = -INFINITY;
-            if (e + 1 > kmax) x.y = -INFINITY;
-          }
-          const float p0 = ex2(x.x), p1 = ex2(x.y);
-          const float2 ds = uf2(mul2(f2(p0, p1), sub2(f2(dp[e], dp[e + 1]), DD)));
-          pk[e / 2] = pack2(ds.x, ds.y);
-        }
-        if (sub == 0 && !uwait(dsempty, ((uint32_t)j & 1u) ^ 1u, abort_flag, err)) { ok = false; break; }
-        put_row16w(sds, qq, sub, r, pk);
+        for (int e = 0; e < 32; ++e)
+          if (e > kmax) p[e] = 0xff800000u;
       }
-      if (!ok) break;
-      fence_async_smem();
+#pragma unroll
+      for (int e = 0; e < 32; e += 2) {
+        const float2 x = uf2(fma2(f2(__uint_as_float(p[e]), __uint_as_float(p[e + 1])), SL2, NL));
+        p[e] = __float_as_uint(ex2(x.x));
+        p[e + 1] = __float_as_uint(ex2(x.y));
+      }
+      if (!uwait(&dpfull[j & 1], (uint32_t)(j >> 1) & 1u, abort_flag, err)) { ok = false; break; }
+      fence_after();
+      const uint32_t tdp = trow + DP + 128u * (uint32_t)(j & 1);
+      uint32_t dp[32], pk[16];
+      tmem_ld32u(tdp, dp);
+#pragma unroll
+      for (int e = 0; e < 32; e += 2) {
+        const float2 ds = uf2(mul2(f2(__uint_as_float(p[e]), __uint_as_float(p[e + 1])),
+                                   sub2(f2(__uint_as_float(dp[e]), __uint_as_float(dp[e + 1])), DD)));
+        pk[e / 2] = pack2(ds.x, ds.y);
+      }
+      tmem_st16u(tdp, pk);
+      tmem_st_wait();
+      fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(dsfull);
     }
     if (ok && uwait(ofull, 0, abort_flag, err)) {
       fence_after();
-      bf16* drow = dqkv + ((size_t)b * S + qc) * ld + (size_t)h * HD;
-#pragma unroll
-      for (int c = qq * (HD / 4); c < (qq + 1) * (HD / 4); c += 16) {
-        float v[16];
-        tmem_ld16(trow + 256 + (uint32_t)c, v);
-        if (q < S) {
-#pragma unroll
-          for (int e = 0; e < 16; ++e) v[e] *= scale;
-          Vec8<bf16>::store(drow + c, v);
-          Vec8<bf16>::store(drow + c + 8, v + 8);
-        }
-      }
+      // one 64-column box for each of the quadrant's first HD / 64 warps
+      if (qq < HD / 64)
+        store_rows(tmem + ((uint32_t)(quad * 32) << 16) + DQ, scale, sq + quad * (HD / 64) * 4096, &tdq, h * HD,
+                   q0 + quad * 32, b, S, qq, qq + 1, lane);
     }
   }
   fence_before();
   __syncthreads();
-  if (warp == 1) tmem_release(fin, tmem);
+  if (warp == 1) tmem_release(fin, tmem, 512);
 }
 
-// dK / dV kernel, 128-query inner blocks; grouped heads and outputs as attn_bwd_dkv_tg_k. Maps: tkv, tq,
-// tdo, all in 128-row boxes.
+// dK / dV kernel. One CTA per 128 keys of one KV head and `hpc` of its query heads (blockIdx.x = kvh *
+// (group / hpc) + share): with hpc == group bf16 straight into dqkv, else fp32 partials part[2][shares of all
+// KV heads][B * S][HD] (dK unscaled), summed per group afterwards. TMEM: NSB buffers of
+// S^T / P^T, then dP^T / dS^T, dV, dK.
 template <int HD>
 __global__ void __launch_bounds__(NTHR_B, 1)
-    attn_bwd_dkv_w_k(const __grid_constant__ CUtensorMap tkv, const __grid_constant__ CUtensorMap tq,
-                     const __grid_constant__ CUtensorMap tdo, const float* __restrict__ lse,
-                     const float* __restrict__ Dv, bf16* __restrict__ dqkv, int S, int H, int Hkv, float scale,
-                     float* __restrict__ part, unsigned* err) {
-  using C_ = WCfg<HD>;
-  constexpr int NST = C_::NST;
+    attn_bwd_dkv_k(const __grid_constant__ CUtensorMap tqkv, const __grid_constant__ CUtensorMap tdo,
+                   const __grid_constant__ CUtensorMap tdkv, const float* __restrict__ lse,
+                   const float* __restrict__ Dv, int S, int H, int Hkv, int hpc, float scale, float* __restrict__ part,
+                   unsigned* err) {
+  using C_ = BCfg<HD>;
+  constexpr int NST = C_::NST, NSB = C_::NSB;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t* sk = smem;
-  uint8_t* sv = sk + C_::T128;
-  uint8_t* sst = sv + C_::T128;                   // stage s: Q_i at s * 2 T128, dO_i after it
-  uint8_t* sp = sst + NST * 2 * C_::T128;         // P^T
-  uint8_t* sds = sp + C_::OPB;                    // dS^T
-  float* stats = (float*)(sds + C_::OPB);         // stage s: -lse2[128], D[128]
-  uint64_t* full = (uint64_t*)(stats + NST * 2 * WB);
+  uint8_t* sk = smem;                             // K and V, at the end the staging of dK and dV
+  uint8_t* sv = sk + C_::T;
+  uint8_t* sst = sv + C_::T;                      // stage s: Q_i at s * 2 T, dO_i after it
+  float* stats = (float*)(sst + NST * 2 * C_::T); // stage s: -lse2[128], D[128]
+  uint64_t* full = (uint64_t*)(stats + NST * 2 * 128);
   uint64_t* empty = full + NST;
   uint64_t* kvfull = empty + NST;
-  uint64_t* sfull = kvfull + 1;
-  uint64_t* sempty = sfull + 1;
-  uint64_t* pfull = sempty + 1;
-  uint64_t* pempty = pfull + 1;
-  uint64_t* ofull = pempty + 1;
+  uint64_t* sfull = kvfull + 1;                   // [NSB]
+  uint64_t* pfull = sfull + NSB;
+  uint64_t* dpfull = pfull + 1;
+  uint64_t* dsfull = dpfull + 1;
+  uint64_t* ofull = dsfull + 1;
   uint64_t* fin = ofull + 1;
   uint32_t* tbase = (uint32_t*)(fin + 1);
   volatile int* abort_flag = (volatile int*)(tbase + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int h = blockIdx.x, b = blockIdx.y, kb = blockIdx.z;   // key block 0 (the longest) first
-  const int kvh = part ? h / (H / Hkv) : h;
-  const int k0 = kb * 128;
-  const int nit = (S + WB - 1) / WB - kb;         // query blocks kb .. : the causal ones
-  const int ld = (H + 2 * Hkv) * HD;
-  const int xq = h * HD, xk = (H + kvh) * HD, xv = (H + Hkv + kvh) * HD;
+  const int b = blockIdx.y, kb = blockIdx.z;   // key block 0 (the longest) first
+  const int shares = H / Hkv / hpc, kvh = blockIdx.x / shares;
+  const int h0 = kvh * (H / Hkv) + (blockIdx.x % shares) * hpc;   // first query head
+  const int k0 = kb * QB;
+  const int per_head = (S + QB - 1) / QB - kb;     // query blocks kb .. : the causal ones
+  const int nit = hpc * per_head;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NST; ++s) { mbar_init(&full[s], 2); mbar_init(&empty[s], 1); }
     mbar_init(kvfull, 1);
-    mbar_init(sfull, 1);
-    mbar_init(sempty, NEW);
+    for (int s = 0; s < NSB; ++s) mbar_init(&sfull[s], 1);
     mbar_init(pfull, NEW);
-    mbar_init(pempty, 1);
+    mbar_init(dpfull, 1);
+    mbar_init(dsfull, NEW);
     mbar_init(ofull, 1);
     mbar_init(fin, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) tmem_alloc512(tbase);
+  if (warp == 1) tmem_alloc(tbase, 512);
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tbase;   // S^T 0-127, dP^T 128-255, dV 256 + HD, dK 256 + HD .. 256 + 2 HD
+  const uint32_t tmem = *tbase;
+  constexpr uint32_t DP = NSB * 128, DVC = DP + 128, DKC = DVC + HD;
   pdl_wait();
   pdl_trigger();
 
   if (warp == 0) {
     // one elected lane: TMA of K, V once and of (Q_i, dO_i) per block; every lane: four of the block's
     // -lse2 and D, loaded one block ahead
+    const bool leader = elect_one();
+    if (leader) {
+      mbar_expect_tx(kvfull, 2 * C_::T);
+      load_tile<HD>(sk, &tqkv, kvfull, (H + kvh) * HD, k0, b);
+      load_tile<HD>(sv, &tqkv, kvfull, (H + Hkv + kvh) * HD, k0, b);
+    }
     int issued[NST];
 #pragma unroll
     for (int s = 0; s < NST; ++s) issued[s] = -1;
-    const bool leader = elect_one();
-    if (leader) {
-      mbar_expect_tx(kvfull, 2 * C_::T128);
-#pragma unroll
-      for (int c = 0; c < HD / 64; ++c) {
-        tma3d(sk + c * 16384, &tkv, kvfull, xk + 64 * c, k0, b);
-        tma3d(sv + c * 16384, &tkv, kvfull, xv + 64 * c, k0, b);
-      }
-    }
     int stage = 0;
     uint32_t phase = 0;
     bool ok = true;
     float nl[4], dd[4];
     auto fetch = [&](int it) {
+      const size_t row = ((size_t)b * H + h0 + it / per_head) * S;
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const int qq2 = (kb + it) * WB + lane * 4 + u;
-        const size_t si = ((size_t)b * H + h) * S + (qq2 < S ? qq2 : 0);
-        nl[u] = qq2 < S ? -lse[si] * kL2e : -INFINITY;
-        dd[u] = qq2 < S ? Dv[si] : 0.f;
+        const int qq = (kb + it % per_head) * QB + lane * 4 + u;
+        nl[u] = qq < S ? -lse[row + qq] * kL2e : -INFINITY;
+        dd[u] = qq < S ? Dv[row + qq] : 0.f;
       }
     };
     fetch(0);
     for (int it = 0; it < nit; ++it) {
-      const int qi0 = (kb + it) * WB;
+      const int h = h0 + it / per_head, qi0 = (kb + it % per_head) * QB;
       if (!uwait(&empty[stage], phase ^ 1u, abort_flag, err)) { ok = false; break; }
       issued[stage] = (int)phase;
       if (leader) {
-        mbar_expect_tx(&full[stage], 2 * C_::T128);
-        uint8_t* st = sst + stage * 2 * C_::T128;
-#pragma unroll
-        for (int c = 0; c < HD / 64; ++c) {
-          tma3d(st + c * 16384, &tq, &full[stage], xq + 64 * c, qi0, b);
-          tma3d(st + C_::T128 + c * 16384, &tdo, &full[stage], h * HD + 64 * c, qi0, b);
-        }
+        mbar_expect_tx(&full[stage], 2 * C_::T);
+        uint8_t* st = sst + stage * 2 * C_::T;
+        load_tile<HD>(st, &tqkv, &full[stage], h * HD, qi0, b);
+        load_tile<HD>(st + C_::T, &tdo, &full[stage], h * HD, qi0, b);
       }
-      float* sl = stats + stage * 2 * WB;
+      float* sl = stats + stage * 256;
       *reinterpret_cast<float4*>(sl + lane * 4) = make_float4(nl[0], nl[1], nl[2], nl[3]);
-      *reinterpret_cast<float4*>(sl + WB + lane * 4) = make_float4(dd[0], dd[1], dd[2], dd[3]);
+      *reinterpret_cast<float4*>(sl + 128 + lane * 4) = make_float4(dd[0], dd[1], dd[2], dd[3]);
       __syncwarp();
       if (lane == 0) mbar_arrive(&full[stage]);
       if (it + 1 < nit) fetch(it + 1);
       if (++stage == NST) { stage = 0; phase ^= 1u; }
     }
-    if (!ok && lane == 0) drain<NST>(full, issued, kvfull);
+    if (!ok && lane == 0) {
+#pragma unroll
+      for (int s = 0; s < NST; ++s) drain1(&full[s], issued[s]);
+      drain1(kvfull, 0);
+    }
   } else if (warp == 1) {
-    constexpr uint32_t id_s = idesc_f16(128, WB, false, false);
-    constexpr uint32_t id_g = idesc_f16(128, HD, false, true);
-    const uint32_t k_addr = su32(sk), v_addr = su32(sv), p_addr = su32(sp), ds_addr = su32(sds);
+    // Order per block: dV += P_i dO_i, S_{i + NSB} over P_i, dK += dS_i Q_i, dP_{i+1} over dS_i. With two score
+    // buffers S is always ready before its P phase begins; with one (head dim 128, where the accumulators
+    // take half of TMEM) the dV product and S_{i+1} run under the dS phase.
+    const uint32_t k_addr = su32(sk), v_addr = su32(sv), st_addr = su32(sst);
     const bool leader = elect_one();   // issues every product and every commit that tracks them
     bool ok = uwait(kvfull, 0, abort_flag, err);
-    fence_after();
-    int stage = 0, pstage = 0;
-    uint32_t phase = 0;
-    auto grads = [&](int ib, int st) -> bool {   // dV += P^T dO_ib, dK += dS^T Q_ib
-      if (!uwait(pfull, (uint32_t)(ib & 1), abort_flag, err)) return false;
+    auto scores = [&](int it) -> bool {   // S^T_it into its buffer
+      const int st = it % NST, sb = it % NSB;
+      if (!uwait(&full[st], (uint32_t)(it / NST) & 1u, abort_flag, err)) return false;
       fence_after();
       if (leader) {
-        const uint32_t qa = su32(sst + st * 2 * C_::T128), da = qa + C_::T128;
-#pragma unroll
-        for (int ks = 0; ks < WB / 16; ++ks) {
-          const uint32_t acc = (ib > 0 || ks > 0) ? 1u : 0u;
-          const uint32_t ao = (ks / 4) * 16384 + (ks % 4) * 32;
-          mma_bf16(tmem + 256, sdesc(p_addr + ao, 16, 1024), sdesc(da + ks * 2048, 16384, 1024), id_g, acc);
-          mma_bf16(tmem + 256 + HD, sdesc(ds_addr + ao, 16, 1024), sdesc(qa + ks * 2048, 16384, 1024), id_g, acc);
-        }
-        mma_commit(&empty[st]);
-        mma_commit(pempty);
+        mma_nt<HD>(tmem + 128 * sb, k_addr, st_addr + st * 2 * C_::T);
+        mma_commit(&sfull[sb]);
       }
       __syncwarp();
       return true;
     };
-    for (int it = 0; ok && it < nit; ++it) {
-      if (!uwait(sempty, ((uint32_t)it & 1u) ^ 1u, abort_flag, err) || !uwait(&full[stage], phase, abort_flag, err)) {
-        ok = false;
-        break;
-      }
-      fence_after();
+    auto dprobs = [&](int it) {   // dP^T_it (its stage has been waited for)
       if (leader) {
-        const uint32_t qa = su32(sst + stage * 2 * C_::T128), da = qa + C_::T128;
-#pragma unroll
-        for (int ks = 0; ks < HD / 16; ++ks) {
-          const int kq = ks / 4, kr = ks % 4;
-          mma_bf16(tmem, sdesc(k_addr + kq * 16384 + kr * 32, 16, 1024), sdesc(qa + kq * 16384 + kr * 32, 16, 1024),
-                   id_s, ks > 0 ? 1u : 0u);
-          mma_bf16(tmem + 128, sdesc(v_addr + kq * 16384 + kr * 32, 16, 1024),
-                   sdesc(da + kq * 16384 + kr * 32, 16, 1024), id_s, ks > 0 ? 1u : 0u);
-        }
-        mma_commit(sfull);
+        mma_nt<HD>(tmem + DP, v_addr, st_addr + (it % NST) * 2 * C_::T + C_::T);
+        mma_commit(dpfull);
       }
       __syncwarp();
-      if (it > 0 && !grads(it - 1, pstage)) { ok = false; break; }
-      pstage = stage;
-      if (++stage == NST) { stage = 0; phase ^= 1u; }
+    };
+    ok = ok && scores(0);
+    if (ok) dprobs(0);
+    if (ok && NSB == 2 && nit > 1) ok = scores(1);
+    for (int it = 0; ok && it < nit; ++it) {
+      const int st = it % NST, sb = it % NSB;
+      const uint32_t qa = st_addr + st * 2 * C_::T;
+      if (!uwait(pfull, (uint32_t)it & 1u, abort_flag, err)) { ok = false; break; }
+      fence_after();
+      if (leader) mma_ta<HD, 32>(tmem + DVC, tmem + 128 * sb, qa + C_::T, it > 0);
+      __syncwarp();
+      if (it + NSB < nit && !scores(it + NSB)) { ok = false; break; }
+      if (!uwait(dsfull, (uint32_t)it & 1u, abort_flag, err)) { ok = false; break; }
+      fence_after();
+      if (leader) {
+        mma_ta<HD, 32>(tmem + DKC, tmem + DP, qa, it > 0);
+        mma_commit(&empty[st]);
+      }
+      __syncwarp();
+      if (it + 1 < nit) dprobs(it + 1);
     }
-    if (ok && !grads(nit - 1, pstage)) ok = false;
     if (leader) {
       if (ok) mma_commit(ofull);
       mma_commit(fin);
     }
     __syncwarp();
   } else {
-    const int quad = warp & 3, qq = (warp - 2) / 4;   // TMEM lane quadrant, 32-column quarter
-    const int r = quad * 32 + lane;                    // key row = TMEM lane
+    const int quad = warp & 3, qq = (warp - 2) >> 2;     // TMEM lane quadrant, 32-column quarter
+    const int r = quad * 32 + lane;                       // key row = TMEM lane
     const int key = k0 + r;
-    const int kmaxw = k0 + quad * 32 + 31;             // largest key of this warp
-    const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
+    const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(32 * qq);
     const uint64_t SL2 = f2(scale * kL2e, scale * kL2e);
     // Only the causal mask is applied: queries >= S have -lse2 = -inf (P = 0) and D = 0, and rows of
     // keys >= S are never stored.
     bool ok = true;
     for (int it = 0; it < nit; ++it) {
-      const int stage = it % NST;
-      const uint32_t phase = (uint32_t)(it / NST) & 1u;
-      if (!uwait(sfull, (uint32_t)it & 1u, abort_flag, err)) { ok = false; break; }
+      const int stage = it % NST, sb = it % NSB;
+      if (!uwait(&sfull[sb], (uint32_t)(it / NSB) & 1u, abort_flag, err)) { ok = false; break; }
       fence_after();
-      // this stage's statistics: its full phase has completed (the S MMA waited on it); the wait orders
+      // this stage's statistics: its full phase has completed (the S product waited on it); the wait orders
       // the producer's stores before these loads
-      if (!uwait(&full[stage], phase, abort_flag, err)) { ok = false; break; }
-      for (int sub = 0; sub < 2; ++sub) {
-        const int c0 = qq * 32 + sub * 16;
-        float svv[16], dp[16];
-        tmem_ld16(trow + (uint32_t)c0, svv);
-        tmem_ld16(trow + 128u + (uint32_t)c0, dp);
-        if (sub == 1) {
-          fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(sempty);
-        }
-        const float4* sl4 = reinterpret_cast<const float4*>(stats + stage * 2 * WB + c0);
-        const float4* sd4 = reinterpret_cast<const float4*>(stats + stage * 2 * WB + WB + c0);
-        const int qbase = (kb + it) * WB + c0;   // query of column 0 of these 16
-        const bool diag = qbase < kmaxw;          // warp-uniform: some column may precede its key
-        const int qlo = key - qbase;              // causal: columns e >= qlo
-        uint32_t pk[8], dk[8];
+      if (!uwait(&full[stage], (uint32_t)(it / NST) & 1u, abort_flag, err)) { ok = false; break; }
+      const float4* sl4 = reinterpret_cast<const float4*>(stats + stage * 256 + 32 * qq);
+      const float4* sd4 = sl4 + 32;
+      uint32_t p[32], pk[16];   // S, then P (fp32 bits)
+      tmem_ld32u(trow + 128u * (uint32_t)sb, p);
+      if (it % per_head == 0) {   // the diagonal block: queries before the key are masked
+        const int qlo = r - 32 * qq;
 #pragma unroll
-        for (int e4 = 0; e4 < 4; ++e4) {
-          const float4 l = sl4[e4], d = sd4[e4];
-          const int e = 4 * e4;
-          float2 xa = uf2(fma2(f2(svv[e], svv[e + 1]), SL2, f2(l.x, l.y)));
-          float2 xb = uf2(fma2(f2(svv[e + 2], svv[e + 3]), SL2, f2(l.z, l.w)));
-          if (diag) {
-            if (e < qlo) xa.x = -INFINITY;
-            if (e + 1 < qlo) xa.y = -INFINITY;
-            if (e + 2 < qlo) xb.x = -INFINITY;
-            if (e + 3 < qlo) xb.y = -INFINITY;
-          }
-          const float p0 = ex2(xa.x), p1 = ex2(xa.y), p2 = ex2(xb.x), p3 = ex2(xb.y);
-          const float2 da = uf2(mul2(f2(p0, p1), sub2(f2(dp[e], dp[e + 1]), f2(d.x, d.y))));
-          const float2 db = uf2(mul2(f2(p2, p3), sub2(f2(dp[e + 2], dp[e + 3]), f2(d.z, d.w))));
-          pk[2 * e4] = pack2(p0, p1);
-          pk[2 * e4 + 1] = pack2(p2, p3);
-          dk[2 * e4] = pack2(da.x, da.y);
-          dk[2 * e4 + 1] = pack2(db.x, db.y);
-        }
-        if (sub == 0 && !uwait(pempty, ((uint32_t)it & 1u) ^ 1u, abort_flag, err)) { ok = false; break; }
-        put_row16w(sp, qq, sub, r, pk);
-        put_row16w(sds, qq, sub, r, dk);
+        for (int e = 0; e < 32; ++e)
+          if (e < qlo) p[e] = 0xff800000u;
       }
-      if (!ok) break;
-      fence_async_smem();
+#pragma unroll
+      for (int e = 0; e < 32; e += 4) {
+        const float4 l = sl4[e / 4];
+        const float2 xa = uf2(fma2(f2(__uint_as_float(p[e]), __uint_as_float(p[e + 1])), SL2, f2(l.x, l.y)));
+        const float2 xb = uf2(fma2(f2(__uint_as_float(p[e + 2]), __uint_as_float(p[e + 3])), SL2, f2(l.z, l.w)));
+        const float p0 = ex2(xa.x), p1 = ex2(xa.y), p2 = ex2(xb.x), p3 = ex2(xb.y);
+        p[e] = __float_as_uint(p0);
+        p[e + 1] = __float_as_uint(p1);
+        p[e + 2] = __float_as_uint(p2);
+        p[e + 3] = __float_as_uint(p3);
+        pk[e / 2] = pack2(p0, p1);
+        pk[e / 2 + 1] = pack2(p2, p3);
+      }
+      tmem_st16u(trow + 128u * (uint32_t)sb, pk);
+      tmem_st_wait();
+      fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(pfull);
+      if (!uwait(dpfull, (uint32_t)it & 1u, abort_flag, err)) { ok = false; break; }
+      fence_after();
+      uint32_t dp[32];
+      tmem_ld32u(trow + DP, dp);
+#pragma unroll
+      for (int e = 0; e < 32; e += 4) {
+        const float4 d = sd4[e / 4];
+        const float2 da = uf2(mul2(f2(__uint_as_float(p[e]), __uint_as_float(p[e + 1])),
+                                   sub2(f2(__uint_as_float(dp[e]), __uint_as_float(dp[e + 1])), f2(d.x, d.y))));
+        const float2 db = uf2(mul2(f2(__uint_as_float(p[e + 2]), __uint_as_float(p[e + 3])),
+                                   sub2(f2(__uint_as_float(dp[e + 2]), __uint_as_float(dp[e + 3])), f2(d.z, d.w))));
+        pk[e / 2] = pack2(da.x, da.y);
+        pk[e / 2 + 1] = pack2(db.x, db.y);
+      }
+      tmem_st16u(trow + DP, pk);
+      tmem_st_wait();
+      fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(dsfull);
     }
     if (ok && uwait(ofull, 0, abort_flag, err)) {
       fence_after();
-      const int kc = min(key, S - 1);
-      const size_t NS = (size_t)gridDim.y * S;
+      const uint32_t tl = tmem + ((uint32_t)(quad * 32) << 16);
+      const int which = qq >> 1;   // 0 dK, 1 dV; two warps of the quadrant each
+      const uint32_t tc = tl + (which ? DVC : DKC);
+      if (part) {   // half of the columns per warp
+        const size_t NS = (size_t)gridDim.y * S;
+        float* pr = part + ((which ? (size_t)gridDim.x * NS : 0) + (size_t)blockIdx.x * NS + (size_t)b * S +
+                            min(key, S - 1)) * HD;
+        for (int c = (qq & 1) * (HD / 2); c < ((qq & 1) + 1) * (HD / 2); c += 32) {
+          uint32_t u[32];
+          tmem_ld32u(tc + (uint32_t)c, u);
+          if (key < S) {
 #pragma unroll
-      for (int c = qq * (HD / 4); c < (qq + 1) * (HD / 4); c += 16) {
-        float gv[16], gk[16];
-        tmem_ld16(trow + 256 + (uint32_t)c, gv);
-        tmem_ld16(trow + 256 + HD + (uint32_t)c, gk);
-        if (key < S) {
-          if (part) {
-            float* pk2 = part + ((size_t)h * NS + (size_t)b * S + kc) * HD + c;
-            float* pv2 = pk2 + (size_t)H * NS * HD;
-#pragma unroll
-            for (int e = 0; e < 16; e += 4) {
-              *reinterpret_cast<float4*>(pk2 + e) = make_float4(gk[e], gk[e + 1], gk[e + 2], gk[e + 3]);
-              *reinterpret_cast<float4*>(pv2 + e) = make_float4(gv[e], gv[e + 1], gv[e + 2], gv[e + 3]);
-            }
-          } else {
-            bf16* dkr = dqkv + ((size_t)b * S + kc) * ld + (size_t)xk + c;
-            bf16* dvr = dqkv + ((size_t)b * S + kc) * ld + (size_t)xv + c;
-#pragma unroll
-            for (int e = 0; e < 16; ++e) gk[e] *= scale;
-            Vec8<bf16>::store(dkr, gk);
-            Vec8<bf16>::store(dkr + 8, gk + 8);
-            Vec8<bf16>::store(dvr, gv);
-            Vec8<bf16>::store(dvr + 8, gv + 8);
+            for (int e = 0; e < 32; e += 4)
+              *reinterpret_cast<uint4*>(pr + c + e) = make_uint4(u[e], u[e + 1], u[e + 2], u[e + 3]);
           }
         }
+      } else if ((qq & 1) < HD / 64) {   // one 64-column box per warp
+        const int x = (which ? H + Hkv + kvh : H + kvh) * HD;
+        store_rows(tc, which ? 1.f : scale, (which ? sv : sk) + quad * (HD / 64) * 4096, &tdkv, x, k0 + quad * 32, b, S,
+                   qq & 1, (qq & 1) + 1, lane);
       }
     }
   }
   fence_before();
   __syncthreads();
-  if (warp == 1) tmem_release(fin, tmem);
+  if (warp == 1) tmem_release(fin, tmem, 512);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 g_enc = nullptr;
@@ -1541,13 +902,23 @@ bool qkv_map(CUtensorMap* m, const void* qkv, int B, int S, int W, int rows) {
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Query heads per CTA of the dK / dV kernel, a divisor of the group: a KV head's whole group in one CTA needs
+// no partials (fp32, 2 B S hd per query head, written and read back), but its longest tile (every query block
+// of every head) must not outlast the others: at most 0.6 of an SM's mean share of the blocks.
+int dkv_heads_per_cta(int B, int Hkv, int group, int nqb) {
+  const double mean = 0.5 * B * Hkv * (double)group * nqb * (nqb + 1) / g_nsm;   // blocks per SM
+  for (int hpc = group; hpc > 1; --hpc)
+    if (group % hpc == 0 && (double)hpc * nqb <= 0.6 * mean) return hpc;
+  return 1;
+}
+
 template <int HD>
 bool bwd_launch(const void* qkv, const void* out, const void* dout, const float* lse, float* D, void* dqkv, int B,
                 int S, int H, int Hkv, cudaStream_t s, cudaMemPool_t pool, unsigned* err, float scale) {
   using C_ = BCfg<HD>;
   static bool attr = false;
-  auto kq = attn_bwd_dq_tg_k<HD>;
-  auto kkv = attn_bwd_dkv_tg_k<HD>;
+  auto kq = attn_bwd_dq_k<HD>;
+  auto kkv = attn_bwd_dkv_k<HD>;
   if (!attr) {
     if (cudaFuncSetAttribute(kq, cudaFuncAttributeMaxDynamicSharedMemorySize, C_::SMEM_DQ) != cudaSuccess ||
         cudaFuncSetAttribute(kkv, cudaFuncAttributeMaxDynamicSharedMemorySize, C_::SMEM_DKV) != cudaSuccess)
@@ -1555,81 +926,42 @@ bool bwd_launch(const void* qkv, const void* out, const void* dout, const float*
     attr = true;
   }
   const int W = (H + 2 * Hkv) * HD, Wo = H * HD;
-  CUtensorMap q128, q64, do128, do64;
-  if (!qkv_map(&q128, qkv, B, S, W, 128) || !qkv_map(&q64, qkv, B, S, W, IB) || !qkv_map(&do128, dout, B, S, Wo, 128) ||
-      !qkv_map(&do64, dout, B, S, Wo, IB))
+  CUtensorMap mq, mdo, mst;   // loads of 128-row boxes; stores of 32-row boxes
+  if (!qkv_map(&mq, qkv, B, S, W, 128) || !qkv_map(&mdo, dout, B, S, Wo, 128) || !qkv_map(&mst, dqkv, B, S, W, 32))
     return false;
+  const int nqb = (S + QB - 1) / QB, group = H / Hkv;
+  const int hpc = dkv_heads_per_cta(B, Hkv, group, nqb), shares = group / hpc;
   float* part = nullptr;
-  if (H > Hkv) {   // grouped heads: one CTA per query head, then a fixed-order group reduction
-    const size_t bytes = 2ull * H * B * S * HD * sizeof(float);
+  if (shares > 1) {   // a KV head's query heads over several CTAs, then a fixed-order reduction
+    const size_t bytes = 2ull * Hkv * shares * B * S * HD * sizeof(float);
     cudaError_t e = pool ? cudaMallocFromPoolAsync((void**)&part, bytes, pool, s) : cudaMallocAsync((void**)&part, bytes, s);
     if (e != cudaSuccess) { cudaGetLastError(); return false; }
   }
-  const int nqb = (S + 127) / 128;
-  cudaError_t e = launch_pdl(kq, dim3(H, B, nqb), NTHR_B, C_::SMEM_DQ, s, q128, do128, q64, (const bf16*)out,
-                             (const bf16*)dout, lse, D, (bf16*)dqkv, S, H, Hkv, scale, err);
+  cudaError_t e = launch_pdl(kq, dim3(H, B, nqb), NTHR_B, C_::SMEM_DQ, s, mq, mdo, mst, (const bf16*)out, (const bf16*)dout,
+                             lse, D, S, H, Hkv, scale, err);
   if (e == cudaSuccess)
-    e = launch_pdl(kkv, dim3(part ? H : Hkv, B, nqb), NTHR_B, C_::SMEM_DKV, s, q128, q64, do64, (const float*)lse,
-                   (const float*)D, (bf16*)dqkv, S, H, Hkv, scale, part, err);
+    e = launch_pdl(kkv, dim3(Hkv * shares, B, nqb), NTHR_B, C_::SMEM_DKV, s, mq, mdo, mst, (const float*)lse,
+                   (const float*)D, S, H, Hkv, hpc, scale, part, err);
   if (part) {
-    if (e == cudaSuccess) launch_reduce_dkv(part, dqkv, B * S, H, Hkv, HD, scale, s);
-    cudaFreeAsync(part, s);
-  }
-  return e == cudaSuccess;
-}
-
-// The 128-wide backward (head dim 64).
-template <int HD>
-bool bwd_w_launch(const void* qkv, const void* out, const void* dout, const float* lse, float* D, void* dqkv, int B,
-                  int S, int H, int Hkv, cudaStream_t s, cudaMemPool_t pool, unsigned* err, float scale) {
-  using C_ = WCfg<HD>;
-  static bool attr = false;
-  auto kq = attn_bwd_dq_w_k<HD>;
-  auto kkv = attn_bwd_dkv_w_k<HD>;
-  if (!attr) {
-    if (cudaFuncSetAttribute(kq, cudaFuncAttributeMaxDynamicSharedMemorySize, C_::SMEM_DQ) != cudaSuccess ||
-        cudaFuncSetAttribute(kkv, cudaFuncAttributeMaxDynamicSharedMemorySize, C_::SMEM_DKV) != cudaSuccess)
-      return false;
-    attr = true;
-  }
-  const int W = (H + 2 * Hkv) * HD, Wo = H * HD;
-  CUtensorMap q128, do128;
-  if (!qkv_map(&q128, qkv, B, S, W, 128) || !qkv_map(&do128, dout, B, S, Wo, 128)) return false;
-  float* part = nullptr;
-  if (H > Hkv) {   // grouped heads: one CTA per query head, then a fixed-order group reduction
-    const size_t bytes = 2ull * H * B * S * HD * sizeof(float);
-    cudaError_t e = pool ? cudaMallocFromPoolAsync((void**)&part, bytes, pool, s) : cudaMallocAsync((void**)&part, bytes, s);
-    if (e != cudaSuccess) { cudaGetLastError(); return false; }
-  }
-  const int nqb = (S + 127) / 128;
-  cudaError_t e = launch_pdl(kq, dim3(H, B, nqb), NTHR_B, C_::SMEM_DQ, s, q128, do128, q128, (const bf16*)out,
-                             (const bf16*)dout, lse, D, (bf16*)dqkv, S, H, Hkv, scale, err);
-  if (e == cudaSuccess)
-    e = launch_pdl(kkv, dim3(part ? H : Hkv, B, nqb), NTHR_B, C_::SMEM_DKV, s, q128, q128, do128, (const float*)lse,
-                   (const float*)D, (bf16*)dqkv, S, H, Hkv, scale, part, err);
-  if (part) {
-    if (e == cudaSuccess) launch_reduce_dkv(part, dqkv, B * S, H, Hkv, HD, scale, s);
+    if (e == cudaSuccess) launch_reduce_dkv(part, dqkv, B * S, H, Hkv, shares, HD, scale, s);
     cudaFreeAsync(part, s);
   }
   return e == cudaSuccess;
 }
 
 template <int HD>
-bool fwd1_launch(const void* qkv, void* out, float* lse, int B, int S, int H, int Hkv, cudaStream_t s, unsigned* err,
-                 float scale) {
-  using C_ = F1Cfg<HD>;
+bool fwd_launch(const void* qkv, void* out, float* lse, int B, int S, int H, int Hkv, cudaStream_t s, unsigned* err,
+                float scale) {
+  using C_ = FCfg<HD>;
   static bool attr = false;
-  auto kern = attn_fwd1_tg_k<HD>;
+  auto kern = attn_fwd_k<HD>;
   if (!attr) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C_::SMEM) != cudaSuccess) return false;
     attr = true;
   }
-  const int W = (H + 2 * Hkv) * HD;
-  CUtensorMap tqk, tvv;
-  if (!qkv_map(&tqk, qkv, B, S, W, 128) || !qkv_map(&tvv, qkv, B, S, W, 64)) return false;
-  const long ntiles = (long)H * B * ((S + QB - 1) / QB);   // persistent: at most one CTA per SM
-  const int grid = (int)std::min<long>(ntiles, g_nsm);
-  return launch_pdl(kern, dim3(grid), NTHR, C_::SMEM, s, tqk, tvv, (bf16*)out, lse, S, B, H, Hkv, scale, err) ==
+  CUtensorMap mq, mo;
+  if (!qkv_map(&mq, qkv, B, S, (H + 2 * Hkv) * HD, 128) || !qkv_map(&mo, out, B, S, H * HD, 32)) return false;
+  return launch_pdl(kern, dim3(H, B, (S + QB - 1) / QB), C_::NTHR, C_::SMEM, s, mq, mo, lse, S, H, Hkv, scale, err) ==
          cudaSuccess;
 }
 
@@ -1641,12 +973,11 @@ bool fwd1_launch(const void* qkv, void* out, float* lse, int B, int S, int H, in
 bool attn_fwd_tcgen05(const void* qkv, void* out, float* lse, int B, int S, int H, int Hkv, int hd, cudaStream_t s,
                       unsigned* err, float scale) {
   if (hd != 64 && hd != 128) return false;
-  if (((uintptr_t)qkv & 15u) || ((uintptr_t)out & 15u) || (long)B * H * ((S + tg::QB - 1) / tg::QB) > 0x7fffffffL)
-    return false;
+  if ((((uintptr_t)qkv | (uintptr_t)out) & 15u) || B > 65535 || (S + 127) / 128 > 65535) return false;
   if (!tg::enc_init()) return false;
   note_launch(1);
-  return hd == 64 ? tg::fwd1_launch<64>(qkv, out, lse, B, S, H, Hkv, s, err, scale)
-                  : tg::fwd1_launch<128>(qkv, out, lse, B, S, H, Hkv, s, err, scale);
+  return hd == 64 ? tg::fwd_launch<64>(qkv, out, lse, B, S, H, Hkv, s, err, scale)
+                  : tg::fwd_launch<128>(qkv, out, lse, B, S, H, Hkv, s, err, scale);
 }
 
 // Returns false when the shape is outside these kernels (head dim 64 or 128, alignment, no sm_103a) or the
@@ -1659,7 +990,7 @@ bool attn_bwd_tcgen05(const void* qkv, const void* out, const void* dout, const 
       (S + 127) / 128 > 65535)
     return false;
   if (!tg::enc_init()) return false;
-  return hd == 64 ? tg::bwd_w_launch<64>(qkv, out, dout, lse, D, dqkv, B, S, H, Hkv, s, pool, err, scale)
+  return hd == 64 ? tg::bwd_launch<64>(qkv, out, dout, lse, D, dqkv, B, S, H, Hkv, s, pool, err, scale)
                   : tg::bwd_launch<128>(qkv, out, dout, lse, D, dqkv, B, S, H, Hkv, s, pool, err, scale);
 }
 

@@ -148,8 +148,9 @@ void attn_fwd(int dt, const void* qkv, void* out, float* lse, int B, int S, int 
 void attn_bwd(int dt, const void* qkv, const void* out, const void* dout, const float* lse, float* Dbuf,
               void* dqkv, int B, int S, int H, int Hkv, int hd, cudaStream_t s, cudaMemPool_t pool = nullptr,
               unsigned* err = nullptr);
-// dK, dV of each KV head (bf16, into dqkv) = fixed-order sums over its query heads of the fp32 partials
-// part[2][H][NS][hd] (dK unscaled; times scale here).
-void launch_reduce_dkv(const float* part, void* dqkv, int NS, int H, int Hkv, int hd, float scale, cudaStream_t s);
+// dK, dV of each KV head (bf16, into dqkv) = fixed-order sums over its `rep` shares of the fp32 partials
+// part[2][Hkv * rep][NS][hd] (dK unscaled; times scale here).
+void launch_reduce_dkv(const float* part, void* dqkv, int NS, int H, int Hkv, int rep, int hd, float scale,
+                       cudaStream_t s);
 
 }  // namespace zl

@@ -1,0 +1,46 @@
+"""The tcgen05 attention at the edges of its 128-row blocks and of its head deal (GPU), against fp32 autograd."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    import paper_2608_07974_gb300 as pkg
+    pkg.build()
+    from paper_2608_07974_gb300 import binding
+    return binding
+
+
+# One block exactly, one row more and one less, a last block of one row; grouped heads whose dK / dV kernel takes
+# one, several or all query heads of a KV head in one CTA (with 152 SMs: 1 of 2, 2 of 4, 4 of 4, 2 of 8, 8 of 8).
+@pytest.mark.parametrize("Bb,S,H,Hkv,hd", [(2, 127, 2, 2, 64), (2, 128, 2, 2, 128), (1, 129, 2, 1, 128), (3, 256, 3, 3, 64),
+                                           (1, 257, 2, 2, 64), (1, 385, 2, 2, 128), (16, 200, 32, 8, 64),
+                                           (40, 129, 32, 8, 128), (16, 257, 32, 4, 128), (8, 641, 64, 8, 64)])
+def test_attention_block_edges(B, Bb, S, H, Hkv, hd):
+    g = torch.Generator(device="cuda").manual_seed(S + 7 * H + hd)
+    W = (H + 2 * Hkv) * hd
+    qkv = torch.randn(Bb * S, W, device="cuda", generator=g).to(torch.bfloat16)
+    dout = torch.randn(Bb * S, H * hd, device="cuda", generator=g).to(torch.bfloat16)
+    out = torch.full((Bb * S, H * hd), float("nan"), device="cuda", dtype=torch.bfloat16)
+    lse = torch.full((Bb, H, S), float("nan"), device="cuda")
+    dqkv = torch.full_like(qkv, float("nan"))
+    B.zl_op_attention(B.ZL_DTYPE_BF16, qkv, out, lse, Bb, S, H, Hkv, hd)
+    B.zl_op_attention_bwd(B.ZL_DTYPE_BF16, qkv, out, dout, lse, dqkv, Bb, S, H, Hkv, hd)
+    torch.cuda.synchronize()
+    x = qkv.float().requires_grad_(True)
+    t = x.view(Bb, S, H + 2 * Hkv, hd).transpose(1, 2)
+    k, v = (t[:, a:a + Hkv].repeat_interleave(H // Hkv, 1) for a in (H, H + Hkv))
+    s = (t[:, :H] @ k.transpose(-1, -2)) / hd ** 0.5
+    s = s.masked_fill(torch.ones(S, S, dtype=torch.bool, device="cuda").triu(1), float("-inf"))
+    ref = (torch.softmax(s, -1) @ v).transpose(1, 2).reshape(Bb * S, H * hd)
+    (gx,) = torch.autograd.grad(ref, x, dout.float())
+    # P, dS and the results are rounded to bf16 (2^-9 relative each, independent errors): well under 1% in norm
+    assert float((lse - torch.logsumexp(s, -1)).abs().max()) <= 1e-5 * S ** 0.5
+    assert float((out.float() - ref).norm() / ref.norm()) <= 1e-2
+    for lo, hi in ((0, H * hd), (H * hd, (H + Hkv) * hd), ((H + Hkv) * hd, W)):
+        assert float((dqkv[:, lo:hi].float() - gx[:, lo:hi]).norm() / gx[:, lo:hi].norm()) <= 1e-2, (lo, hi)
+    again = torch.empty_like(dqkv)
+    B.zl_op_attention_bwd(B.ZL_DTYPE_BF16, qkv, out, dout, lse, again, Bb, S, H, Hkv, hd)
+    assert torch.equal(again, dqkv)   # fixed summation order
