@@ -415,8 +415,8 @@ __global__ void __launch_bounds__(NTHR_B, 1)
   uint64_t* sfull = qfull + 1;
   uint64_t* sread = sfull + 1;                    // the elementwise warps have S in registers
   uint64_t* dpfull = sread + 1;                   // [2]
-  uint64_t* dsfull = dpfull + 2;
-  uint64_t* ofull = dsfull + 1;
+  uint64_t* dsfull = dpfull + 2;                  // [2] (the warps may be a block ahead of the MMA warp's wait)
+  uint64_t* ofull = dsfull + 2;
   uint64_t* fin = ofull + 1;
   uint32_t* tbase = (uint32_t*)(fin + 1);
   volatile int* abort_flag = (volatile int*)(tbase + 1);
@@ -432,7 +432,8 @@ __global__ void __launch_bounds__(NTHR_B, 1)
     mbar_init(sread, NEW);
     mbar_init(&dpfull[0], 1);
     mbar_init(&dpfull[1], 1);
-    mbar_init(dsfull, NEW);
+    mbar_init(&dsfull[0], NEW);
+    mbar_init(&dsfull[1], NEW);
     mbar_init(ofull, 1);
     mbar_init(fin, 1);
     *abort_flag = 0;
@@ -514,7 +515,7 @@ __global__ void __launch_bounds__(NTHR_B, 1)
     ok = ok && scores(0);
     for (int j = 0; ok && j < nkb; ++j) {
       if (j + 1 < nkb && (!uwait(sread, (uint32_t)j & 1u, abort_flag, err) || !scores(j + 1))) { ok = false; break; }
-      if (!uwait(dsfull, (uint32_t)j & 1u, abort_flag, err)) { ok = false; break; }
+      if (!uwait(&dsfull[j & 1], (uint32_t)(j >> 1) & 1u, abort_flag, err)) { ok = false; break; }
       fence_after();
       if (leader) {
         const int ks = j % NK;
@@ -602,7 +603,7 @@ __global__ void __launch_bounds__(NTHR_B, 1)
       tmem_st_wait();
       fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(dsfull);
+      if (lane == 0) mbar_arrive(&dsfull[j & 1]);
     }
     if (ok && uwait(ofull, 0, abort_flag, err)) {
       fence_after();
@@ -639,8 +640,8 @@ __global__ void __launch_bounds__(NTHR_B, 1)
   uint64_t* empty = full + NST;
   uint64_t* kvfull = empty + NST;
   uint64_t* sfull = kvfull + 1;                   // [NSB]
-  uint64_t* pfull = sfull + NSB;
-  uint64_t* dpfull = pfull + 1;
+  uint64_t* pfull = sfull + NSB;                  // [NSB] (with two, a block ahead of the MMA warp's wait)
+  uint64_t* dpfull = pfull + NSB;
   uint64_t* dsfull = dpfull + 1;
   uint64_t* ofull = dsfull + 1;
   uint64_t* fin = ofull + 1;
@@ -658,7 +659,7 @@ __global__ void __launch_bounds__(NTHR_B, 1)
     for (int s = 0; s < NST; ++s) { mbar_init(&full[s], 2); mbar_init(&empty[s], 1); }
     mbar_init(kvfull, 1);
     for (int s = 0; s < NSB; ++s) mbar_init(&sfull[s], 1);
-    mbar_init(pfull, NEW);
+    for (int s = 0; s < NSB; ++s) mbar_init(&pfull[s], NEW);
     mbar_init(dpfull, 1);
     mbar_init(dsfull, NEW);
     mbar_init(ofull, 1);
@@ -755,7 +756,7 @@ __global__ void __launch_bounds__(NTHR_B, 1)
     for (int it = 0; ok && it < nit; ++it) {
       const int st = it % NST, sb = it % NSB;
       const uint32_t qa = st_addr + st * 2 * C_::T;
-      if (!uwait(pfull, (uint32_t)it & 1u, abort_flag, err)) { ok = false; break; }
+      if (!uwait(&pfull[sb], (uint32_t)(it / NSB) & 1u, abort_flag, err)) { ok = false; break; }
       fence_after();
       if (leader) mma_ta<HD, 32>(tmem + DVC, tmem + 128 * sb, qa + C_::T, it > 0);
       __syncwarp();
@@ -817,7 +818,7 @@ __global__ void __launch_bounds__(NTHR_B, 1)
       tmem_st_wait();
       fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(pfull);
+      if (lane == 0) mbar_arrive(&pfull[sb]);
       if (!uwait(dpfull, (uint32_t)it & 1u, abort_flag, err)) { ok = false; break; }
       fence_after();
       uint32_t dp[32];
