@@ -2,7 +2,7 @@
 // fp32 accumulator in TMEM, double buffered) -> tcgen05.ld epilogue (bias, residual, bf16 store,
 // or fp32 accumulate into a gradient, or the fused AdamW step of the weight). Persistent,
 // warp-specialised: warp 0 issues TMA loads, warp 1 owns TMEM and issues the MMAs (one thread),
-// warps 2-5 (fused update: 4-11) drain the accumulator.
+// warps 2-5 (fused update: 4-11) drain the accumulator. Large products run on CTA pairs (cta_group::2).
 // Every mbarrier wait is bounded: on expiry the kernel raises ZL_DEVERR_TIMEOUT and unwinds.
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -31,18 +31,19 @@ constexpr int kThreadsUpd = 128 + 32 * kUpdWarps;
 constexpr int kRegsLow = 56, kRegsUpd = 224;
 static_assert(128 * kRegsLow + 32 * kUpdWarps * kRegsUpd <= kThreadsUpd * 168, "register split above the pool");
 
-template <int BN, bool UPD = false>
+template <int BN, bool UPD = false, bool PAIR = false>
 struct Cfg {
   // BN = 64 stays under 114 KB of shared memory so two CTAs (and TMEM allocations) fit on an SM.
-  static constexpr int STAGES = UPD ? (BN == 256 ? 4 : (kUpdWarps > 8 ? 5 : 6)) : (BN == 256 ? 4 : (BN == 128 ? 6 : 3));
+  static constexpr int STAGES = PAIR ? (BN == 256 ? 6 : 8) : (BN == 256 ? 4 : (BN == 128 ? 6 : 3));
   static constexpr int A_BYTES = BM * BK * 2;
-  static constexpr int B_BYTES = BN * BK * 2;
+  static constexpr int B_BYTES = (PAIR ? BN / 2 : BN) * BK * 2;   // a pair's CTA holds half of the B tile
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int TMEM_COLS = 2 * BN;
   // epilogue staging: per epilogue warp two buffers of 32 rows x 128 B (the TMA store box), or, in the
   // fused-update kernels, one 32 x 32 accumulator piece per epilogue warp
   static constexpr int OUT_BYTES = UPD ? kUpdWarps * 32 * 128 : 4 * 2 * 32 * 128;
   static constexpr int SMEM = STAGES * STAGE_BYTES + OUT_BYTES + 1024 + 256;
+  static_assert(SMEM <= 232448, "shared memory per CTA");
 };
 
 // Mode 4, one chunk: 16 rows x 32 columns of the tensor (rows row0 + 16 h .., columns col0 ..), whose
@@ -102,10 +103,6 @@ __device__ __forceinline__ void upd_apply(const GemmUpdate& u, const AdamHP& h, 
   }
 }
 
-struct UpdMaps {   // (reserved: the fused update reads and writes its state directly)
-  CUtensorMap unused;
-};
-
 struct Args {
   int M, N, K, mode;       // mode 0/1: bf16 C (+bias, +R); 2: fp32 C += acc; 3: fp32 store into split slice;
                            // 4: the AdamW step of the tensor in `u` with this tile as (the last part of) its gradient
@@ -124,10 +121,10 @@ struct Args {
 };
 
 // Instruction descriptor of kind::f16: fp32 accumulator, bf16 A and B, operand majors, N, M.
-template <int BN, bool A_MN, bool B_MN>
+template <int BN, bool A_MN, bool B_MN, bool PAIR>
 __device__ __forceinline__ constexpr uint32_t idesc() {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((A_MN ? 1u : 0u) << 15) | ((B_MN ? 1u : 0u) << 16) |
-         ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+         ((uint32_t)(BN >> 3) << 17) | ((uint32_t)((PAIR ? 2 * BM : BM) >> 4) << 24);
 }
 
 // Tile order: groups of G tile rows sweep the tile columns, so the rows of A a group reads and the
@@ -152,15 +149,16 @@ __device__ __forceinline__ void unit_tile(const Args& g, int unit, int num_tiles
 }
 
 // UPD: the fused optimizer epilogue (mode 4) is compiled in (a kernel of its own, so the other modes keep
-// their register budget). PAIR: the CTA runs in a cluster of two that share each B tile: each loads half
-// of it and multicasts it to both (TMA), each CTA's MMA commit frees the stage in both, so every SM copies
-// half as much of B from L2 as alone.
+// their register budget). PAIR: two CTAs of a cluster work as one (cta_group::2) on a 256 x BN tile: each holds
+// its own 128 rows of A, half of the B tile and its own 128 rows of the accumulator, and the products that the
+// first CTA issues read both CTAs' shared memory. What bounds the single-CTA mainloop is shared memory (128
+// bytes a cycle): a 128 x 256 x 64 block reads 48 KB and its copies write 48 KB, 768 cycles against 512 of
+// products. A pair's CTA reads and writes 32 KB each per 512 cycles, and six stages fit instead of four.
 template <int BN, bool A_MN, bool B_MN, bool UPD = false, bool PAIR = false>
 __global__ void __launch_bounds__(UPD ? kThreadsUpd : kThreads, 1)
     gemm_tc_k(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
-              const __grid_constant__ CUtensorMap tcm, const Args g, const __grid_constant__ UpdMaps um) {
-  using C_ = Cfg<BN, UPD>;
-  constexpr uint16_t kPairMask = 3;
+              const __grid_constant__ CUtensorMap tcm, const Args g) {
+  using C_ = Cfg<BN, UPD, PAIR>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* outbuf = smem + C_::STAGES * C_::STAGE_BYTES;   // 1024-byte aligned (stage sizes are)
@@ -173,27 +171,36 @@ __global__ void __launch_bounds__(UPD ? kThreadsUpd : kThreads, 1)
   volatile int* abort_flag = (volatile int*)(tbase + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < C_::STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], PAIR ? 2 : 1); }
-    for (int a = 0; a < 2; ++a) { mbar_init(&tfull[a], 1); mbar_init(&tempty[a], UPD ? kUpdWarps : 4); }
+    for (int s = 0; s < C_::STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+    // a pair uses the first CTA's full and tempty barriers; both CTAs' epilogue warps arrive on tempty
+    for (int a = 0; a < 2; ++a) { mbar_init(&tfull[a], 1); mbar_init(&tempty[a], (UPD ? kUpdWarps : 4) * (PAIR ? 2 : 1)); }
     mbar_init(fin, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tbase)),
-                 "r"((uint32_t)C_::TMEM_COLS)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (PAIR) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tbase)),
+                   "r"((uint32_t)C_::TMEM_COLS)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tbase)),
+                   "r"((uint32_t)C_::TMEM_COLS)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   fence_before();
   __syncthreads();
   fence_after();
-  // a pair's copies land in both CTAs' shared memory: both sets of barriers exist before any is issued
+  // a pair's CTAs signal each other's barriers: both sets exist before anything is issued
   if (PAIR) cluster_sync();
   const uint32_t crank = PAIR ? cluster_rank() : 0u;
   const int unit0 = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const int ustride = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
   const uint32_t tmem = *tbase;
+  const uint32_t tempty_addr = PAIR ? cluster_addr(tempty, 0) : 0u;   // the first CTA's
   // Programmatic dependent launch: the set-up above may overlap the previous kernel of the stream;
   // every thread waits for that kernel (and its memory) before touching global memory, and lets the
   // next GEMM of the stream begin its own set-up.
@@ -225,32 +232,40 @@ __global__ void __launch_bounds__(UPD ? kThreadsUpd : kThreads, 1)
           if (!uwait(&empty[stage], phase ^ 1u, abort_flag, g.err)) { ok = false; break; }
           issued[stage] = (int)phase;
           if (leader) {
-            mbar_expect_tx(&full[stage], C_::STAGE_BYTES);
             uint8_t* sa = smem + stage * C_::STAGE_BYTES;
             uint8_t* sb = sa + C_::A_BYTES;
             const int k0 = kb * BK;
-            if (!A_MN) {
-              tma2d(sa, &ta, &full[stage], k0, tm * BM);
-            } else {
-              tma2d(sa, &ta, &full[stage], tm * BM, k0);
-              tma2d(sa + 8192, &ta, &full[stage], tm * BM + 64, k0);
-            }
-            if (PAIR) {   // this CTA's half of the B tile, into both CTAs
+            if constexpr (PAIR) {   // this CTA's rows of A and its half of the B tile, on the first CTA's barrier
+              if (crank == 0) mbar_expect_tx(&full[stage], 2 * C_::STAGE_BYTES);
+              const uint32_t bar = cluster_addr(&full[stage], 0);
               constexpr int HB = BN / 2;
+              const int n0 = tn * BN + (int)crank * HB;
+              if (!A_MN) {
+                tma2d_pair(sa, &ta, bar, k0, tm * BM);
+              } else {
+                tma2d_pair(sa, &ta, bar, tm * BM, k0);
+                tma2d_pair(sa + 8192, &ta, bar, tm * BM + 64, k0);
+              }
               if (!B_MN) {
-                tma2d_mc(sb + crank * (HB * 128), &tb, &full[stage], k0, tn * BN + (int)crank * HB, kPairMask);
+                tma2d_pair(sb, &tb, bar, k0, n0);
               } else {
   #pragma unroll
-                for (int j = 0; j < HB / 64; ++j) {
-                  const int jj = (int)crank * (HB / 64) + j;
-                  tma2d_mc(sb + jj * 8192, &tb, &full[stage], tn * BN + 64 * jj, k0, kPairMask);
-                }
+                for (int j = 0; j < HB / 64; ++j) tma2d_pair(sb + j * 8192, &tb, bar, n0 + 64 * j, k0);
               }
-            } else if (!B_MN) {
-              tma2d(sb, &tb, &full[stage], k0, tn * BN);
             } else {
+              mbar_expect_tx(&full[stage], C_::STAGE_BYTES);
+              if (!A_MN) {
+                tma2d(sa, &ta, &full[stage], k0, tm * BM);
+              } else {
+                tma2d(sa, &ta, &full[stage], tm * BM, k0);
+                tma2d(sa + 8192, &ta, &full[stage], tm * BM + 64, k0);
+              }
+              if (!B_MN) {
+                tma2d(sb, &tb, &full[stage], k0, tn * BN);
+              } else {
   #pragma unroll
-              for (int j = 0; j < BN / 64; ++j) tma2d(sb + j * 8192, &tb, &full[stage], tn * BN + 64 * j, k0);
+                for (int j = 0; j < BN / 64; ++j) tma2d(sb + j * 8192, &tb, &full[stage], tn * BN + 64 * j, k0);
+              }
             }
           }
           __syncwarp();
@@ -258,8 +273,8 @@ __global__ void __launch_bounds__(UPD ? kThreadsUpd : kThreads, 1)
         }
       }
       if (PAIR && ok) {
-        // both CTAs' commits for the last fill of every stage have arrived: no arrival from the peer (and no
-        // copy of this CTA's into the peer) is still on its way when the CTAs exit
+        // the commits for the last fill of every stage have arrived: no copy and no arrival is still on its way
+        // when the CTAs exit
   #pragma unroll 1
         for (int s = 0; s < C_::STAGES; ++s)
           if (issued[s] >= 0 && !uwait(&empty[s], (uint32_t)issued[s], abort_flag, g.err)) break;
@@ -267,21 +282,22 @@ __global__ void __launch_bounds__(UPD ? kThreadsUpd : kThreads, 1)
       if (!ok && lane == 0) {   // unwinding: let the copies already in flight land before the CTA exits
         for (int s = 0; s < C_::STAGES; ++s) {
           if (issued[s] < 0) continue;
-          const unsigned long long t0 = gtimer();
-          while (!mbar_test(&full[s], (uint32_t)issued[s]) && gtimer() - t0 < 100000000ull) {
+          const unsigned long long t0 = gtimer();   // (a pair's second CTA has no barrier of its own to test: 10 ms)
+          while ((PAIR && crank != 0) ? gtimer() - t0 < 10000000ull
+                                      : (!mbar_test(&full[s], (uint32_t)issued[s]) && gtimer() - t0 < 100000000ull)) {
           }
         }
       }
     } else if (warp == 1) {
       // ---------------- MMA issuer ----------------
       // The whole warp runs the loop and the waits; one elected lane issues every product and every
-      // commit that tracks them.
-      constexpr uint32_t id = idesc<BN, A_MN, B_MN>();
+      // commit that tracks them (of a pair, the first CTA's, for both).
+      constexpr uint32_t id = idesc<BN, A_MN, B_MN, PAIR>();
       const bool leader = elect_one();
       int stage = 0, it = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int unit = unit0; ok && unit < num_units; unit += ustride, ++it) {
+      for (int unit = unit0; (!PAIR || crank == 0) && ok && unit < num_units; unit += ustride, ++it) {
         const int acc = it & 1;
         const uint32_t aph = (uint32_t)(it >> 1) & 1u;
         if (!uwait(&tempty[acc], aph ^ 1u, abort_flag, g.err)) break;
@@ -297,19 +313,27 @@ __global__ void __launch_bounds__(UPD ? kThreadsUpd : kThreads, 1)
             for (int kk = 0; kk < BK / 16; ++kk) {
               const uint64_t ad = A_MN ? sdesc(a0 + kk * 2048, 8192, 1024) : sdesc(a0 + kk * 32, 16, 1024);
               const uint64_t bd = B_MN ? sdesc(b0 + kk * 2048, 8192, 1024) : sdesc(b0 + kk * 32, 16, 1024);
-              mma_bf16(d, ad, bd, id, (kb > kb0 || kk > 0) ? 1u : 0u);
+              const uint32_t add = (kb > kb0 || kk > 0) ? 1u : 0u;
+              if (PAIR) mma_bf16_pair(d, ad, bd, id, add);
+              else mma_bf16(d, ad, bd, id, add);
             }
-            if (PAIR) mma_commit_mc(&empty[stage], kPairMask);   // the stage is free in both CTAs' view
+            if (PAIR) mma_commit_pair(&empty[stage]);   // the stage is free in both CTAs
             else mma_commit(&empty[stage]);
           }
           __syncwarp();
           if (++stage == C_::STAGES) { stage = 0; phase ^= 1u; }
         }
-        if (ok && leader) mma_commit(&tfull[acc]);
+        if (ok && leader) {
+          if (PAIR) mma_commit_pair(&tfull[acc]);
+          else mma_commit(&tfull[acc]);
+        }
         __syncwarp();
       }
       // all MMAs issued by the leader complete before TMEM is released
-      if (leader) mma_commit(fin);
+      if (leader) {
+        if (!PAIR) mma_commit(fin);
+        else if (crank == 0) mma_commit_pair(fin);
+      }
       __syncwarp();
     }
   } else if constexpr (UPD) {
@@ -375,7 +399,10 @@ __global__ void __launch_bounds__(UPD ? kThreadsUpd : kThreads, 1)
           if (p == NP - 1) {
             fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&tempty[acc]);
+            if (lane == 0) {
+              if (PAIR) mbar_arrive_cluster(tempty_addr + 8u * (uint32_t)acc);
+              else mbar_arrive(&tempty[acc]);
+            }
           }
           if (g.alpha != 1.f) {
   #pragma unroll
@@ -558,7 +585,10 @@ __global__ void __launch_bounds__(UPD ? kThreadsUpd : kThreads, 1)
       }
       fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&tempty[acc]);
+      if (lane == 0) {
+        if (PAIR) mbar_arrive_cluster(tempty_addr + 8u * (uint32_t)acc);
+        else mbar_arrive(&tempty[acc]);
+      }
     }
     if (lane == 0) bulk_wait_all();   // every store of this warp has landed in global memory
   }
@@ -579,8 +609,12 @@ __global__ void __launch_bounds__(UPD ? kThreadsUpd : kThreads, 1)
   }
   if (warp == 1) {
     fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)C_::TMEM_COLS)
-                 : "memory");
+    if constexpr (PAIR)
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)C_::TMEM_COLS)
+                   : "memory");
+    else
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)C_::TMEM_COLS)
+                   : "memory");
   }
 }
 
@@ -708,7 +742,7 @@ bool make_map_c(CUtensorMap* m, const Args& a) {
 
 template <int BN, bool A_MN, bool B_MN, bool UPD = false, bool PAIR = false>
 bool launch(const Args& a, const void* A, const void* B, cudaStream_t s, int ctas_per_sm) {
-  using C_ = Cfg<BN, UPD>;
+  using C_ = Cfg<BN, UPD, PAIR>;
   static bool attr = false;
   static int max_pairs = 0;   // clusters of two that can be resident at once
   auto kern = gemm_tc_k<BN, A_MN, B_MN, UPD, PAIR>;
@@ -749,8 +783,6 @@ bool launch(const Args& a, const void* A, const void* B, cudaStream_t s, int cta
                         : make_map(&tb, B, (uint64_t)a.K, (uint64_t)a.N, 64, PAIR ? BN / 2 : BN);
   CUtensorMap tcm;
   if (!okA || !okB || !make_map_c(&tcm, a)) return false;
-  UpdMaps um;
-  std::memset(&um, 0, sizeof um);
   int grid;
   if (PAIR) {   // one cluster of two per pair of tile rows, as many as can be resident
     const int units = (a.tiles_m + 1) / 2 * a.tiles_n * a.splits;
@@ -774,7 +806,7 @@ bool launch(const Args& a, const void* A, const void* B, cudaStream_t s, int cta
   at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = PAIR ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, kern, ta, tb, tcm, a, um) == cudaSuccess;
+  return cudaLaunchKernelEx(&cfg, kern, ta, tb, tcm, a) == cudaSuccess;
 }
 
 template <bool A_MN, bool B_MN>
@@ -791,31 +823,53 @@ bool launch_upd(int bn, bool pair, const Args& a, const void* A, const void* B, 
   return pair ? launch<128, true, true, true, true>(a, A, B, s, 1) : launch<128, true, true, true>(a, A, B, s, 1);
 }
 
-// Tile width and split count from a wave model: units of 128 x BN x (K / splits) run on 152 (BN
-// 256/128) or 304 (BN 64) slots, each k block (64 deep) of a unit taking the time measured for that
-// tile on GB300 (4096^3 and transformer-shape sweeps; the operands of the mode-2 kernel are both
-// MN-major and load in more boxes), plus, for splits, the fp32 partial traffic and the reduction.
-void choose(int mode, int M, int N, int K, int& bn_out, int& splits_out, bool no64 = false) {
-  const double hbm = 6.0e12;                  // bytes/s for the partials
+// The plan of a product: tile width, split count, and whether CTA pairs run it.
+struct Plan {
+  int bn, splits, pair;
+};
+
+// The plan with the least predicted time (us): a fixed cost (launch, set-up, first loads), then waves of units
+// (a tile, or a pair's two, times K / splits) on 152 SMs (76 pairs, or 304 slots of width 64), each 64-deep k
+// block of a unit at the rate measured for its kernel and no wave shorter than a tile's epilogue, the last
+// wave's epilogue, and for splits the fp32 partials through HBM and the reduction. Fitted to every plan on 53
+// shapes (4096^3, the GPT-2, 1.1B and 7B layer and head shapes, ragged ones from 203 rows): 8% off at the
+// median of both sides, the chosen plan within 4% of the fastest one on all but a few small shapes. Pairs win wherever
+// their 256-row tiles fill the SMs (7B QKV forward 117 us against 131 alone; 4096^3 79.5 against 94); single
+// CTAs win where those tiles would leave SMs idle (4096 x 768 x 768 9.3 against 9.9). mode 4 (fused update):
+// a unit's epilogue streams its optimizer state, which is its time when the products are short.
+Plan choose(int mode, int M, int N, int K) {
+  struct Kind {
+    int bn, pair;
+    double kb, epi;
+  };
+  static const Kind kinds[] = {{256, 1, 0.295, 2.6}, {128, 1, 0.200, 2.1}, {256, 0, 0.350, 1.6}, {128, 0, 0.240, 1.4},
+                               {64, 0, 0.330, 0.6}};
+  const double hbm = 6.0e6;                  // bytes / us
+  const bool dw = mode == 2 || mode == 4;    // both operands MN-major
   const int nk = (K + BK - 1) / BK;
+  const double state = mode == 4 ? 26.0 * M * N : 0.0;
   double best = 1e30;
-  for (int bn : {256, 128, 64}) {
-    if (no64 && bn == 64) continue;
-    const double kb = mode == 2 ? (bn == 256 ? 0.40e-6 : bn == 128 ? 0.30e-6 : 0.36e-6)
-                                : (bn == 256 ? 0.36e-6 : bn == 128 ? 0.29e-6 : 0.32e-6);
-    const long tiles = (long)((M + BM - 1) / BM) * ((N + bn - 1) / bn);
-    const int cps = bn == 64 ? 2 : 1;
+  Plan p{128, 1, 0};
+  for (const Kind& c : kinds) {
+    if (mode == 4 && c.bn == 64) continue;
+    if (c.pair && M <= BM) continue;   // nothing to pair
+    const long tm = (M + BM - 1) / BM, tn = (N + c.bn - 1) / c.bn;
+    const long tiles = c.pair ? (tm + 1) / 2 * tn : tm * tn;
+    const long slots = c.pair ? g_sms / 2 : (long)g_sms * (c.bn == 64 ? 2 : 1);
+    // the update's epilogue per unit: 26 bytes for each element of a CTA's tile at about 85 bytes per ns and SM
+    const double epi = c.epi + (mode == 4 ? 26.0 * BM * c.bn / 85e3 : 0.0);
     for (int sp : {1, 2, 3, 4, 6, 8}) {
-      if (sp > 1 && nk / sp < 6) continue;
+      if (sp > 1 && nk / sp < 4) continue;
       const int kps = (nk + sp - 1) / sp;
-      const long units = tiles * sp;
-      const long slots = (long)g_sms * cps;
-      const long waves = (units + slots - 1) / slots;
-      double t = waves * kps * kb;
-      if (sp > 1) t += (double)sp * M * N * 4.0 * 2.0 / hbm + 3e-6;
-      if (t < best * 0.97) { best = t; bn_out = bn; splits_out = sp; }
+      const long waves = (tiles * sp + slots - 1) / slots;
+      const double e = sp > 1 ? c.epi : epi;
+      double t = 2.8 + waves * std::max(kps * c.kb * (dw ? 1.06 : 1.0), e) + e;
+      if (sp > 1) t += (8.0 * sp * M * N + state) / hbm + 2.0;
+      else t = std::max(t, state / hbm + 2.8);
+      if (t < best * 0.98) { best = t; p = Plan{c.bn, sp, c.pair}; }
     }
   }
+  return p;
 }
 
 }  // namespace tc
@@ -844,10 +898,8 @@ bool run_tc(int mode, int M, int N, int K, const void* A, const void* B, void* C
     return false;
   if ((mode == 0 || mode == 1) && K % 8 != 0) return false;
   if (mode >= 2 && M % 8 != 0) return false;
-  int bn = 128, splits = 1;
-  tc::choose(mode == 4 ? 2 : mode, M, N, K, bn, splits, mode == 4);
-  // CTA pairs sharing B tiles wherever there are two tile rows to pair (BN 64 runs two CTAs per SM instead)
-  int pair = bn >= 128 && M > tc::BM ? 1 : 0;
+  const tc::Plan plan = tc::choose(mode, M, N, K);
+  int bn = plan.bn, splits = plan.splits, pair = plan.pair;
   if (const char* force = std::getenv("ZL_GEMM_TILE")) {   // test hook "BN:SPLITS[:PAIR]": forces the plan
     int fb = 0, fs = 0, fp = -1;
     const int nf = std::sscanf(force, "%d:%d:%d", &fb, &fs, &fp);
@@ -861,7 +913,6 @@ bool run_tc(int mode, int M, int N, int K, const void* A, const void* B, void* C
   if (rope) {   // one split (the reduction does not rotate); tiles of 128 or 256 columns (heads never straddle)
     splits = 1;
     if (bn < 128) bn = 128;
-    pair = bn >= 128 && M > tc::BM ? pair : 0;
   }
   tc::Args a;
   a.M = M; a.N = N; a.K = K; a.mode = mode;

@@ -102,21 +102,34 @@ __device__ __forceinline__ void tma2d(void* dst, const CUtensorMap* m, uint64_t*
       : "memory");
 }
 
-// 2-D TMA load multicast to the CTAs of `mask` in this CTA's cluster: the box lands at the same shared
-// offset in each of them and completes bytes on the mbarrier at the same offset in each.
-__device__ __forceinline__ void tma2d_mc(void* dst, const CUtensorMap* m, uint64_t* bar, int c0, int c1,
-                                         uint16_t mask) {
+// CTA pairs (cta_group::2): two CTAs of a cluster work as one on M = 256 products. The address of `p` in the
+// shared memory of the cluster's CTA `rank`, as a shared::cluster address.
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(su32(p)), "r"(rank));
+  return r;
+}
+// 2-D TMA load into this CTA's shared memory that completes bytes on an mbarrier of either CTA of the pair.
+__device__ __forceinline__ void tma2d_pair(void* dst, const CUtensorMap* m, uint32_t bar, int c0, int c1) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster"
-      " [%0], [%1, {%3, %4}], [%2], %5;" ::"r"(su32(dst)),
-      "l"((unsigned long long)m), "r"(su32(bar)), "r"(c0), "r"(c1), "h"(mask)
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], "
+      "[%2];" ::"r"(su32(dst)),
+      "l"((unsigned long long)m), "r"(bar), "r"(c0), "r"(c1)
       : "memory");
 }
-// Commit of this thread's prior tcgen05 operations, arriving on the mbarrier at the same shared offset in
-// every CTA of `mask` (cluster).
-__device__ __forceinline__ void mma_commit_mc(uint64_t* bar, uint16_t mask) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::
-                   "r"(su32(bar)), "h"(mask)
+// Arrival on an mbarrier of another CTA of the cluster (cluster_addr).
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mma_bf16_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
+      "l"(a), "l"(b), "r"(id), "r"(acc));
+}
+// Commit of this thread's prior pair products, arriving on the mbarrier at the same shared offset in both CTAs.
+__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::
+                   "r"(su32(bar)), "h"((uint16_t)3)
                : "memory");
 }
 __device__ __forceinline__ uint32_t cluster_rank() {
