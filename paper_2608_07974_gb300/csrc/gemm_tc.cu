@@ -836,8 +836,10 @@ struct Plan {
 // median of both sides, the chosen plan within 4% of the fastest one on all but a few small shapes. Pairs win wherever
 // their 256-row tiles fill the SMs (7B QKV forward 117 us against 131 alone; 4096^3 79.5 against 94); single
 // CTAs win where those tiles would leave SMs idle (4096 x 768 x 768 9.3 against 9.9). mode 4 (fused update):
-// a unit's epilogue streams its optimizer state, which is its time when the products are short.
+// a unit's epilogue streams its optimizer state, which is its time when the products are short. Its split count is
+// mode 2's, so the fused and the unfused update sum the gradient in the same order (the tile does not matter).
 Plan choose(int mode, int M, int N, int K) {
+  const int same_splits = mode == 4 ? choose(2, M, N, K).splits : 0;
   struct Kind {
     int bn, pair;
     double kb, epi;
@@ -860,6 +862,7 @@ Plan choose(int mode, int M, int N, int K) {
     const double epi = c.epi + (mode == 4 ? 26.0 * BM * c.bn / 85e3 : 0.0);
     for (int sp : {1, 2, 3, 4, 6, 8}) {
       if (sp > 1 && nk / sp < 4) continue;
+      if (same_splits && sp != same_splits) continue;
       const int kps = (nk + sp - 1) / sp;
       const long waves = (tiles * sp + slots - 1) / slots;
       const double e = sp > 1 ? c.epi : epi;
