@@ -1,7 +1,9 @@
-// Causal softmax attention with grouped KV heads, forward and backward, CUDA-core version:
-// one warp per query (or key) row, fp32 online softmax. Query head h reads KV head
-// h / (H / Hkv). Scale 1/sqrt(hd). The forward saves the row log-sum-exp for the backward.
+// Causal softmax attention with grouped KV heads: the dispatch, the head padding of the tcgen05 kernels, and
+// the CUDA-core version (fp32; bf16 where no tensor-core kernel takes the shape). Query head h reads KV
+// head h / (H / Hkv). Scale 1/sqrt(hd). The forward saves the row log-sum-exp for the backward.
 #include <math.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "ops.h"
@@ -9,152 +11,242 @@
 namespace zl {
 
 namespace {
-constexpr int R = 4;   // dims per lane: head_dim <= 128
+// ------------------------------------------------------------------------------------------------
+// CUDA-core kernels. A CTA works on 32 query (or key) rows of one head, LPR lanes per row (four; eight where a row
+// would not fit four lanes' registers): lane `sub` holds the head dims 4 (LPR c + sub) .. + 3 (HDP: hd rounded up
+// to 32, 64 or 128, zero padded). The other side comes in tiles of 32 rows through shared memory (read as 16-byte broadcasts), four
+// of its rows at a time, so that four dot products and their shuffle steps are in flight together.
+// One warp per row with one key at a time, which these replace, waited for five shuffles and a global load per
+// key: 4 x 64 tokens, 4 heads of 32 (the tiny fp32 workload) is bound by that chain, not by its 17 MFLOP.
+// ------------------------------------------------------------------------------------------------
+constexpr int AR = 32;   // rows per CTA and per tile
 
-template <typename T>
-__device__ __forceinline__ void load_row(const T* p, int hd, int lane, float* v, float scale) {
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int d = lane + 32 * r;
-    v[r] = d < hd ? to_f(p[d]) * scale : 0.f;
+template <int HDP>
+constexpr int kLpr = HDP == 128 ? 8 : 4;   // lanes per row
+template <int HDP>
+struct RowV {
+  static constexpr int L = kLpr<HDP>, NC = HDP / (4 * L), N = HDP / L;
+  float v[N];
+};
+
+// Rows r0 .. r0 + AR - 1 (below `rows`) of a [rows, ld] matrix, hd columns, into an [AR][HDP + 4] tile.
+template <typename T, int HDP>
+__device__ __forceinline__ void tile_rows(float* dst, const T* src, int ld, int r0, int rows, int hd) {
+  for (int e = threadIdx.x; e < AR * HDP / 2; e += AR * kLpr<HDP>) {   // pairs: hd is even
+    const int r = e / (HDP / 2), d = (e % (HDP / 2)) * 2;
+    const bool ok = r0 + r < rows && d < hd;
+    const T* p = src + (size_t)(ok ? r0 + r : 0) * ld + (ok ? d : 0);
+    dst[r * (HDP + 4) + d] = ok ? to_f(p[0]) : 0.f;
+    dst[r * (HDP + 4) + d + 1] = ok ? to_f(p[1]) : 0.f;
   }
 }
-template <typename T>
-__device__ __forceinline__ float dot_row(const T* p, int hd, int lane, const float* v) {
-  float s = 0.f;
+template <typename T, int HDP>
+__device__ __forceinline__ void load_row(RowV<HDP>& o, const T* p, int hd, int sub, float scale, bool ok) {
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int d = lane + 32 * r;
-    if (d < hd) s += v[r] * to_f(p[d]);
+  for (int c = 0; c < RowV<HDP>::NC; ++c)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int d = 4 * (RowV<HDP>::L * c + sub) + q;
+      o.v[4 * c + q] = ok && d < hd ? to_f(p[d]) * scale : 0.f;
+    }
+}
+template <typename T, int HDP>
+__device__ __forceinline__ void store_row(T* p, const RowV<HDP>& o, int hd, int sub, float scale) {
+#pragma unroll
+  for (int c = 0; c < RowV<HDP>::NC; ++c)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int d = 4 * (RowV<HDP>::L * c + sub) + q;
+      if (d < hd) p[d] = from_f<T>(o.v[4 * c + q] * scale);
+    }
+}
+// The row's dot products with tile rows j .. j + 3, in every one of its lanes.
+template <int HDP>
+__device__ __forceinline__ void dot4(float* s, const RowV<HDP>& a, const float* tile, int j, int sub) {
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const float* t = tile + (j + u) * (HDP + 4) + 4 * sub;
+    float x = 0.f;
+#pragma unroll
+    for (int c = 0; c < RowV<HDP>::NC; ++c) {
+      const float4 b = *reinterpret_cast<const float4*>(t + 4 * RowV<HDP>::L * c);
+      x = fmaf(a.v[4 * c], b.x, x);
+      x = fmaf(a.v[4 * c + 1], b.y, x);
+      x = fmaf(a.v[4 * c + 2], b.z, x);
+      x = fmaf(a.v[4 * c + 3], b.w, x);
+    }
+    s[u] = x;
   }
-  return warp_sum(s);
+#pragma unroll
+  for (int x = 1; x < RowV<HDP>::L; x *= 2)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s[u] += __shfl_xor_sync(0xffffffffu, s[u], x);
+}
+// o += sum_u w[u] * tile row j + u
+template <int HDP>
+__device__ __forceinline__ void axpy4(RowV<HDP>& o, const float* w, const float* tile, int j, int sub) {
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const float* t = tile + (j + u) * (HDP + 4) + 4 * sub;
+#pragma unroll
+    for (int c = 0; c < RowV<HDP>::NC; ++c) {
+      const float4 b = *reinterpret_cast<const float4*>(t + 4 * RowV<HDP>::L * c);
+      o.v[4 * c] = fmaf(w[u], b.x, o.v[4 * c]);
+      o.v[4 * c + 1] = fmaf(w[u], b.y, o.v[4 * c + 1]);
+      o.v[4 * c + 2] = fmaf(w[u], b.z, o.v[4 * c + 2]);
+      o.v[4 * c + 3] = fmaf(w[u], b.w, o.v[4 * c + 3]);
+    }
+  }
 }
 
-template <typename T>
-__global__ void attn_fwd_k(const T* __restrict__ qkv, T* __restrict__ out, float* __restrict__ lse, int B, int S,
-                           int H, int Hkv, int hd, float scale) {
-  const long gw = (blockIdx.x * (long)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (gw >= (long)B * H * S) return;
-  const int i = S - 1 - (int)(gw % S);              // long rows first
-  const int h = (int)((gw / S) % H), b = (int)(gw / ((long)S * H));
-  const int ld = (H + 2 * Hkv) * hd, kvh = h / (H / Hkv);
-  float q[R], o[R] = {0.f, 0.f, 0.f, 0.f};
-  load_row(qkv + (size_t)(b * S + i) * ld + h * hd, hd, lane, q, scale);
+template <typename T, int HDP>
+__global__ void __launch_bounds__(AR * kLpr<HDP>) attn_fwd_k(const T* __restrict__ qkv, T* __restrict__ out, float* __restrict__ lse,
+                                                  int S, int H, int Hkv, int hd, float scale, int nt) {
+  __shared__ __align__(16) float ks[AR * (HDP + 4)], vs[AR * (HDP + 4)];
+  pdl_wait();
+  pdl_trigger();
+  const int h = blockIdx.x / nt, b = blockIdx.y, i0 = (nt - 1 - (int)blockIdx.x % nt) * AR;   // long rows first
+  const int ld = (H + 2 * Hkv) * hd, kvh = h / (H / Hkv), sub = threadIdx.x % kLpr<HDP>, i = i0 + threadIdx.x / kLpr<HDP>;
+  const T* base = qkv + (size_t)b * S * ld;
+  RowV<HDP> q, o;
+  load_row<T, HDP>(q, base + (size_t)min(i, S - 1) * ld + h * hd, hd, sub, scale, i < S);
+#pragma unroll
+  for (int d = 0; d < RowV<HDP>::N; ++d) o.v[d] = 0.f;
   float m = -INFINITY, l = 0.f;
-  const T* kb = qkv + (size_t)b * S * ld + (H + kvh) * hd;
-  const T* vb = qkv + (size_t)b * S * ld + (H + Hkv + kvh) * hd;
-  for (int j = 0; j <= i; ++j) {
-    const float s = dot_row(kb + (size_t)j * ld, hd, lane, q);
-    const float mn = fmaxf(m, s);
-    const float corr = expf(m - mn), p = expf(s - mn);
-    l = l * corr + p;
-    const T* vr = vb + (size_t)j * ld;
+  for (int j0 = 0; j0 <= i0; j0 += AR) {
+    __syncthreads();
+    tile_rows<T, HDP>(ks, base + (H + kvh) * hd, ld, j0, S, hd);
+    tile_rows<T, HDP>(vs, base + (H + Hkv + kvh) * hd, ld, j0, S, hd);
+    __syncthreads();
+#pragma unroll 1
+    for (int j = 0; j < AR; j += 4) {
+      float s[4];
+      dot4<HDP>(s, q, ks, j, sub);
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int d = lane + 32 * r;
-      o[r] = o[r] * corr + (d < hd ? p * to_f(vr[d]) : 0.f);
-    }
-    m = mn;
-  }
-  T* orow = out + (size_t)(b * S + i) * H * hd + h * hd;
-  const float inv = 1.f / l;
+      for (int u = 0; u < 4; ++u)
+        if (j0 + j + u > i) s[u] = -INFINITY;
+      const float mn = fmaxf(m, fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3])));
+      if (mn > -INFINITY) {   // (past the row's last key a warp still runs for its other rows)
+        const float corr = expf(m - mn);
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int d = lane + 32 * r;
-    if (d < hd) orow[d] = from_f<T>(o[r] * inv);
-  }
-  if (lane == 0) lse[((size_t)b * H + h) * S + i] = m + logf(l);
-}
-
-// D_i = sum_d dO_i[d] * O_i[d]
-template <typename T>
-__global__ void attn_bwd_d_k(const T* __restrict__ out, const T* __restrict__ dout, float* __restrict__ D, int B,
-                             int S, int H, int hd) {
-  const long gw = (blockIdx.x * (long)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (gw >= (long)B * H * S) return;
-  const int i = (int)(gw % S), h = (int)((gw / S) % H), b = (int)(gw / ((long)S * H));
-  const size_t o = (size_t)(b * S + i) * H * hd + h * hd;
-  float v[R];
-  load_row(out + o, hd, lane, v, 1.f);
-  const float s = dot_row(dout + o, hd, lane, v);
-  if (lane == 0) D[((size_t)b * H + h) * S + i] = s;
-}
-
-template <typename T>
-__global__ void attn_bwd_dq_k(const T* __restrict__ qkv, const T* __restrict__ dout, const float* __restrict__ lse,
-                              const float* __restrict__ D, T* __restrict__ dqkv, int B, int S, int H, int Hkv, int hd,
-                              float scale) {
-  const long gw = (blockIdx.x * (long)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (gw >= (long)B * H * S) return;
-  const int i = S - 1 - (int)(gw % S), h = (int)((gw / S) % H), b = (int)(gw / ((long)S * H));
-  const int ld = (H + 2 * Hkv) * hd, kvh = h / (H / Hkv);
-  float q[R], dO[R], dq[R] = {0.f, 0.f, 0.f, 0.f};
-  load_row(qkv + (size_t)(b * S + i) * ld + h * hd, hd, lane, q, scale);
-  load_row(dout + (size_t)(b * S + i) * H * hd + h * hd, hd, lane, dO, 1.f);
-  const size_t si = ((size_t)b * H + h) * S + i;
-  const float L = lse[si], Di = D[si];
-  const T* kb = qkv + (size_t)b * S * ld + (H + kvh) * hd;
-  const T* vb = qkv + (size_t)b * S * ld + (H + Hkv + kvh) * hd;
-  for (int j = 0; j <= i; ++j) {
-    const T* kr = kb + (size_t)j * ld;
-    const float p = expf(dot_row(kr, hd, lane, q) - L);
-    const float dp = dot_row(vb + (size_t)j * ld, hd, lane, dO);
-    const float ds = p * (dp - Di);
+        for (int u = 0; u < 4; ++u) s[u] = expf(s[u] - mn);
+        l = l * corr + ((s[0] + s[1]) + (s[2] + s[3]));
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int d = lane + 32 * r;
-      if (d < hd) dq[r] += ds * to_f(kr[d]);
-    }
-  }
-  T* dr = dqkv + (size_t)(b * S + i) * ld + h * hd;
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int d = lane + 32 * r;
-    if (d < hd) dr[d] = from_f<T>(dq[r] * scale);
-  }
-}
-
-template <typename T>
-__global__ void attn_bwd_dkv_k(const T* __restrict__ qkv, const T* __restrict__ dout, const float* __restrict__ lse,
-                               const float* __restrict__ D, T* __restrict__ dqkv, int B, int S, int H, int Hkv, int hd,
-                               float scale) {
-  const long gw = (blockIdx.x * (long)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (gw >= (long)B * Hkv * S) return;
-  const int j = (int)(gw % S), kvh = (int)((gw / S) % Hkv), b = (int)(gw / ((long)S * Hkv));
-  const int ld = (H + 2 * Hkv) * hd, rep = H / Hkv;
-  float k[R], v[R], dk[R] = {0.f, 0.f, 0.f, 0.f}, dv[R] = {0.f, 0.f, 0.f, 0.f};
-  load_row(qkv + (size_t)(b * S + j) * ld + (H + kvh) * hd, hd, lane, k, scale);
-  load_row(qkv + (size_t)(b * S + j) * ld + (H + Hkv + kvh) * hd, hd, lane, v, 1.f);
-  for (int hh = 0; hh < rep; ++hh) {
-    const int h = kvh * rep + hh;
-    for (int i = j; i < S; ++i) {
-      const T* qr = qkv + (size_t)(b * S + i) * ld + h * hd;
-      const T* dor = dout + (size_t)(b * S + i) * H * hd + h * hd;
-      const size_t si = ((size_t)b * H + h) * S + i;
-      const float p = expf(dot_row(qr, hd, lane, k) - lse[si]);
-      const float dp = dot_row(dor, hd, lane, v);
-      const float ds = p * (dp - D[si]);
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int d = lane + 32 * r;
-        if (d < hd) { dv[r] += p * to_f(dor[d]); dk[r] += ds * to_f(qr[d]); }
+        for (int d = 0; d < RowV<HDP>::N; ++d) o.v[d] *= corr;
+        axpy4<HDP>(o, s, vs, j, sub);
+        m = mn;
       }
     }
   }
-  T* dkr = dqkv + (size_t)(b * S + j) * ld + (H + kvh) * hd;
-  T* dvr = dqkv + (size_t)(b * S + j) * ld + (H + Hkv + kvh) * hd;
+  if (i >= S) return;
+  store_row<T, HDP>(out + (size_t)(b * S + i) * H * hd + h * hd, o, hd, sub, 1.f / l);
+  if (sub == 0) lse[((size_t)b * H + h) * S + i] = m + logf(l);
+}
+
+// Of head y's 2 nt blocks the first nt form dQ of 32 queries each, the others (y < Hkv) dK and dV of 32 keys of KV
+// head y, summed over its query heads in order. D = rowsum(dO * O) is formed wherever a row needs it.
+template <typename T, int HDP>
+__global__ void __launch_bounds__(AR * kLpr<HDP>) attn_bwd_k(const T* __restrict__ qkv, const T* __restrict__ out,
+                                                  const T* __restrict__ dout, const float* __restrict__ lse,
+                                                  T* __restrict__ dqkv, int S, int H, int Hkv, int hd, float scale,
+                                                  int nt) {
+  __shared__ __align__(16) float ta[AR * (HDP + 4)], tb[AR * (HDP + 4)];
+  __shared__ float sl[AR], sd[AR];
+  pdl_wait();
+  pdl_trigger();
+  const int b = blockIdx.y, sub = threadIdx.x % kLpr<HDP>, row = threadIdx.x / kLpr<HDP>;
+  const int y = blockIdx.x / (2 * nt), x = blockIdx.x % (2 * nt);
+  const int ld = (H + 2 * Hkv) * hd, lo = H * hd, rep = H / Hkv;
+  const T* base = qkv + (size_t)b * S * ld;
+  auto row_d = [&](int h, int i) {   // D of query i, in each of its lanes
+    const size_t o = (size_t)(b * S + min(i, S - 1)) * lo + h * hd;
+    float d2 = 0.f;
+#pragma unroll 4
+    for (int d = sub; d < hd; d += kLpr<HDP>) d2 = fmaf(to_f(out[o + d]), to_f(dout[o + d]), d2);
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int d = lane + 32 * r;
-    if (d < hd) { dkr[d] = from_f<T>(dk[r] * scale); dvr[d] = from_f<T>(dv[r]); }
+    for (int m = 1; m < kLpr<HDP>; m *= 2) d2 += __shfl_xor_sync(0xffffffffu, d2, m);
+    return d2;
+  };
+  if (x < nt) {
+    const int h = y, kvh = h / rep, i0 = (nt - 1 - x) * AR, i = i0 + row;
+    RowV<HDP> q, g, dq;
+    load_row<T, HDP>(q, base + (size_t)min(i, S - 1) * ld + h * hd, hd, sub, scale, i < S);
+    load_row<T, HDP>(g, dout + (size_t)(b * S + min(i, S - 1)) * lo + h * hd, hd, sub, 1.f, i < S);
+#pragma unroll
+    for (int d = 0; d < RowV<HDP>::N; ++d) dq.v[d] = 0.f;
+    const float D = row_d(h, i), L = lse[((size_t)b * H + h) * S + min(i, S - 1)];
+    for (int j0 = 0; j0 <= i0; j0 += AR) {
+      __syncthreads();
+      tile_rows<T, HDP>(ta, base + (H + kvh) * hd, ld, j0, S, hd);
+      tile_rows<T, HDP>(tb, base + (H + Hkv + kvh) * hd, ld, j0, S, hd);
+      __syncthreads();
+#pragma unroll 1
+      for (int j = 0; j < AR; j += 4) {
+        float s[4], dp[4];
+        dot4<HDP>(s, q, ta, j, sub);
+        dot4<HDP>(dp, g, tb, j, sub);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) s[u] = j0 + j + u <= i ? expf(s[u] - L) * (dp[u] - D) : 0.f;
+        axpy4<HDP>(dq, s, ta, j, sub);
+      }
+    }
+    if (i < S) store_row<T, HDP>(dqkv + (size_t)(b * S + i) * ld + h * hd, dq, hd, sub, scale);
+    return;
+  }
+  if (y >= Hkv) return;
+  const int kvh = y, j0 = (x - nt) * AR, j = j0 + row;
+  RowV<HDP> k, v, dk, dv;
+  load_row<T, HDP>(k, base + (size_t)min(j, S - 1) * ld + (H + kvh) * hd, hd, sub, scale, j < S);
+  load_row<T, HDP>(v, base + (size_t)min(j, S - 1) * ld + (H + Hkv + kvh) * hd, hd, sub, 1.f, j < S);
+#pragma unroll
+  for (int d = 0; d < RowV<HDP>::N; ++d) dk.v[d] = dv.v[d] = 0.f;
+  for (int hh = 0; hh < rep; ++hh) {
+    const int h = kvh * rep + hh;
+    for (int i0 = j0; i0 < S; i0 += AR) {
+      __syncthreads();
+      tile_rows<T, HDP>(ta, base + h * hd, ld, i0, S, hd);
+      tile_rows<T, HDP>(tb, dout + (size_t)b * S * lo + h * hd, lo, i0, S, hd);
+      const float D = row_d(h, i0 + row);
+      if (sub == 0) {
+        sd[row] = D;
+        sl[row] = i0 + row < S ? lse[((size_t)b * H + h) * S + i0 + row] : INFINITY;
+      }
+      __syncthreads();
+#pragma unroll 1
+      for (int i = 0; i < AR; i += 4) {
+        float s[4], dp[4];
+        dot4<HDP>(s, k, ta, i, sub);
+        dot4<HDP>(dp, v, tb, i, sub);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          s[u] = i0 + i + u >= j ? expf(s[u] - sl[i + u]) : 0.f;
+          dp[u] = s[u] * (dp[u] - sd[i + u]);
+        }
+        axpy4<HDP>(dv, s, tb, i, sub);
+        axpy4<HDP>(dk, dp, ta, i, sub);
+      }
+    }
+  }
+  if (j < S) {
+    store_row<T, HDP>(dqkv + (size_t)(b * S + j) * ld + (H + kvh) * hd, dk, hd, sub, scale);
+    store_row<T, HDP>(dqkv + (size_t)(b * S + j) * ld + (H + Hkv + kvh) * hd, dv, hd, sub, 1.f);
   }
 }
 
-inline int warps_grid(long rows) { return (int)((rows * 32 + 255) / 256); }
+template <typename T, int HDP>
+void cuda_core_fwd(const void* qkv, void* out, float* lse, int B, int S, int H, int Hkv, int hd, float scale,
+                   cudaStream_t s) {
+  const int nt = (S + AR - 1) / AR;
+  launch_pdl(attn_fwd_k<T, HDP>, dim3((unsigned)H * nt, B), AR * kLpr<HDP>, 0, s, (const T*)qkv, (T*)out, lse, S, H, Hkv, hd, scale,
+             nt);
+}
+template <typename T, int HDP>
+void cuda_core_bwd(const void* qkv, const void* out, const void* dout, const float* lse, void* dqkv, int B, int S, int H,
+                   int Hkv, int hd, float scale, cudaStream_t s) {
+  const int nt = (S + AR - 1) / AR;
+  launch_pdl(attn_bwd_k<T, HDP>, dim3((unsigned)H * 2 * nt, B), AR * kLpr<HDP>, 0, s, (const T*)qkv, (const T*)out, (const T*)dout, lse,
+             (T*)dqkv, S, H, Hkv, hd, scale, nt);
+}
 
 // Head padding for the tcgen05 kernels (head dims 64 and 128): dst [N, nh * hp] from src [N, nh * hd] with
 // each head's columns hd .. hp - 1 zero (pad), or src [N, nh * hp] back to dst [N, nh * hd] (unpad).
@@ -257,37 +349,32 @@ bool attn_bwd_padded(const void* qkv, const void* out, const void* dout, const f
 
 void attn_fwd(int dt, const void* qkv, void* out, float* lse, int B, int S, int H, int Hkv, int hd, cudaStream_t s,
               unsigned* err, cudaMemPool_t pool) {
-  if (dt == BF16 && attn_fwd_tcgen05(qkv, out, lse, B, S, H, Hkv, hd, s, err, 1.f / sqrtf((float)hd))) return;
+  const float scale = 1.f / sqrtf((float)hd);
+  if (dt == BF16 && attn_fwd_tcgen05(qkv, out, lse, B, S, H, Hkv, hd, s, err, scale)) return;
   if (dt == BF16 && attn_fwd_padded(qkv, out, lse, B, S, H, Hkv, hd, s, err, pool)) return;
   note_launch(1);
   if (dt == BF16 && attn_fwd_tc(qkv, out, lse, B, S, H, Hkv, hd, s)) return;
-  const float scale = 1.f / sqrtf((float)hd);
-  const int g = warps_grid((long)B * H * S);
-  if (dt == BF16) attn_fwd_k<bf16><<<g, 256, 0, s>>>((const bf16*)qkv, (bf16*)out, lse, B, S, H, Hkv, hd, scale);
-  else attn_fwd_k<float><<<g, 256, 0, s>>>((const float*)qkv, (float*)out, lse, B, S, H, Hkv, hd, scale);
+#define CC(T)                                                                                  \
+  if (hd <= 32) cuda_core_fwd<T, 32>(qkv, out, lse, B, S, H, Hkv, hd, scale, s);               \
+  else if (hd <= 64) cuda_core_fwd<T, 64>(qkv, out, lse, B, S, H, Hkv, hd, scale, s);          \
+  else cuda_core_fwd<T, 128>(qkv, out, lse, B, S, H, Hkv, hd, scale, s);
+  if (dt == BF16) { CC(bf16) } else { CC(float) }
+#undef CC
 }
 
 void attn_bwd(int dt, const void* qkv, const void* out, const void* dout, const float* lse, float* Dbuf, void* dqkv,
               int B, int S, int H, int Hkv, int hd, cudaStream_t s, cudaMemPool_t pool, unsigned* err) {
-  note_launch(dt == BF16 ? (H > Hkv ? 3 : 2) : 3);
+  note_launch(dt == BF16 ? (H > Hkv ? 3 : 2) : 1);
   const float scale = 1.f / sqrtf((float)hd);
-  const int gq = warps_grid((long)B * H * S), gk = warps_grid((long)B * Hkv * S);
   if (dt == BF16 && attn_bwd_tcgen05(qkv, out, dout, lse, Dbuf, dqkv, B, S, H, Hkv, hd, s, pool, err, scale)) return;
   if (dt == BF16 && attn_bwd_padded(qkv, out, dout, lse, Dbuf, dqkv, B, S, H, Hkv, hd, s, pool, err)) return;
   if (dt == BF16 && attn_bwd_tc(qkv, out, dout, lse, Dbuf, dqkv, B, S, H, Hkv, hd, s, pool)) return;
-  if (dt == BF16) {
-    attn_bwd_d_k<bf16><<<gq, 256, 0, s>>>((const bf16*)out, (const bf16*)dout, Dbuf, B, S, H, hd);
-    attn_bwd_dq_k<bf16><<<gq, 256, 0, s>>>((const bf16*)qkv, (const bf16*)dout, lse, Dbuf, (bf16*)dqkv, B, S, H, Hkv,
-                                           hd, scale);
-    attn_bwd_dkv_k<bf16><<<gk, 256, 0, s>>>((const bf16*)qkv, (const bf16*)dout, lse, Dbuf, (bf16*)dqkv, B, S, H,
-                                            Hkv, hd, scale);
-  } else {
-    attn_bwd_d_k<float><<<gq, 256, 0, s>>>((const float*)out, (const float*)dout, Dbuf, B, S, H, hd);
-    attn_bwd_dq_k<float><<<gq, 256, 0, s>>>((const float*)qkv, (const float*)dout, lse, Dbuf, (float*)dqkv, B, S, H,
-                                            Hkv, hd, scale);
-    attn_bwd_dkv_k<float><<<gk, 256, 0, s>>>((const float*)qkv, (const float*)dout, lse, Dbuf, (float*)dqkv, B, S,
-                                             H, Hkv, hd, scale);
-  }
+#define CC(T)                                                                                        \
+  if (hd <= 32) cuda_core_bwd<T, 32>(qkv, out, dout, lse, dqkv, B, S, H, Hkv, hd, scale, s);         \
+  else if (hd <= 64) cuda_core_bwd<T, 64>(qkv, out, dout, lse, dqkv, B, S, H, Hkv, hd, scale, s);    \
+  else cuda_core_bwd<T, 128>(qkv, out, dout, lse, dqkv, B, S, H, Hkv, hd, scale, s);
+  if (dt == BF16) { CC(bf16) } else { CC(float) }
+#undef CC
 }
 
 }  // namespace zl

@@ -359,7 +359,7 @@ void GW(zl_ctx* c, cudaStream_t s, Chunk& k, int li, PK p, int M, int N, int K, 
   // operands, then read theta, m, v and write them back, plus the compute copy
   const double upd = 24.0 * mn + (c->dt == BF16 ? 2.0 : 0.0) * mn;
   ProfScope ps(c, s, PC_GEMM_UPD, 2.0 * mn * (double)K, e * ((double)M * K + (double)N * K) + upd);
-  if (c->dt == BF16 && gemm_tc_update(M, N, K, A, B, u, c->d_err, s, c->pool)) return;
+  if (c->dt == BF16 ? gemm_tc_update(M, N, K, A, B, u, c->d_err, s, c->pool) : gemm_f32_update(M, N, K, A, B, u, s)) return;
   // the gradient in the accumulator (or, where the matrix has none, a zeroed pool buffer), then the step
   float* tmp = nullptr;
   if (!g) {

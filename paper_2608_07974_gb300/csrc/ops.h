@@ -117,6 +117,8 @@ struct GemmUpdate {
 // (the caller then forms the gradient with gemm() and applies the step with launch_adamw_ranges).
 bool gemm_tc_update(int M, int N, int K, const void* A, const void* B, const GemmUpdate& u, unsigned* err,
                     cudaStream_t s, cudaMemPool_t pool, float alpha = 1.f);
+// The same in fp32 (comp and g NULL) on the CUDA-core kernel; false when its alignment rules do not hold.
+bool gemm_f32_update(int M, int N, int K, const void* A, const void* B, const GemmUpdate& u, cudaStream_t s);
 // Rotate-half RoPE applied by the forward QKV product's epilogue: output columns < cols (the query and key
 // heads, head dim hd = 64 or 128) of row n are rotated by the angles of position n % S, (cos, sin) pairs
 // from cs [S][hd / 2][2] (fp32). The product is rounded to the output type before the rotation, as a

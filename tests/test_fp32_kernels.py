@@ -1,0 +1,60 @@
+"""The fp32 CUDA-core kernels at the edges of their tiles, splits and head-dim classes (GPU), against float64."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    import paper_2608_07974_gb300 as pkg
+    pkg.build()
+    from paper_2608_07974_gb300 import binding
+    return binding
+
+
+# Tiles of 32 with K in 1, 2 or 4 shares (the last one short), tiles of 64, ragged rows and columns, and rows that
+# are not a multiple of 16 bytes (the plain kernel).
+@pytest.mark.parametrize("mode", [0, 1, 2])
+@pytest.mark.parametrize("M,N,K", [(32, 32, 64), (256, 128, 344), (256, 384, 128), (100, 36, 260), (4, 4, 4), (36, 1200, 512),
+                                   (1300, 1236, 68), (33, 35, 37), (256, 688, 128), (64, 64, 1028)])
+def test_fp32_gemm(B, mode, M, N, K):
+    g = torch.Generator(device="cuda").manual_seed(M + 3 * N + 7 * K)
+    shp = {0: ((M, K), (N, K)), 1: ((M, K), (K, N)), 2: ((K, M), (K, N))}[mode]
+    a, b = (torch.randn(*s, device="cuda", generator=g) for s in shp)
+    c0 = torch.randn(M, N, device="cuda", generator=g)
+    bias, c = torch.randn(N, device="cuda", generator=g), c0.clone()
+    p = {0: lambda: a.double() @ b.double().T, 1: lambda: a.double() @ b.double(), 2: lambda: a.double().T @ b.double()}[mode]()
+    if mode == 2:
+        B.zl_op_gemm(0, 2, M, N, K, a, b, c)
+        ref = c0.double() + p
+    else:
+        B.zl_op_gemm_ex(0, mode, M, N, K, a, b, c, bias, c0, 0)
+        ref = p + bias.double() + c0.double()
+    # an fp32 sum of K unit-variance products: at most K rounding errors of 2^-24 of a partial sum of about sqrt(K)
+    assert float((c - ref).abs().max()) <= 2.0 ** -24 * 4 * (K + 8) ** 0.5 * max(8.0, K ** 0.5)
+    assert float((c - ref).norm() / ref.norm()) <= 1e-6
+
+
+@pytest.mark.parametrize("Bb,S,H,Hkv,hd", [(4, 64, 4, 4, 32), (1, 31, 2, 1, 30), (2, 33, 4, 2, 34), (1, 65, 3, 3, 64),
+                                           (2, 96, 4, 1, 66), (1, 100, 2, 2, 128), (1, 1, 2, 2, 2)])
+def test_fp32_attention(B, Bb, S, H, Hkv, hd):
+    g = torch.Generator(device="cuda").manual_seed(S + 7 * H + hd)
+    W = (H + 2 * Hkv) * hd
+    qkv, dout = torch.randn(Bb * S, W, device="cuda", generator=g), torch.randn(Bb * S, H * hd, device="cuda", generator=g)
+    out, dqkv = torch.full_like(dout, float("nan")), torch.full_like(qkv, float("nan"))
+    lse = torch.full((Bb, H, S), float("nan"), device="cuda")
+    B.zl_op_attention(0, qkv, out, lse, Bb, S, H, Hkv, hd)
+    B.zl_op_attention_bwd(0, qkv, out, dout, lse, dqkv, Bb, S, H, Hkv, hd)
+    torch.cuda.synchronize()
+    x = qkv.double().requires_grad_(True)
+    t = x.view(Bb, S, H + 2 * Hkv, hd).transpose(1, 2)
+    k, v = (t[:, a:a + Hkv].repeat_interleave(H // Hkv, 1) for a in (H, H + Hkv))
+    s = (t[:, :H] @ k.transpose(-1, -2)) / hd ** 0.5
+    s = s.masked_fill(torch.ones(S, S, dtype=torch.bool, device="cuda").triu(1), float("-inf"))
+    ref = (torch.softmax(s, -1) @ v).transpose(1, 2).reshape(Bb * S, H * hd)
+    (gx,) = torch.autograd.grad(ref, x, dout.double())
+    # fp32 sums of up to max(S, hd) terms and expf (2 ulp): a few 1e-7 relative to the values' scale
+    assert float((lse - torch.logsumexp(s, -1).detach()).abs().max()) <= 1e-5
+    assert float((out - ref.detach()).abs().max()) <= 1e-5 * max(1.0, float(ref.detach().abs().max()))
+    assert float((dqkv - gx).abs().max()) <= 1e-5 * max(1.0, float(gx.abs().max()))
