@@ -158,6 +158,7 @@ struct zl_ctx {
   std::vector<cudaEvent_t> live_ring;
   long live_seq = 0;
   unsigned* d_err = nullptr;
+  unsigned* h_err = nullptr;     // pinned copy of *d_err
   int* d_count = nullptr;        // [K + 1] one |Omega| per stream
   float* d_losses = nullptr;     // [K + 1]
   float* h_losses = nullptr;     // pinned [K + 1]
@@ -955,20 +956,23 @@ void join_all(zl_ctx* c) {
 
 zl_status sync_all(zl_ctx* c, int timeout_ms) {
   join_all(c);
+  // the error word comes back with the wait itself, not in a copy of its own after it
+  CK(cudaMemcpyAsync(c->h_err, c->d_err, 4, cudaMemcpyDeviceToHost, c->user));
   rec(c->ev_sync, c->user);
+  // without a limit the runtime waits (and sees the end at once: polling with a sleep cost 50-120 us a call, which
+  // every read of a loss or a tensor paid); with one, polling
+  if (timeout_ms < 0) CK(cudaEventSynchronize(c->ev_sync));
   const auto t0 = std::chrono::steady_clock::now();
-  for (;;) {
+  while (timeout_ms >= 0) {
     cudaError_t e = cudaEventQuery(c->ev_sync);
     if (e == cudaSuccess) break;
     if (e != cudaErrorNotReady) CK(e);
-    if (timeout_ms >= 0 &&
-        std::chrono::duration_cast<std::chrono::milliseconds>(std::chrono::steady_clock::now() - t0).count() >
+    if (std::chrono::duration_cast<std::chrono::milliseconds>(std::chrono::steady_clock::now() - t0).count() >
             timeout_ms)
       raise_err(ZL_ERR_TIMEOUT, "zl_synchronize: queued work did not finish in time");
     std::this_thread::sleep_for(std::chrono::microseconds(50));
   }
-  unsigned err = 0;
-  CK(cudaMemcpy(&err, c->d_err, 4, cudaMemcpyDeviceToHost));
+  const unsigned err = *c->h_err;
   if (err) {
     CK(cudaMemset(c->d_err, 0, 4));
     std::string m = "device-side argument error:";
@@ -1095,6 +1099,7 @@ void free_ctx(zl_ctx* c) {
   if (c->aux && !shared) cudaStreamDestroy(c->aux);
   for (void* p : c->statics) cudaFree(p);
   if (c->h_losses) cudaFreeHost(c->h_losses);
+  if (c->h_err) cudaFreeHost(c->h_err);
   if (c->pool) cudaMemPoolDestroy(c->pool);
   delete c;
 }
@@ -1389,6 +1394,7 @@ zl_status zl_create(const zl_model_dims* dims, int K, const int* bounds, const z
     c->d_losses = (float*)salloc(c, (size_t)(K + 1) * 4);
     CK(cudaMemset(c->d_losses, 0, (size_t)(K + 1) * 4));
     CK(cudaMallocHost(&c->h_losses, (size_t)(K + 1) * 4));
+    CK(cudaMallocHost(&c->h_err, 4));
     CK(cudaDeviceSynchronize());
     return ZL_OK;
   });
@@ -1493,6 +1499,10 @@ zl_status zl_get_param(zl_ctx* c, const char* name, int which, void* dst, size_t
       for (int j = 0; j < f.trows; ++j)
         for (int o = 0; o < f.tcols; ++o) t[(size_t)o * f.trows + j] = h[(size_t)j * f.tcols + o];
       CK(cudaMemcpy(dst, t.data(), bytes, on_device ? cudaMemcpyHostToDevice : cudaMemcpyHostToHost));
+    } else if (f.brows > 0 && on_device && ((uintptr_t)dst & 15u) == 0) {   // blocked -> row-major, straight there
+      launch_blk_permute((const float*)srcp, (float*)dst, f.brows, f.bcols, 0, 0);
+      CHECK_LAUNCH();
+      CK(cudaStreamSynchronize(0));
     } else if (f.brows > 0) {   // blocked master or moment -> row-major
       float* tmp = nullptr;
       CK(cudaMalloc(&tmp, bytes));
