@@ -441,65 +441,102 @@ void carve_layer(zl_ctx* c, Arena& a, LayerSave& sv, int N, int B, int S, bool w
   for (int i = 0; i < 4; ++i) sv.u[i] = r > 0 ? a.take((size_t)N * r * e) : nullptr;
 }
 
-// LoRA on linear i (Delta w = s B A, Section II-A): u = X A^T [N, r16], out += s u (B^T).
-void lora_fwd(zl_ctx* c, Chunk& k, int li, int i, const void* X, void* out, void* u, int N, cudaStream_t s) {
+// u = scale X A^T [N, r16] for a LoRA factor A [r16, in].
+void lora_down(zl_ctx* c, const void* X, const void* A, void* u, int N, int in, float scale, cudaStream_t s) {
   const int r = lora_r16(c->cfg.lora_rank);
-  if (r <= 0) return;
-  const Layer& L = k.layers[li];
-  G(c, s, 0, N, r, L.lin_in[i], X, TrainC(c, k, L.la[i]), u, nullptr, nullptr);
-  G(c, s, 1, N, L.lin_out[i], r, u, TrainC(c, k, L.lb[i]), out, nullptr, out, c->cfg.lora_scale);
+  if (c->dt == BF16 && r == 16 && in % 8 == 0) {
+    const double e = (double)esz(c);
+    ProfScope p(c, s, PC_GEMM, 2.0 * N * r * (double)in, e * ((double)N * in + (double)r * in + (double)N * r));
+    launch_rank16(X, A, u, N, in, scale, s);
+    return;
+  }
+  G(c, s, 0, N, r, in, X, A, u, nullptr, nullptr, scale);
 }
 
-// LoRA backward of linear i, after dX holds dY W: du = s dY B; d(B^T) += s u^T dY; dA += du^T X;
-// dX += du A.
-void lora_bwd(zl_ctx* c, Chunk& k, int li, int i, const void* X, const void* u, const void* dY, void* dX, void* du,
-              int N, cudaStream_t s) {
+// C = A op(B) (+ bias) (+ R) + u F for a LoRA term u [M, r16], F [r16, N]: one product with further k blocks where the
+// tensor-core kernel takes it, else the term as a product of its own onto C.
+void G_lora(zl_ctx* c, cudaStream_t s, int mode, int M, int N, int K, const void* A, const void* B, void* C,
+            const float* bias, const void* R, const void* u, const void* F) {
   const int r = lora_r16(c->cfg.lora_rank);
-  if (r <= 0) return;
+  if (c->dt == BF16) {
+    const double e = (double)esz(c), m = M, n = N, kk = K + r;
+    ProfScope p(c, s, PC_GEMM, 2.0 * m * n * kk, e * (m * kk + n * kk + (R ? 2.0 : 1.0) * m * n));
+    if (gemm_tc_ext(mode, M, N, K, A, B, C, bias, R, GemmExt{u, F, r}, nullptr, c->d_err, s, c->pool)) return;
+    p.keep = false;
+  }
+  G(c, s, mode, M, N, K, A, B, C, bias, R);
+  G(c, s, 1, M, N, r, u, F, C, nullptr, C);
+}
+
+// One linear of the layer forward, out = X W^T (+ bias) (+ R), with LoRA on it (Delta w = s B A, Section II-A): u = s X
+// A^T is kept for the backward, out += u B^T.
+void linear_fwd(zl_ctx* c, Chunk& k, int li, int i, const void* X, void* out, const float* bias, const void* R, void* u,
+                int N, cudaStream_t s) {
   const Layer& L = k.layers[li];
-  const float sc = c->cfg.lora_scale;
-  G(c, s, 0, N, r, L.lin_out[i], dY, TrainC(c, k, L.lb[i]), du, nullptr, nullptr, sc);
-  G(c, s, 2, r, L.lin_out[i], N, u, dY, k.grad + L.lb[i], nullptr, nullptr, sc);
-  G(c, s, 2, r, L.lin_in[i], N, du, X, k.grad + L.la[i], nullptr, nullptr);
-  G(c, s, 1, N, L.lin_in[i], r, du, TrainC(c, k, L.la[i]), dX, nullptr, dX);
+  const void* W = Wc(c, k, li, (PK)kLoraP[i]);
+  const int in = L.lin_in[i], o = L.lin_out[i];
+  if (lora_r16(c->cfg.lora_rank) <= 0) {
+    G(c, s, 0, N, o, in, X, W, out, bias, R);
+    return;
+  }
+  lora_down(c, X, TrainC(c, k, L.la[i]), u, N, in, c->cfg.lora_scale, s);
+  G_lora(c, s, 0, N, o, in, X, W, out, bias, R, u, TrainC(c, k, L.lb[i]));
+}
+
+// dX = dY W of linear i and, with LoRA, its term and factor gradients: du = s dY B; dX += du A; d(B^T) += u^T dY
+// (u carries the scale); dA += du^T X.
+void linear_bwd_dx(zl_ctx* c, Chunk& k, int li, int i, const void* X, const void* u, const void* dY, void* dX, void* du,
+                   int N, cudaStream_t s) {
+  const Layer& L = k.layers[li];
+  const void* W = Wc(c, k, li, (PK)kLoraP[i]);
+  const int in = L.lin_in[i], o = L.lin_out[i], r = lora_r16(c->cfg.lora_rank);
+  if (r <= 0) {
+    G(c, s, 1, N, in, o, dY, W, dX, nullptr, nullptr);
+    return;
+  }
+  lora_down(c, dY, TrainC(c, k, L.lb[i]), du, N, o, c->cfg.lora_scale, s);
+  G_lora(c, s, 1, N, in, o, dY, W, dX, nullptr, nullptr, du, TrainC(c, k, L.la[i]));
+  G(c, s, 2, r, o, N, u, dY, k.grad + L.lb[i], nullptr, nullptr);
+  G(c, s, 2, r, in, N, du, X, k.grad + L.la[i], nullptr, nullptr);
 }
 
 void layer_fwd(zl_ctx* c, Chunk& k, int li, LayerSave& sv, const void* x, void* y, int B, int S, cudaStream_t s) {
   const int N = B * S, dt = c->dt;
   sv.x = x;
   NF(c, s, x, Wm(k, li, P_N1W), Wm(k, li, P_N1B), sv.xn1, sv.rstd1, sv.mean1, N);
-  // Llama without LoRA on the QKV product: RoPE in the product's epilogue; otherwise a RoPE pass after
-  // the product (and after the LoRA term, which the rotation must see)
+  // Llama: RoPE in the QKV product's epilogue (after the LoRA term, which is part of the product); otherwise a RoPE
+  // pass after the product
   bool rotated = false;
-  if (c->llama && dt == BF16 && lora_r16(c->cfg.lora_rank) <= 0) {
-    const double e = (double)esz(c), M = N, Nq = c->qkvw, K = c->d;
+  if (c->llama && dt == BF16) {
+    const int r16 = lora_r16(c->cfg.lora_rank);
+    const Layer& L = k.layers[li];
+    if (r16 > 0) lora_down(c, sv.xn1, TrainC(c, k, L.la[0]), sv.u[0], N, c->d, c->cfg.lora_scale, s);
+    const double e = (double)esz(c), M = N, Nq = c->qkvw, K = c->d + r16;
     ProfScope p(c, s, PC_GEMM, 2.0 * M * Nq * K, e * (M * K + Nq * K + M * Nq));
     const GemmRope r{c->rope_cs, S, c->hd, (c->H + c->Hkv) * c->hd};
-    rotated = gemm_tc_rope(N, c->qkvw, c->d, sv.xn1, Wc(c, k, li, P_WQKV), sv.qkv, Wm(k, li, P_BQKV), r, c->d_err,
-                           s, c->pool);
+    const void* W = Wc(c, k, li, P_WQKV);
+    rotated = r16 > 0 ? gemm_tc_ext(0, N, c->qkvw, c->d, sv.xn1, W, sv.qkv, nullptr, nullptr,
+                                    GemmExt{sv.u[0], TrainC(c, k, L.lb[0]), r16}, &r, c->d_err, s, c->pool)
+                      : gemm_tc_rope(N, c->qkvw, c->d, sv.xn1, W, sv.qkv, Wm(k, li, P_BQKV), r, c->d_err, s, c->pool);
     p.keep = rotated;
   }
   if (!rotated) {
-    G(c, s, 0, N, c->qkvw, c->d, sv.xn1, Wc(c, k, li, P_WQKV), sv.qkv, Wm(k, li, P_BQKV), nullptr);
-    lora_fwd(c, k, li, 0, sv.xn1, sv.qkv, sv.u[0], N, s);
+    linear_fwd(c, k, li, 0, sv.xn1, sv.qkv, Wm(k, li, P_BQKV), nullptr, sv.u[0], N, s);
     if (c->llama) {
       ProfScope p(c, s, PC_ELEM, 0, 2.0 * esz(c) * (double)N * (c->H + c->Hkv) * c->hd);
       launch_rope(dt, sv.qkv, c->rope_cs, N, S, c->H, c->Hkv, c->hd, 0, s);
     }
   }
   AF(c, s, sv.qkv, sv.att, sv.lse, B, S);
-  G(c, s, 0, N, c->d, c->ad, sv.att, Wc(c, k, li, P_WO), sv.x2, Wm(k, li, P_BO), x);
-  lora_fwd(c, k, li, 1, sv.att, sv.x2, sv.u[1], N, s);
+  linear_fwd(c, k, li, 1, sv.att, sv.x2, Wm(k, li, P_BO), x, sv.u[1], N, s);
   NF(c, s, sv.x2, Wm(k, li, P_N2W), Wm(k, li, P_N2B), sv.xn2, sv.rstd2, sv.mean2, N);
-  G(c, s, 0, N, c->f1, c->d, sv.xn2, Wc(c, k, li, P_W1), sv.hid, Wm(k, li, P_B1), nullptr);
-  lora_fwd(c, k, li, 2, sv.xn2, sv.hid, sv.u[2], N, s);
+  linear_fwd(c, k, li, 2, sv.xn2, sv.hid, Wm(k, li, P_B1), nullptr, sv.u[2], N, s);
   {
     ProfScope p(c, s, PC_ELEM, 0, esz(c) * (double)N * (c->f1 + c->f));
     if (c->llama) launch_swiglu_fwd(dt, sv.hid, sv.act, N, c->f, s);
     else launch_gelu_fwd(dt, sv.hid, sv.act, (size_t)N * c->f, s);
   }
-  G(c, s, 0, N, c->d, c->f, sv.act, Wc(c, k, li, P_W2), y, Wm(k, li, P_B2), sv.x2);
-  lora_fwd(c, k, li, 3, sv.act, y, sv.u[3], N, s);
+  linear_fwd(c, k, li, 3, sv.act, y, Wm(k, li, P_B2), sv.x2, sv.u[3], N, s);
   CHECK_LAUNCH();
 }
 
@@ -600,39 +637,35 @@ void layer_bwd(zl_ctx* c, Chunk& k, int li, LayerSave& sv, const void* dy, void*
   // Every dX product comes before the weight-gradient product of the same matrix, which may update the
   // matrix in place (fused update).
   // FFN
-  G(c, s, 1, N, c->f, c->d, dy, Wc(c, k, li, P_W2), w.da, nullptr, nullptr);
+  linear_bwd_dx(c, k, li, 3, sv.act, sv.u[3], dy, w.da, w.du, N, s);
   GW(c, s, k, li, P_W2, c->d, c->f, N, dy, sv.act);
   bias_grad(c, dy, N, c->d, Gm(k, li, P_B2), w, q);
-  lora_bwd(c, k, li, 3, sv.act, sv.u[3], dy, w.da, w.du, N, s);
   {
     ProfScope p(c, s, PC_ELEM, 0, esz(c) * (double)N * (2.0 * c->f1 + c->f));
     if (c->llama) launch_swiglu_bwd(dt, sv.hid, w.da, w.dhid, N, c->f, s);
     else launch_gelu_bwd(dt, sv.hid, w.da, w.dhid, (size_t)N * c->f, s);
   }
   q.need(k.ev_ln1, q.ln1);   // the layer above's LN1 parameter sums read dxn
-  G(c, s, 1, N, c->d, c->f1, w.dhid, Wc(c, k, li, P_W1), w.dxn, nullptr, nullptr);
+  linear_bwd_dx(c, k, li, 2, sv.xn2, sv.u[2], w.dhid, w.dxn, w.du, N, s);
   GW(c, s, k, li, P_W1, c->f1, c->d, N, w.dhid, sv.xn2);
   bias_grad(c, w.dhid, N, c->f1, Gm(k, li, P_B1), w, q);
-  lora_bwd(c, k, li, 2, sv.xn2, sv.u[2], w.dhid, w.dxn, w.du, N, s);
   NBX(c, s, sv.x2, Wm(k, li, P_N2W), sv.rstd2, sv.mean2, w.dxn, dy, w.dx2, N);
   norm_param_grad(c, sv.x2, sv.rstd2, sv.mean2, w.dxn, N, Gm(k, li, P_N2W), Gm(k, li, P_N2B), w, q);
   q.ln2 = q.mark(k.ev_ln2);
   // attention
-  G(c, s, 1, N, c->ad, c->d, w.dx2, Wc(c, k, li, P_WO), w.datt, nullptr, nullptr);
+  linear_bwd_dx(c, k, li, 1, sv.att, sv.u[1], w.dx2, w.datt, w.du, N, s);
   GW(c, s, k, li, P_WO, c->d, c->ad, N, w.dx2, sv.att);
   bias_grad(c, w.dx2, N, c->d, Gm(k, li, P_BO), w, q);
-  lora_bwd(c, k, li, 1, sv.att, sv.u[1], w.dx2, w.datt, w.du, N, s);
   AB(c, s, sv.qkv, sv.att, w.datt, sv.lse, w.D, w.dqkv, B, S);
   if (c->llama) {
     ProfScope p(c, s, PC_ELEM, 0, 2.0 * esz(c) * (double)N * (c->H + c->Hkv) * c->hd);
     launch_rope(dt, w.dqkv, c->rope_cs, N, S, c->H, c->Hkv, c->hd, 1, s);
   }
   q.need(k.ev_ln2, q.ln2);        // LN2 parameter sums read dxn, which the next product overwrites
-  G(c, s, 1, N, c->d, c->qkvw, w.dqkv, Wc(c, k, li, P_WQKV), w.dxn, nullptr, nullptr);
+  linear_bwd_dx(c, k, li, 0, sv.xn1, sv.u[0], w.dqkv, w.dxn, w.du, N, s);
   GW(c, s, k, li, P_WQKV, c->qkvw, c->d, N, w.dqkv, sv.xn1);
   bias_grad(c, w.dqkv, N, c->qkvw, Gm(k, li, P_BQKV), w, q);
   q.layer = q.mark(k.ev_layer);   // after this layer's sums over dy, dhid, dx2 and dqkv
-  lora_bwd(c, k, li, 0, sv.xn1, sv.u[0], w.dqkv, w.dxn, w.du, N, s);
   norm_param_grad(c, sv.x, sv.rstd1, sv.mean1, w.dxn, N, Gm(k, li, P_N1W), Gm(k, li, P_N1B), w, q);
   q.ln1 = q.mark(k.ev_ln1);
   if (dx) NBX(c, s, sv.x, Wm(k, li, P_N1W), sv.rstd1, sv.mean1, w.dxn, w.dx2, dx, N);

@@ -118,6 +118,8 @@ struct Args {
   GemmUpdate u;               // mode 4
   const float2* rope_cs;      // mode 0: rotate-half RoPE of columns < rope_cols (heads of rope_hd = 64 or 128),
   int rope_S, rope_hd, rope_cols;   // row n by position n % rope_S (NULL: none)
+  int nk2;                    // modes 0/1: further k blocks, of a second product A2 B2 into the same accumulator
+                              // (A2 [M, K2] K-major, B2 [K2, N] MN-major; a map's rows past K2 are zeros)
 };
 
 // Instruction descriptor of kind::f16: fp32 accumulator, bf16 A and B, operand majors, N, M.
@@ -157,7 +159,8 @@ __device__ __forceinline__ void unit_tile(const Args& g, int unit, int num_tiles
 template <int BN, bool A_MN, bool B_MN, bool UPD = false, bool PAIR = false>
 __global__ void __launch_bounds__(UPD ? kThreadsUpd : kThreads, 1)
     gemm_tc_k(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
-              const __grid_constant__ CUtensorMap tcm, const Args g) {
+              const __grid_constant__ CUtensorMap tcm, const __grid_constant__ CUtensorMap ta2,
+              const __grid_constant__ CUtensorMap tb2, const Args g) {
   using C_ = Cfg<BN, UPD, PAIR>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -206,7 +209,7 @@ __global__ void __launch_bounds__(UPD ? kThreadsUpd : kThreads, 1)
   // next GEMM of the stream begin its own set-up.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int nk = (g.K + BK - 1) / BK;
+  const int nk1 = (g.K + BK - 1) / BK, nk = nk1 + (A_MN ? 0 : g.nk2);
   const int num_tiles = (PAIR ? (g.tiles_m + 1) / 2 : g.tiles_m) * g.tiles_n;
   const int num_units = num_tiles * g.splits;
 
@@ -234,37 +237,42 @@ __global__ void __launch_bounds__(UPD ? kThreadsUpd : kThreads, 1)
           if (leader) {
             uint8_t* sa = smem + stage * C_::STAGE_BYTES;
             uint8_t* sb = sa + C_::A_BYTES;
-            const int k0 = kb * BK;
+            // the second product's blocks follow the first's, from its own maps, B2 as an MN-major operand
+            const bool ext = !A_MN && kb >= nk1;
+            const int k0 = (ext ? kb - nk1 : kb) * BK;
+            const CUtensorMap* ma = ext ? &ta2 : &ta;
+            const CUtensorMap* mb = ext ? &tb2 : &tb;
+            const bool b_mn = B_MN || ext;
             if constexpr (PAIR) {   // this CTA's rows of A and its half of the B tile, on the first CTA's barrier
               if (crank == 0) mbar_expect_tx(&full[stage], 2 * C_::STAGE_BYTES);
               const uint32_t bar = cluster_addr(&full[stage], 0);
               constexpr int HB = BN / 2;
               const int n0 = tn * BN + (int)crank * HB;
               if (!A_MN) {
-                tma2d_pair(sa, &ta, bar, k0, tm * BM);
+                tma2d_pair(sa, ma, bar, k0, tm * BM);
               } else {
-                tma2d_pair(sa, &ta, bar, tm * BM, k0);
-                tma2d_pair(sa + 8192, &ta, bar, tm * BM + 64, k0);
+                tma2d_pair(sa, ma, bar, tm * BM, k0);
+                tma2d_pair(sa + 8192, ma, bar, tm * BM + 64, k0);
               }
-              if (!B_MN) {
-                tma2d_pair(sb, &tb, bar, k0, n0);
+              if (!b_mn) {
+                tma2d_pair(sb, mb, bar, k0, n0);
               } else {
   #pragma unroll
-                for (int j = 0; j < HB / 64; ++j) tma2d_pair(sb + j * 8192, &tb, bar, n0 + 64 * j, k0);
+                for (int j = 0; j < HB / 64; ++j) tma2d_pair(sb + j * 8192, mb, bar, n0 + 64 * j, k0);
               }
             } else {
               mbar_expect_tx(&full[stage], C_::STAGE_BYTES);
               if (!A_MN) {
-                tma2d(sa, &ta, &full[stage], k0, tm * BM);
+                tma2d(sa, ma, &full[stage], k0, tm * BM);
               } else {
-                tma2d(sa, &ta, &full[stage], tm * BM, k0);
-                tma2d(sa + 8192, &ta, &full[stage], tm * BM + 64, k0);
+                tma2d(sa, ma, &full[stage], tm * BM, k0);
+                tma2d(sa + 8192, ma, &full[stage], tm * BM + 64, k0);
               }
-              if (!B_MN) {
-                tma2d(sb, &tb, &full[stage], k0, tn * BN);
+              if (!b_mn) {
+                tma2d(sb, mb, &full[stage], k0, tn * BN);
               } else {
   #pragma unroll
-                for (int j = 0; j < BN / 64; ++j) tma2d(sb + j * 8192, &tb, &full[stage], tn * BN + 64 * j, k0);
+                for (int j = 0; j < BN / 64; ++j) tma2d(sb + j * 8192, mb, &full[stage], tn * BN + 64 * j, k0);
               }
             }
           }
@@ -292,7 +300,7 @@ __global__ void __launch_bounds__(UPD ? kThreadsUpd : kThreads, 1)
       // ---------------- MMA issuer ----------------
       // The whole warp runs the loop and the waits; one elected lane issues every product and every
       // commit that tracks them (of a pair, the first CTA's, for both).
-      constexpr uint32_t id = idesc<BN, A_MN, B_MN, PAIR>();
+      constexpr uint32_t id = idesc<BN, A_MN, B_MN, PAIR>(), id_mn = idesc<BN, A_MN, true, PAIR>();
       const bool leader = elect_one();
       int stage = 0, it = 0;
       uint32_t phase = 0;
@@ -311,11 +319,13 @@ __global__ void __launch_bounds__(UPD ? kThreadsUpd : kThreads, 1)
             const uint32_t a0 = su32(smem + stage * C_::STAGE_BYTES), b0 = a0 + C_::A_BYTES;
   #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk) {
+              const bool b_mn = B_MN || (!A_MN && kb >= nk1);
               const uint64_t ad = A_MN ? sdesc(a0 + kk * 2048, 8192, 1024) : sdesc(a0 + kk * 32, 16, 1024);
-              const uint64_t bd = B_MN ? sdesc(b0 + kk * 2048, 8192, 1024) : sdesc(b0 + kk * 32, 16, 1024);
+              const uint64_t bd = b_mn ? sdesc(b0 + kk * 2048, 8192, 1024) : sdesc(b0 + kk * 32, 16, 1024);
+              const uint32_t idk = b_mn ? id_mn : id;
               const uint32_t add = (kb > kb0 || kk > 0) ? 1u : 0u;
-              if (PAIR) mma_bf16_pair(d, ad, bd, id, add);
-              else mma_bf16(d, ad, bd, id, add);
+              if (PAIR) mma_bf16_pair(d, ad, bd, idk, add);
+              else mma_bf16(d, ad, bd, idk, add);
             }
             if (PAIR) mma_commit_pair(&empty[stage]);   // the stage is free in both CTAs
             else mma_commit(&empty[stage]);
@@ -741,7 +751,7 @@ bool make_map_c(CUtensorMap* m, const Args& a) {
 }
 
 template <int BN, bool A_MN, bool B_MN, bool UPD = false, bool PAIR = false>
-bool launch(const Args& a, const void* A, const void* B, cudaStream_t s, int ctas_per_sm) {
+bool launch(const Args& a, const void* A, const void* B, cudaStream_t s, int ctas_per_sm, const GemmExt* ext = nullptr) {
   using C_ = Cfg<BN, UPD, PAIR>;
   static bool attr = false;
   static int max_pairs = 0;   // clusters of two that can be resident at once
@@ -783,6 +793,10 @@ bool launch(const Args& a, const void* A, const void* B, cudaStream_t s, int cta
                         : make_map(&tb, B, (uint64_t)a.K, (uint64_t)a.N, 64, PAIR ? BN / 2 : BN);
   CUtensorMap tcm;
   if (!okA || !okB || !make_map_c(&tcm, a)) return false;
+  CUtensorMap ta2 = ta, tb2 = tb;
+  if (ext && (A_MN || !make_map(&ta2, ext->A2, (uint64_t)ext->K2, (uint64_t)a.M, 64, BM) ||
+              !make_map(&tb2, ext->B2, (uint64_t)a.N, (uint64_t)ext->K2, 64, 64)))
+    return false;
   int grid;
   if (PAIR) {   // one cluster of two per pair of tile rows, as many as can be resident
     const int units = (a.tiles_m + 1) / 2 * a.tiles_n * a.splits;
@@ -806,14 +820,17 @@ bool launch(const Args& a, const void* A, const void* B, cudaStream_t s, int cta
   at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = PAIR ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, kern, ta, tb, tcm, a) == cudaSuccess;
+  return cudaLaunchKernelEx(&cfg, kern, ta, tb, tcm, ta2, tb2, a) == cudaSuccess;
 }
 
 template <bool A_MN, bool B_MN>
-bool launch_bn(int bn, bool pair, const Args& a, const void* A, const void* B, cudaStream_t s) {
-  if (bn == 256) return pair ? launch<256, A_MN, B_MN, false, true>(a, A, B, s, 1) : launch<256, A_MN, B_MN>(a, A, B, s, 1);
-  if (bn == 128) return pair ? launch<128, A_MN, B_MN, false, true>(a, A, B, s, 1) : launch<128, A_MN, B_MN>(a, A, B, s, 1);
-  return launch<64, A_MN, B_MN>(a, A, B, s, 2);
+bool launch_bn(int bn, bool pair, const Args& a, const void* A, const void* B, cudaStream_t s,
+               const GemmExt* e = nullptr) {
+  if (bn == 256)
+    return pair ? launch<256, A_MN, B_MN, false, true>(a, A, B, s, 1, e) : launch<256, A_MN, B_MN>(a, A, B, s, 1, e);
+  if (bn == 128)
+    return pair ? launch<128, A_MN, B_MN, false, true>(a, A, B, s, 1, e) : launch<128, A_MN, B_MN>(a, A, B, s, 1, e);
+  return launch<64, A_MN, B_MN>(a, A, B, s, 2, e);
 }
 
 // The fused-update kernels (mode 4): 128 x 128 or 128 x 256 tiles, one CTA per SM.
@@ -885,7 +902,7 @@ namespace {
 // is outside the kernel's rules.
 bool run_tc(int mode, int M, int N, int K, const void* A, const void* B, void* C, const float* bias, const void* R,
             unsigned* err, cudaStream_t s, cudaMemPool_t pool, float alpha, int rmode, const GemmUpdate* u,
-            const GemmRope* rope = nullptr) {
+            const GemmRope* rope = nullptr, const GemmExt* ext = nullptr) {
   if (!tc::init()) return false;
   if (M < 16 || N < 16 || K < 16) return false;
   auto al16 = [](const void* p) { return ((uintptr_t)p & 15u) == 0; };
@@ -901,6 +918,8 @@ bool run_tc(int mode, int M, int N, int K, const void* A, const void* B, void* C
     return false;
   if ((mode == 0 || mode == 1) && K % 8 != 0) return false;
   if (mode >= 2 && M % 8 != 0) return false;
+  if (ext && (mode > 1 || ext->K2 < 16 || ext->K2 % 8 != 0 || !ext->A2 || !ext->B2 || !al16(ext->A2) || !al16(ext->B2)))
+    return false;
   const tc::Plan plan = tc::choose(mode, M, N, K);
   int bn = plan.bn, splits = plan.splits, pair = plan.pair;
   if (const char* force = std::getenv("ZL_GEMM_TILE")) {   // test hook "BN:SPLITS[:PAIR]": forces the plan
@@ -932,7 +951,8 @@ bool run_tc(int mode, int M, int N, int K, const void* A, const void* B, void* C
   const double a_bytes = (double)M * K * 2.0, b_bytes = (double)N * K * 2.0;
   a.group_m = (a_bytes <= 48e6 || a_bytes <= b_bytes) ? a.tiles_m : std::min(8, a.tiles_m);
   if (pair) a.group_m = (a.group_m + 1) / 2;   // in pairs of tile rows
-  const int nk = (K + tc::BK - 1) / tc::BK;
+  a.nk2 = ext ? (ext->K2 + tc::BK - 1) / tc::BK : 0;
+  const int nk = (K + tc::BK - 1) / tc::BK + a.nk2;
   a.kb_per_split = (nk + splits - 1) / splits;
   a.splits = (nk + a.kb_per_split - 1) / a.kb_per_split;   // no empty split (its slice would never be formed)
   float* ws = nullptr;
@@ -954,8 +974,8 @@ bool run_tc(int mode, int M, int N, int K, const void* A, const void* B, void* C
   }
   note_launch(1);
   bool ok;
-  if (mode == 0) ok = tc::launch_bn<false, false>(bn, pair, a, A, B, s);
-  else if (mode == 1) ok = tc::launch_bn<false, true>(bn, pair, a, A, B, s);
+  if (mode == 0) ok = tc::launch_bn<false, false>(bn, pair, a, A, B, s, ext);
+  else if (mode == 1) ok = tc::launch_bn<false, true>(bn, pair, a, A, B, s, ext);
   else if (a.mode == 4) ok = tc::launch_upd(bn, pair, a, A, B, s);
   else ok = tc::launch_bn<true, true>(bn, pair, a, A, B, s);
   if (ws) {
@@ -987,6 +1007,11 @@ bool gemm_tc_update(int M, int N, int K, const void* A, const void* B, const Gem
 bool gemm_tc_rope(int M, int N, int K, const void* A, const void* B, void* C, const float* bias, const GemmRope& r,
                   unsigned* err, cudaStream_t s, cudaMemPool_t pool) {
   return run_tc(0, M, N, K, A, B, C, bias, nullptr, err, s, pool, 1.f, 0, nullptr, &r);
+}
+
+bool gemm_tc_ext(int mode, int M, int N, int K, const void* A, const void* B, void* C, const float* bias, const void* R,
+                 const GemmExt& e, const GemmRope* rope, unsigned* err, cudaStream_t s, cudaMemPool_t pool) {
+  return run_tc(mode, M, N, K, A, B, C, bias, R, err, s, pool, 1.f, 0, nullptr, rope, &e);
 }
 
 }  // namespace zl

@@ -131,6 +131,17 @@ struct GemmRope {
 // tensor-core product or the rotation's rules do not hold (the caller then runs gemm() and launch_rope).
 bool gemm_tc_rope(int M, int N, int K, const void* A, const void* B, void* C, const float* bias, const GemmRope& r,
                   unsigned* err, cudaStream_t s, cudaMemPool_t pool);
+// C = A op(B) + A2 B2 (+ bias) (+ R), modes 0 and 1: a second product (A2 [M, K2], B2 [K2, N], bf16, K2 a multiple
+// of 8 from 16) as further k blocks of the first, in one accumulation; with `rope` (mode 0, no R) rotated as by
+// gemm_tc_rope. False when the tensor-core rules do not hold.
+struct GemmExt {
+  const void *A2, *B2;
+  int K2;
+};
+bool gemm_tc_ext(int mode, int M, int N, int K, const void* A, const void* B, void* C, const float* bias, const void* R,
+                 const GemmExt& e, const GemmRope* rope, unsigned* err, cudaStream_t s, cudaMemPool_t pool);
+// U [N, 16] = scale * X [N, K] W [16, K]^T in bf16 (K % 8 == 0, 16-byte aligned rows): the rank-16 products of LoRA.
+void launch_rank16(const void* X, const void* W, void* U, int N, int K, float scale, cudaStream_t s);
 bool gemm_tc_available();
 bool gemm_tc(int mode, int M, int N, int K, const void* A, const void* B, void* C, const float* bias, const void* R,
              unsigned* err, cudaStream_t s, cudaMemPool_t pool, float alpha, int rmode = 0);

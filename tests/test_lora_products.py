@@ -1,0 +1,36 @@
+"""LoRA's products folded into the base products (bf16): ranks around one and two k blocks of 64, ragged token
+counts, head dims with and without the rotation in the epilogue, both architectures, against the oracle in fp32
+on the same bf16-rounded weights."""
+import pytest
+import torch
+
+import synth
+from tests.gpu_common import cosine, engine_for, oracle_for, rel
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("arch,rank,heads,kv,hd,batch,seq", [
+    (synth.ARCH_LLAMA, 4, 4, 2, 64, 3, 67), (synth.ARCH_LLAMA, 16, 2, 2, 128, 2, 130), (synth.ARCH_LLAMA, 20, 4, 4, 64, 1, 40),
+    (synth.ARCH_LLAMA, 70, 4, 1, 64, 2, 64), (synth.ARCH_LLAMA, 8, 4, 4, 50, 2, 33), (synth.ARCH_GPT2, 4, 4, 4, 64, 5, 51)])
+def test_lora_gradients(arch, rank, heads, kv, hd, batch, seq):
+    d = synth.ModelDims(arch, 2, heads * hd, heads, kv, 328, 640, 256)
+    w = synth.Workload("lora-products", d, "bf16", batch=batch, seq=seq, K=2, steps=1, seed=77)
+    P = synth.make_params(d, w.seed)
+    P.update(synth.make_lora_params(d, w.seed, rank, b_std=0.05))
+    P = {n: (synth.round_bf16(t) if t.dim() == 2 else t) for n, t in P.items()}
+    kw = dict(accum_m=2, lora_rank=rank, lora_scale=16.0 / rank)   # a window of two: the gradients stay readable
+    eng = engine_for(w, **kw)
+    eng.load(P)
+    ids, labels = synth.make_batch(w, 0)
+    losses = eng.step(ids.cuda(), labels.cuda())
+    orc = oracle_for(w, P, dtype=torch.float32, **kw)
+    h = eng.embed(ids.cuda()).float().cpu().view(batch, seq, -1)
+    for k in (1, 2):
+        L, g, _ = orc.local_grad(k, h, labels)
+        assert rel(losses[k - 1], L) <= 2e-2
+        for n in orc.chunk_names(k):
+            assert cosine(eng.get(n, 1), g[n]) >= 0.999, (k, n)
+        h = eng.forward_chunk(k, h.view(batch * seq, -1).to(torch.bfloat16).cuda(), None, batch, seq)
+        h = h.float().cpu().view(batch, seq, -1)
+    eng.close()
