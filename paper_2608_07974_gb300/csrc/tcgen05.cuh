@@ -37,10 +37,14 @@ __device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
 }
 // Waits for the phase of the given parity; false if the kernel is unwinding or the wait expired. The
 // limit is counted in SM cycles (clock64 is cheap to read; at lower clocks the limit only grows).
+// LAZY: sleeps between its tests, for a warp that waits long and is needed late (its polling takes issue slots
+// from the warps that work).
+template <bool LAZY = false>
 __device__ inline bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag, unsigned* err) {
   if (mbar_test(b, parity)) return true;
   const long long t0 = clock64();
   for (;;) {
+    if (LAZY) __nanosleep(256);
     if (mbar_test(b, parity)) return true;
     if (*abort_flag) return false;
     if (clock64() - t0 > kTimeoutCycles) {
@@ -52,8 +56,9 @@ __device__ inline bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abo
 }
 
 // The same wait by every lane of a warp (warp-uniform control flow); true only if it held for all.
+template <bool LAZY = false>
 __device__ __forceinline__ bool uwait(uint64_t* b, uint32_t parity, volatile int* abort_flag, unsigned* err) {
-  const bool ok = mbar_wait(b, parity, abort_flag, err);
+  const bool ok = mbar_wait<LAZY>(b, parity, abort_flag, err);
   return __all_sync(0xffffffffu, ok);
 }
 // One lane of the (converged) warp; tcgen05.mma and the tcgen05.commit that tracks it are issued inside
