@@ -189,6 +189,7 @@ __global__ void __launch_bounds__(FCfg<HD>::NTHR, 2)
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (warp == 2 && lane < 2) prefetch_map(lane == 0 ? &tqkv : &tout);   // under the kernel before
   if (warp == 1) tmem_alloc(tbase, C_::COLS);
   fence_before();
   __syncthreads();
@@ -520,6 +521,7 @@ __global__ void __launch_bounds__(NTHR_DQ, 1)
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (warp == 2 && lane < 2) prefetch_map(lane == 0 ? &tqkv : &tdo);   // under the kernel before
   if (warp == 1) tmem_alloc(tbase, 512);
   fence_before();
   __syncthreads();
@@ -808,6 +810,7 @@ __global__ void __launch_bounds__(NTHR_DKV, 1)
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (warp == 2 && lane < 2) prefetch_map(lane == 0 ? &tqkv : &tdo);   // under the kernel before
   if (warp == 1) tmem_alloc(tbase, 512);
   fence_before();
   __syncthreads();

@@ -181,6 +181,7 @@ __global__ void __launch_bounds__(UPD ? kThreadsUpd : kThreads, 1)
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (warp == 2 && lane < 3) prefetch_map(lane == 0 ? &ta : lane == 1 ? &tb : &tcm);   // under the kernel before
   if (warp == 1) {
     if constexpr (PAIR) {
       asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tbase)),

@@ -1065,34 +1065,36 @@ void launch_count_valid(const int32_t* labels, int N, int V, int* count, unsigne
   launch_pdl(count_valid_k, 1, 1024, 0, s, labels, N, V, count, err);
 }
 
-__global__ void loss_reduce_k(const float* __restrict__ rl, int N, const int* count, float* out) {
+// Per-thread sums, then warp and block sums by shuffles, in fp64 and a fixed order.
+__global__ void __launch_bounds__(1024) loss_reduce_k(const float* __restrict__ rl, int N, const int* count, float* out) {
   pdl_wait();
   pdl_trigger();
-  __shared__ double sh[1024];
+  __shared__ double sh[32];
   double acc = 0.0;
   for (int i0 = threadIdx.x; i0 < N; i0 += 4 * blockDim.x) {   // 4 loads in flight, added in index order
     float v[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) v[q] = i0 + q * (int)blockDim.x < N ? rl[i0 + q * blockDim.x] : 0.f;
+    acc += ((double)v[0] + (double)v[1]) + ((double)v[2] + (double)v[3]);
+  }
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if (i0 + q * (int)blockDim.x < N) acc += (double)v[q];
-  }
-  sh[threadIdx.x] = acc;
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
   __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    const int c = *count;
-    *out = c > 0 ? (float)(sh[0] / (double)c) : 0.f;
+  if (threadIdx.x < 32) {
+    acc = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (threadIdx.x == 0) {
+      const int c = *count;
+      *out = c > 0 ? (float)(acc / (double)c) : 0.f;
+    }
   }
 }
 
 void launch_loss_reduce(const float* row_loss, int N, const int* count, float* out, cudaStream_t s) {
   note_launch(1);
-  launch_pdl(loss_reduce_k, 1, 1024, 0, s, row_loss, N, count, out);
+  launch_pdl(loss_reduce_k, 1, N <= 1024 ? 256 : 1024, 0, s, row_loss, N, count, out);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1100,16 +1102,25 @@ void launch_loss_reduce(const float* row_loss, int N, const int* count, float* o
 // ------------------------------------------------------------------------------------------
 // Advances a chunk's optimizer step count t (device memory, so a replayed CUDA graph keeps counting)
 // and writes this step's learning rate and bias corrections: hp = {lr_t, 1 - beta1^t, 1 - beta2^t}.
+// The powers by repeated squaring, one lane each (at most 126 fp64 products, a few 1e-15 relative, far below the
+// fp32 they are rounded to): two fp64 pow() calls in one thread took 9 us on every chunk's chain, this about 3.
 __global__ void adamw_tick_k(long long* __restrict__ t, float* __restrict__ hp, float lr0, int schedule,
                              float gamma, float b1, float b2) {
   pdl_wait();
   pdl_trigger();
   const long long tt = *t + 1;
-  *t = tt;
-  const double lr = schedule == 1 ? (double)lr0 / sqrt((double)(tt - 1) + (double)gamma) : (double)lr0;
-  hp[0] = (float)lr;
-  hp[1] = (float)(1.0 - pow((double)b1, (double)tt));
-  hp[2] = (float)(1.0 - pow((double)b2, (double)tt));
+  __syncwarp();   // every lane has read the count
+  if (threadIdx.x == 0) {
+    *t = tt;
+    hp[0] = (float)(schedule == 1 ? (double)lr0 / sqrt((double)(tt - 1) + (double)gamma) : (double)lr0);
+  } else if (threadIdx.x <= 2) {
+    double b = (double)(threadIdx.x == 1 ? b1 : b2), p = 1.0;
+    for (long long e = tt; e > 0; e >>= 1) {
+      if (e & 1) p *= b;
+      b *= b;
+    }
+    hp[threadIdx.x] = (float)(1.0 - p);
+  }
 }
 
 __global__ void adamw_k(float4* __restrict__ th, float4* __restrict__ g, float4* __restrict__ m,
@@ -1135,7 +1146,7 @@ __global__ void adamw_k(float4* __restrict__ th, float4* __restrict__ g, float4*
 void launch_adamw_tick(long long* t, float* hp, float lr0, int schedule, float gamma, float b1, float b2,
                        cudaStream_t s) {
   note_launch(1);
-  launch_pdl(adamw_tick_k, 1, 1, 0, s, t, hp, lr0, schedule, gamma, b1, b2);
+  launch_pdl(adamw_tick_k, 1, 32, 0, s, t, hp, lr0, schedule, gamma, b1, b2);
 }
 
 void launch_adamw(float* theta, float* g, float* m, float* v, void* comp, size_t n, long long* t, float* hp,

@@ -235,6 +235,11 @@ __device__ __forceinline__ void mma_bf16_ta(uint32_t d, uint32_t a, uint64_t b, 
       "r"(a), "l"(b), "r"(id), "r"(acc));
 }
 
+// Brings a kernel parameter's tensor map into the descriptor cache, ahead of its first use.
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* m) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)m) : "memory");
+}
+
 // TMA 3-D tile load (coordinates innermost first).
 __device__ __forceinline__ void tma3d(void* dst, const CUtensorMap* m, uint64_t* bar, int c0, int c1, int c2) {
   asm volatile(
