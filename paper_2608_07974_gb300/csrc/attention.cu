@@ -4,6 +4,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "ops.h"
@@ -14,8 +15,12 @@ namespace {
 // ------------------------------------------------------------------------------------------------
 // CUDA-core kernels. A CTA works on 32 query (or key) rows of one head, LPR lanes per row (four; eight where a row
 // would not fit four lanes' registers): lane `sub` holds the head dims 4 (LPR c + sub) .. + 3 (HDP: hd rounded up
-// to 32, 64 or 128, zero padded). The other side comes in tiles of 32 rows through shared memory (read as 16-byte broadcasts), four
-// of its rows at a time, so that four dot products and their shuffle steps are in flight together.
+// to 32, 64 or 128, zero padded). The other side comes in tiles of 32 rows through shared memory (read as 16-byte
+// broadcasts), eight of its rows at a time (four in the backward), so that their dot products and shuffle steps are
+// in flight together. A tile's rows are loaded into registers during the tile before, 16 bytes a load, because on
+// small shapes the loads' latency is the kernel: with scalar loads between the barriers 4 x 64 tokens, 4 heads of
+// 32 took 9.2 us forward and 14.4 us backward, with these 5.7 and 10.1 (2 x 512 tokens, 16 heads of 64 over 4: 139
+// and 713, now 137 and 581: there shared-memory reads, one per four multiply-adds, are the bound).
 // One warp per row with one key at a time, which these replace, waited for five shuffles and a global load per
 // key: 4 x 64 tokens, 4 heads of 32 (the tiny fp32 workload) is bound by that chain, not by its 17 MFLOP.
 // ------------------------------------------------------------------------------------------------
@@ -29,26 +34,50 @@ struct RowV {
   float v[N];
 };
 
-// Rows r0 .. r0 + AR - 1 (below `rows`) of a [rows, ld] matrix, hd columns, into an [AR][HDP + 4] tile.
+// This lane's part of a row of hd columns; `vec`: fp32 rows that start on 16 bytes, hd a multiple of four. All of a
+// thread's loads are in flight together.
 template <typename T, int HDP>
-__device__ __forceinline__ void tile_rows(float* dst, const T* src, int ld, int r0, int rows, int hd) {
-  for (int e = threadIdx.x; e < AR * HDP / 2; e += AR * kLpr<HDP>) {   // pairs: hd is even
-    const int r = e / (HDP / 2), d = (e % (HDP / 2)) * 2;
-    const bool ok = r0 + r < rows && d < hd;
-    const T* p = src + (size_t)(ok ? r0 + r : 0) * ld + (ok ? d : 0);
-    dst[r * (HDP + 4) + d] = ok ? to_f(p[0]) : 0.f;
-    dst[r * (HDP + 4) + d + 1] = ok ? to_f(p[1]) : 0.f;
+__device__ __forceinline__ void load_row(RowV<HDP>& o, const T* p, int hd, int sub, bool ok, bool vec) {
+#pragma unroll
+  for (int c = 0; c < RowV<HDP>::NC; ++c) {
+    const int d = 4 * (RowV<HDP>::L * c + sub);
+    if constexpr (std::is_same<T, float>::value) {
+      if (vec) {
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (ok && d < hd) x = *reinterpret_cast<const float4*>(p + d);
+        o.v[4 * c] = x.x;
+        o.v[4 * c + 1] = x.y;
+        o.v[4 * c + 2] = x.z;
+        o.v[4 * c + 3] = x.w;
+        continue;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) o.v[4 * c + q] = ok && d + q < hd ? to_f(p[d + q]) : 0.f;
   }
 }
-template <typename T, int HDP>
-__device__ __forceinline__ void load_row(RowV<HDP>& o, const T* p, int hd, int sub, float scale, bool ok) {
+template <int HDP>
+__device__ __forceinline__ void scale_row(RowV<HDP>& o, float f) {
+#pragma unroll
+  for (int d = 0; d < RowV<HDP>::N; ++d) o.v[d] *= f;
+}
+// The row into an [AR][HDP + 4] tile.
+template <int HDP>
+__device__ __forceinline__ void put_row(float* tile, const RowV<HDP>& o, int row, int sub) {
 #pragma unroll
   for (int c = 0; c < RowV<HDP>::NC; ++c)
+    *reinterpret_cast<float4*>(tile + row * (HDP + 4) + 4 * (RowV<HDP>::L * c + sub)) =
+        make_float4(o.v[4 * c], o.v[4 * c + 1], o.v[4 * c + 2], o.v[4 * c + 3]);
+}
+// The dot product of two rows, in each of the row's lanes.
+template <int HDP>
+__device__ __forceinline__ float dot_rows(const RowV<HDP>& a, const RowV<HDP>& b) {
+  float x = 0.f;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int d = 4 * (RowV<HDP>::L * c + sub) + q;
-      o.v[4 * c + q] = ok && d < hd ? to_f(p[d]) * scale : 0.f;
-    }
+  for (int d = 0; d < RowV<HDP>::N; ++d) x = fmaf(a.v[d], b.v[d], x);
+#pragma unroll
+  for (int m = 1; m < RowV<HDP>::L; m *= 2) x += __shfl_xor_sync(0xffffffffu, x, m);
+  return x;
 }
 template <typename T, int HDP>
 __device__ __forceinline__ void store_row(T* p, const RowV<HDP>& o, int hd, int sub, float scale) {
@@ -60,11 +89,12 @@ __device__ __forceinline__ void store_row(T* p, const RowV<HDP>& o, int hd, int 
       if (d < hd) p[d] = from_f<T>(o.v[4 * c + q] * scale);
     }
 }
-// The row's dot products with tile rows j .. j + 3, in every one of its lanes.
-template <int HDP>
-__device__ __forceinline__ void dot4(float* s, const RowV<HDP>& a, const float* tile, int j, int sub) {
+constexpr int AF = 8, AB = 4;   // tile rows worked on at a time, forward and backward (eight spill there)
+// The row's dot products with tile rows j .. j + U - 1, in every one of its lanes.
+template <int HDP, int U>
+__device__ __forceinline__ void dot_tile(float* s, const RowV<HDP>& a, const float* tile, int j, int sub) {
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
+  for (int u = 0; u < U; ++u) {
     const float* t = tile + (j + u) * (HDP + 4) + 4 * sub;
     float x = 0.f;
 #pragma unroll
@@ -80,13 +110,13 @@ __device__ __forceinline__ void dot4(float* s, const RowV<HDP>& a, const float* 
 #pragma unroll
   for (int x = 1; x < RowV<HDP>::L; x *= 2)
 #pragma unroll
-    for (int u = 0; u < 4; ++u) s[u] += __shfl_xor_sync(0xffffffffu, s[u], x);
+    for (int u = 0; u < U; ++u) s[u] += __shfl_xor_sync(0xffffffffu, s[u], x);
 }
 // o += sum_u w[u] * tile row j + u
-template <int HDP>
-__device__ __forceinline__ void axpy4(RowV<HDP>& o, const float* w, const float* tile, int j, int sub) {
+template <int HDP, int U>
+__device__ __forceinline__ void axpy_tile(RowV<HDP>& o, const float* w, const float* tile, int j, int sub) {
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
+  for (int u = 0; u < U; ++u) {
     const float* t = tile + (j + u) * (HDP + 4) + 4 * sub;
 #pragma unroll
     for (int c = 0; c < RowV<HDP>::NC; ++c) {
@@ -101,39 +131,51 @@ __device__ __forceinline__ void axpy4(RowV<HDP>& o, const float* w, const float*
 
 template <typename T, int HDP>
 __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_fwd_k(const T* __restrict__ qkv, T* __restrict__ out, float* __restrict__ lse,
-                                                  int S, int H, int Hkv, int hd, float scale, int nt) {
+                                                  int S, int H, int Hkv, int hd, float scale, int nt, bool vec) {
   __shared__ __align__(16) float ks[AR * (HDP + 4)], vs[AR * (HDP + 4)];
   pdl_wait();
   pdl_trigger();
   const int h = blockIdx.x / nt, b = blockIdx.y, i0 = (nt - 1 - (int)blockIdx.x % nt) * AR;   // long rows first
-  const int ld = (H + 2 * Hkv) * hd, kvh = h / (H / Hkv), sub = threadIdx.x % kLpr<HDP>, i = i0 + threadIdx.x / kLpr<HDP>;
+  const int ld = (H + 2 * Hkv) * hd, kvh = h / (H / Hkv), sub = threadIdx.x % kLpr<HDP>, row = threadIdx.x / kLpr<HDP>, i = i0 + row;
   const T* base = qkv + (size_t)b * S * ld;
-  RowV<HDP> q, o;
-  load_row<T, HDP>(q, base + (size_t)min(i, S - 1) * ld + h * hd, hd, sub, scale, i < S);
+  RowV<HDP> q, o, kn, vn;   // kn, vn: this thread's part of the next tile's rows, loaded during the tile before
+  auto fetch = [&](int j) {
+    const T* p = base + (size_t)min(j + row, S - 1) * ld + (H + kvh) * hd;
+    load_row<T, HDP>(kn, p, hd, sub, j + row < S, vec);
+    load_row<T, HDP>(vn, p + Hkv * hd, hd, sub, j + row < S, vec);
+  };
+  load_row<T, HDP>(q, base + (size_t)min(i, S - 1) * ld + h * hd, hd, sub, i < S, vec);
+  fetch(0);
+  scale_row<HDP>(q, scale);
 #pragma unroll
   for (int d = 0; d < RowV<HDP>::N; ++d) o.v[d] = 0.f;
   float m = -INFINITY, l = 0.f;
   for (int j0 = 0; j0 <= i0; j0 += AR) {
     __syncthreads();
-    tile_rows<T, HDP>(ks, base + (H + kvh) * hd, ld, j0, S, hd);
-    tile_rows<T, HDP>(vs, base + (H + Hkv + kvh) * hd, ld, j0, S, hd);
+    put_row<HDP>(ks, kn, row, sub);
+    put_row<HDP>(vs, vn, row, sub);
     __syncthreads();
+    if (j0 + AR <= i0) fetch(j0 + AR);
 #pragma unroll 1
-    for (int j = 0; j < AR; j += 4) {
-      float s[4];
-      dot4<HDP>(s, q, ks, j, sub);
+    for (int j = 0; j < AR; j += AF) {
+      float s[AF];
+      dot_tile<HDP, AF>(s, q, ks, j, sub);
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+      for (int u = 0; u < AF; ++u)
         if (j0 + j + u > i) s[u] = -INFINITY;
-      const float mn = fmaxf(m, fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3])));
+      float mn = m;
+#pragma unroll
+      for (int u = 0; u < AF; ++u) mn = fmaxf(mn, s[u]);
       if (mn > -INFINITY) {   // (past the row's last key a warp still runs for its other rows)
         const float corr = expf(m - mn);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) s[u] = expf(s[u] - mn);
-        l = l * corr + ((s[0] + s[1]) + (s[2] + s[3]));
+        for (int u = 0; u < AF; ++u) s[u] = expf(s[u] - mn);
+        float ls = 0.f;
 #pragma unroll
-        for (int d = 0; d < RowV<HDP>::N; ++d) o.v[d] *= corr;
-        axpy4<HDP>(o, s, vs, j, sub);
+        for (int u = 0; u < AF; u += 2) ls += s[u] + s[u + 1];
+        l = l * corr + ls;
+        scale_row<HDP>(o, corr);
+        axpy_tile<HDP, AF>(o, s, vs, j, sub);
         m = mn;
       }
     }
@@ -149,7 +191,7 @@ template <typename T, int HDP>
 __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_bwd_k(const T* __restrict__ qkv, const T* __restrict__ out,
                                                   const T* __restrict__ dout, const float* __restrict__ lse,
                                                   T* __restrict__ dqkv, int S, int H, int Hkv, int hd, float scale,
-                                                  int nt) {
+                                                  int nt, bool vec) {
   __shared__ __align__(16) float ta[AR * (HDP + 4)], tb[AR * (HDP + 4)];
   __shared__ float sl[AR], sd[AR];
   pdl_wait();
@@ -158,36 +200,38 @@ __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_bwd_k(const T* __restrict
   const int y = blockIdx.x / (2 * nt), x = blockIdx.x % (2 * nt);
   const int ld = (H + 2 * Hkv) * hd, lo = H * hd, rep = H / Hkv;
   const T* base = qkv + (size_t)b * S * ld;
-  auto row_d = [&](int h, int i) {   // D of query i, in each of its lanes
-    const size_t o = (size_t)(b * S + min(i, S - 1)) * lo + h * hd;
-    float d2 = 0.f;
-#pragma unroll 4
-    for (int d = sub; d < hd; d += kLpr<HDP>) d2 = fmaf(to_f(out[o + d]), to_f(dout[o + d]), d2);
-#pragma unroll
-    for (int m = 1; m < kLpr<HDP>; m *= 2) d2 += __shfl_xor_sync(0xffffffffu, d2, m);
-    return d2;
-  };
   if (x < nt) {
     const int h = y, kvh = h / rep, i0 = (nt - 1 - x) * AR, i = i0 + row;
-    RowV<HDP> q, g, dq;
-    load_row<T, HDP>(q, base + (size_t)min(i, S - 1) * ld + h * hd, hd, sub, scale, i < S);
-    load_row<T, HDP>(g, dout + (size_t)(b * S + min(i, S - 1)) * lo + h * hd, hd, sub, 1.f, i < S);
+    RowV<HDP> q, g, dq, kn, vn;   // kn, vn: the next tile's rows
+    auto fetch = [&](int j) {
+      const T* p = base + (size_t)min(j + row, S - 1) * ld + (H + kvh) * hd;
+      load_row<T, HDP>(kn, p, hd, sub, j + row < S, vec);
+      load_row<T, HDP>(vn, p + Hkv * hd, hd, sub, j + row < S, vec);
+    };
+    const size_t io = (size_t)(b * S + min(i, S - 1)) * lo + h * hd;
+    load_row<T, HDP>(q, base + (size_t)min(i, S - 1) * ld + h * hd, hd, sub, i < S, vec);
+    load_row<T, HDP>(g, dout + io, hd, sub, i < S, vec);
+    load_row<T, HDP>(dq, out + io, hd, sub, i < S, vec);
+    const float L = lse[((size_t)b * H + h) * S + min(i, S - 1)];
+    fetch(0);
+    scale_row<HDP>(q, scale);
+    const float D = dot_rows<HDP>(dq, g);
 #pragma unroll
     for (int d = 0; d < RowV<HDP>::N; ++d) dq.v[d] = 0.f;
-    const float D = row_d(h, i), L = lse[((size_t)b * H + h) * S + min(i, S - 1)];
     for (int j0 = 0; j0 <= i0; j0 += AR) {
       __syncthreads();
-      tile_rows<T, HDP>(ta, base + (H + kvh) * hd, ld, j0, S, hd);
-      tile_rows<T, HDP>(tb, base + (H + Hkv + kvh) * hd, ld, j0, S, hd);
+      put_row<HDP>(ta, kn, row, sub);
+      put_row<HDP>(tb, vn, row, sub);
       __syncthreads();
+      if (j0 + AR <= i0) fetch(j0 + AR);
 #pragma unroll 1
-      for (int j = 0; j < AR; j += 4) {
-        float s[4], dp[4];
-        dot4<HDP>(s, q, ta, j, sub);
-        dot4<HDP>(dp, g, tb, j, sub);
+      for (int j = 0; j < AR; j += AB) {
+        float s[AB], dp[AB];
+        dot_tile<HDP, AB>(s, q, ta, j, sub);
+        dot_tile<HDP, AB>(dp, g, tb, j, sub);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) s[u] = j0 + j + u <= i ? expf(s[u] - L) * (dp[u] - D) : 0.f;
-        axpy4<HDP>(dq, s, ta, j, sub);
+        for (int u = 0; u < AB; ++u) s[u] = j0 + j + u <= i ? expf(s[u] - L) * (dp[u] - D) : 0.f;
+        axpy_tile<HDP, AB>(dq, s, ta, j, sub);
       }
     }
     if (i < S) store_row<T, HDP>(dqkv + (size_t)(b * S + i) * ld + h * hd, dq, hd, sub, scale);
@@ -195,35 +239,48 @@ __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_bwd_k(const T* __restrict
   }
   if (y >= Hkv) return;
   const int kvh = y, j0 = (x - nt) * AR, j = j0 + row;
-  RowV<HDP> k, v, dk, dv;
-  load_row<T, HDP>(k, base + (size_t)min(j, S - 1) * ld + (H + kvh) * hd, hd, sub, scale, j < S);
-  load_row<T, HDP>(v, base + (size_t)min(j, S - 1) * ld + (H + Hkv + kvh) * hd, hd, sub, 1.f, j < S);
+  RowV<HDP> k, v, dk, dv, qn, gn, on;   // qn, gn, on, ln: the next tile's query, dO and O rows and log-sum-exp
+  float ln;
+  auto fetch = [&](int h, int i) {
+    const bool ok = i + row < S;
+    const size_t n = (size_t)min(i + row, S - 1);
+    load_row<T, HDP>(qn, base + n * ld + h * hd, hd, sub, ok, vec);
+    load_row<T, HDP>(gn, dout + ((size_t)b * S + n) * lo + h * hd, hd, sub, ok, vec);
+    load_row<T, HDP>(on, out + ((size_t)b * S + n) * lo + h * hd, hd, sub, ok, vec);
+    ln = ok ? lse[((size_t)b * H + h) * S + n] : INFINITY;
+  };
+  load_row<T, HDP>(k, base + (size_t)min(j, S - 1) * ld + (H + kvh) * hd, hd, sub, j < S, vec);
+  load_row<T, HDP>(v, base + (size_t)min(j, S - 1) * ld + (H + Hkv + kvh) * hd, hd, sub, j < S, vec);
+  fetch(kvh * rep, j0);
+  scale_row<HDP>(k, scale);
 #pragma unroll
   for (int d = 0; d < RowV<HDP>::N; ++d) dk.v[d] = dv.v[d] = 0.f;
   for (int hh = 0; hh < rep; ++hh) {
     const int h = kvh * rep + hh;
     for (int i0 = j0; i0 < S; i0 += AR) {
       __syncthreads();
-      tile_rows<T, HDP>(ta, base + h * hd, ld, i0, S, hd);
-      tile_rows<T, HDP>(tb, dout + (size_t)b * S * lo + h * hd, lo, i0, S, hd);
-      const float D = row_d(h, i0 + row);
+      put_row<HDP>(ta, qn, row, sub);
+      put_row<HDP>(tb, gn, row, sub);
+      const float D = dot_rows<HDP>(on, gn);
       if (sub == 0) {
         sd[row] = D;
-        sl[row] = i0 + row < S ? lse[((size_t)b * H + h) * S + i0 + row] : INFINITY;
+        sl[row] = ln;
       }
       __syncthreads();
+      if (i0 + AR < S) fetch(h, i0 + AR);
+      else if (hh + 1 < rep) fetch(h + 1, j0);
 #pragma unroll 1
-      for (int i = 0; i < AR; i += 4) {
-        float s[4], dp[4];
-        dot4<HDP>(s, k, ta, i, sub);
-        dot4<HDP>(dp, v, tb, i, sub);
+      for (int i = 0; i < AR; i += AB) {
+        float s[AB], dp[AB];
+        dot_tile<HDP, AB>(s, k, ta, i, sub);
+        dot_tile<HDP, AB>(dp, v, tb, i, sub);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < AB; ++u) {
           s[u] = i0 + i + u >= j ? expf(s[u] - sl[i + u]) : 0.f;
           dp[u] = s[u] * (dp[u] - sd[i + u]);
         }
-        axpy4<HDP>(dv, s, tb, i, sub);
-        axpy4<HDP>(dk, dp, ta, i, sub);
+        axpy_tile<HDP, AB>(dv, s, tb, i, sub);
+        axpy_tile<HDP, AB>(dk, dp, ta, i, sub);
       }
     }
   }
@@ -237,15 +294,18 @@ template <typename T, int HDP>
 void cuda_core_fwd(const void* qkv, void* out, float* lse, int B, int S, int H, int Hkv, int hd, float scale,
                    cudaStream_t s) {
   const int nt = (S + AR - 1) / AR;
+  const bool vec = std::is_same<T, float>::value && hd % 4 == 0 && ((uintptr_t)qkv & 15u) == 0;
   launch_pdl(attn_fwd_k<T, HDP>, dim3((unsigned)H * nt, B), AR * kLpr<HDP>, 0, s, (const T*)qkv, (T*)out, lse, S, H, Hkv, hd, scale,
-             nt);
+             nt, vec);
 }
 template <typename T, int HDP>
 void cuda_core_bwd(const void* qkv, const void* out, const void* dout, const float* lse, void* dqkv, int B, int S, int H,
                    int Hkv, int hd, float scale, cudaStream_t s) {
   const int nt = (S + AR - 1) / AR;
+  const bool vec = std::is_same<T, float>::value && hd % 4 == 0 &&
+                   (((uintptr_t)qkv | (uintptr_t)out | (uintptr_t)dout) & 15u) == 0;
   launch_pdl(attn_bwd_k<T, HDP>, dim3((unsigned)H * 2 * nt, B), AR * kLpr<HDP>, 0, s, (const T*)qkv, (const T*)out, (const T*)dout, lse,
-             (T*)dqkv, S, H, Hkv, hd, scale, nt);
+             (T*)dqkv, S, H, Hkv, hd, scale, nt, vec);
 }
 
 // Head padding for the tcgen05 kernels (head dims 64 and 128): dst [N, nh * hp] from src [N, nh * hd] with

@@ -58,3 +58,24 @@ def test_fp32_attention(B, Bb, S, H, Hkv, hd):
     assert float((lse - torch.logsumexp(s, -1).detach()).abs().max()) <= 1e-5
     assert float((out - ref.detach()).abs().max()) <= 1e-5 * max(1.0, float(ref.detach().abs().max()))
     assert float((dqkv - gx).abs().max()) <= 1e-5 * max(1.0, float(gx.abs().max()))
+
+
+# Rows off 16 bytes take single loads, the others 16-byte ones: the same values in the same order.
+@pytest.mark.parametrize("S,H,Hkv,hd", [(65, 4, 2, 32), (40, 2, 2, 64)])
+def test_fp32_attention_alignment(B, S, H, Hkv, hd):
+    g = torch.Generator(device="cuda").manual_seed(S)
+    W = (H + 2 * Hkv) * hd
+    qkv, dout = torch.randn(S, W, device="cuda", generator=g), torch.randn(S, H * hd, device="cuda", generator=g)
+    res = []
+    for off in (0, 1):
+        def at(t):
+            b = torch.empty(t.numel() + off, device="cuda")
+            b[off:].copy_(t.flatten())
+            return b[off:].view(t.shape)
+        q, d, lse = at(qkv), at(dout), torch.empty(1, H, S, device="cuda")
+        out, dqkv = at(dout), at(qkv)
+        B.zl_op_attention(0, q, out, lse, 1, S, H, Hkv, hd)
+        B.zl_op_attention_bwd(0, q, out, d, lse, dqkv, 1, S, H, Hkv, hd)
+        res.append((out.clone(), lse, dqkv.clone()))
+    for a, b in zip(*res):
+        assert torch.equal(a, b)
