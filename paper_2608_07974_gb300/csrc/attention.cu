@@ -61,6 +61,31 @@ __device__ __forceinline__ void scale_row(RowV<HDP>& o, float f) {
 #pragma unroll
   for (int d = 0; d < RowV<HDP>::N; ++d) o.v[d] *= f;
 }
+// Rotate-half RoPE of a row of HDP columns (hd = HDP), whose pairs (d, d + HDP / 2) lie in one lane: this lane's part
+// of the position's (cos, sin) pairs, and the rotation as the separate pass rounds it (sg = -1: the inverse).
+template <int HDP>
+struct RopeV {
+  float4 v[RowV<HDP>::NC];   // chunk c: pairs 4 (L c + sub) .. + 3
+};
+template <int HDP>
+__device__ __forceinline__ void load_rope(RopeV<HDP>& t, const float2* cs, int pos, int sub) {
+#pragma unroll
+  for (int c = 0; c < RowV<HDP>::NC / 2; ++c) {
+    const float4* p = reinterpret_cast<const float4*>(cs + (size_t)pos * (HDP / 2) + 4 * (RowV<HDP>::L * c + sub));
+    t.v[2 * c] = p[0];
+    t.v[2 * c + 1] = p[1];
+  }
+}
+template <int HDP>
+__device__ __forceinline__ void rotate_row(RowV<HDP>& o, const RopeV<HDP>& t, float sg) {
+  constexpr int HN = RowV<HDP>::N / 2;
+#pragma unroll
+  for (int d = 0; d < HN; ++d) {
+    const float4 p = t.v[d / 2];
+    const float a = o.v[d], b = o.v[d + HN];
+    rope_rot(a, b, d & 1 ? p.z : p.x, sg * (d & 1 ? p.w : p.y), o.v[d], o.v[d + HN]);
+  }
+}
 // The row into an [AR][HDP + 4] tile.
 template <int HDP>
 __device__ __forceinline__ void put_row(float* tile, const RowV<HDP>& o, int row, int sub) {
@@ -129,9 +154,9 @@ __device__ __forceinline__ void axpy_tile(RowV<HDP>& o, const float* w, const fl
   }
 }
 
-template <typename T, int HDP>
+template <typename T, int HDP, bool ROPE>
 __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_fwd_k(const T* __restrict__ qkv, T* __restrict__ out, float* __restrict__ lse,
-                                                  int S, int H, int Hkv, int hd, float scale, int nt, bool vec) {
+                                                  int S, int H, int Hkv, int hd, float scale, int nt, bool vec, const float2* __restrict__ cs) {
   __shared__ __align__(16) float ks[AR * (HDP + 4)], vs[AR * (HDP + 4)];
   pdl_wait();
   pdl_trigger();
@@ -139,19 +164,24 @@ __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_fwd_k(const T* __restrict
   const int ld = (H + 2 * Hkv) * hd, kvh = h / (H / Hkv), sub = threadIdx.x % kLpr<HDP>, row = threadIdx.x / kLpr<HDP>, i = i0 + row;
   const T* base = qkv + (size_t)b * S * ld;
   RowV<HDP> q, o, kn, vn;   // kn, vn: this thread's part of the next tile's rows, loaded during the tile before
+  RopeV<HDP> tq, tn;        // and their rotations
   auto fetch = [&](int j) {
     const T* p = base + (size_t)min(j + row, S - 1) * ld + (H + kvh) * hd;
     load_row<T, HDP>(kn, p, hd, sub, j + row < S, vec);
     load_row<T, HDP>(vn, p + Hkv * hd, hd, sub, j + row < S, vec);
+    if (ROPE) load_rope<HDP>(tn, cs, min(j + row, S - 1), sub);
   };
   load_row<T, HDP>(q, base + (size_t)min(i, S - 1) * ld + h * hd, hd, sub, i < S, vec);
+  if (ROPE) load_rope<HDP>(tq, cs, min(i, S - 1), sub);
   fetch(0);
+  if (ROPE) rotate_row<HDP>(q, tq, 1.f);
   scale_row<HDP>(q, scale);
 #pragma unroll
   for (int d = 0; d < RowV<HDP>::N; ++d) o.v[d] = 0.f;
   float m = -INFINITY, l = 0.f;
   for (int j0 = 0; j0 <= i0; j0 += AR) {
     __syncthreads();
+    if (ROPE) rotate_row<HDP>(kn, tn, 1.f);
     put_row<HDP>(ks, kn, row, sub);
     put_row<HDP>(vs, vn, row, sub);
     __syncthreads();
@@ -187,11 +217,11 @@ __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_fwd_k(const T* __restrict
 
 // Of head y's 2 nt blocks the first nt form dQ of 32 queries each, the others (y < Hkv) dK and dV of 32 keys of KV
 // head y, summed over its query heads in order. D = rowsum(dO * O) is formed wherever a row needs it.
-template <typename T, int HDP>
+template <typename T, int HDP, bool ROPE>
 __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_bwd_k(const T* __restrict__ qkv, const T* __restrict__ out,
                                                   const T* __restrict__ dout, const float* __restrict__ lse,
                                                   T* __restrict__ dqkv, int S, int H, int Hkv, int hd, float scale,
-                                                  int nt, bool vec) {
+                                                  int nt, bool vec, const float2* __restrict__ cs) {
   __shared__ __align__(16) float ta[AR * (HDP + 4)], tb[AR * (HDP + 4)];
   __shared__ float sl[AR], sd[AR];
   pdl_wait();
@@ -203,23 +233,28 @@ __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_bwd_k(const T* __restrict
   if (x < nt) {
     const int h = y, kvh = h / rep, i0 = (nt - 1 - x) * AR, i = i0 + row;
     RowV<HDP> q, g, dq, kn, vn;   // kn, vn: the next tile's rows
+    RopeV<HDP> tq, tn;
     auto fetch = [&](int j) {
       const T* p = base + (size_t)min(j + row, S - 1) * ld + (H + kvh) * hd;
       load_row<T, HDP>(kn, p, hd, sub, j + row < S, vec);
       load_row<T, HDP>(vn, p + Hkv * hd, hd, sub, j + row < S, vec);
+      if (ROPE) load_rope<HDP>(tn, cs, min(j + row, S - 1), sub);
     };
     const size_t io = (size_t)(b * S + min(i, S - 1)) * lo + h * hd;
     load_row<T, HDP>(q, base + (size_t)min(i, S - 1) * ld + h * hd, hd, sub, i < S, vec);
     load_row<T, HDP>(g, dout + io, hd, sub, i < S, vec);
     load_row<T, HDP>(dq, out + io, hd, sub, i < S, vec);
     const float L = lse[((size_t)b * H + h) * S + min(i, S - 1)];
+    if (ROPE) load_rope<HDP>(tq, cs, min(i, S - 1), sub);
     fetch(0);
+    if (ROPE) rotate_row<HDP>(q, tq, 1.f);
     scale_row<HDP>(q, scale);
     const float D = dot_rows<HDP>(dq, g);
 #pragma unroll
     for (int d = 0; d < RowV<HDP>::N; ++d) dq.v[d] = 0.f;
     for (int j0 = 0; j0 <= i0; j0 += AR) {
       __syncthreads();
+      if (ROPE) rotate_row<HDP>(kn, tn, 1.f);
       put_row<HDP>(ta, kn, row, sub);
       put_row<HDP>(tb, vn, row, sub);
       __syncthreads();
@@ -234,12 +269,15 @@ __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_bwd_k(const T* __restrict
         axpy_tile<HDP, AB>(dq, s, ta, j, sub);
       }
     }
-    if (i < S) store_row<T, HDP>(dqkv + (size_t)(b * S + i) * ld + h * hd, dq, hd, sub, scale);
+    scale_row<HDP>(dq, scale);
+    if (ROPE) rotate_row<HDP>(dq, tq, -1.f);
+    if (i < S) store_row<T, HDP>(dqkv + (size_t)(b * S + i) * ld + h * hd, dq, hd, sub, 1.f);
     return;
   }
   if (y >= Hkv) return;
   const int kvh = y, j0 = (x - nt) * AR, j = j0 + row;
   RowV<HDP> k, v, dk, dv, qn, gn, on;   // qn, gn, on, ln: the next tile's query, dO and O rows and log-sum-exp
+  RopeV<HDP> tk, tn;
   float ln;
   auto fetch = [&](int h, int i) {
     const bool ok = i + row < S;
@@ -248,10 +286,13 @@ __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_bwd_k(const T* __restrict
     load_row<T, HDP>(gn, dout + ((size_t)b * S + n) * lo + h * hd, hd, sub, ok, vec);
     load_row<T, HDP>(on, out + ((size_t)b * S + n) * lo + h * hd, hd, sub, ok, vec);
     ln = ok ? lse[((size_t)b * H + h) * S + n] : INFINITY;
+    if (ROPE) load_rope<HDP>(tn, cs, (int)n, sub);
   };
   load_row<T, HDP>(k, base + (size_t)min(j, S - 1) * ld + (H + kvh) * hd, hd, sub, j < S, vec);
   load_row<T, HDP>(v, base + (size_t)min(j, S - 1) * ld + (H + Hkv + kvh) * hd, hd, sub, j < S, vec);
+  if (ROPE) load_rope<HDP>(tk, cs, min(j, S - 1), sub);
   fetch(kvh * rep, j0);
+  if (ROPE) rotate_row<HDP>(k, tk, 1.f);
   scale_row<HDP>(k, scale);
 #pragma unroll
   for (int d = 0; d < RowV<HDP>::N; ++d) dk.v[d] = dv.v[d] = 0.f;
@@ -259,6 +300,7 @@ __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_bwd_k(const T* __restrict
     const int h = kvh * rep + hh;
     for (int i0 = j0; i0 < S; i0 += AR) {
       __syncthreads();
+      if (ROPE) rotate_row<HDP>(qn, tn, 1.f);
       put_row<HDP>(ta, qn, row, sub);
       put_row<HDP>(tb, gn, row, sub);
       const float D = dot_rows<HDP>(on, gn);
@@ -284,28 +326,30 @@ __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_bwd_k(const T* __restrict
       }
     }
   }
+  scale_row<HDP>(dk, scale);
+  if (ROPE) rotate_row<HDP>(dk, tk, -1.f);
   if (j < S) {
-    store_row<T, HDP>(dqkv + (size_t)(b * S + j) * ld + (H + kvh) * hd, dk, hd, sub, scale);
+    store_row<T, HDP>(dqkv + (size_t)(b * S + j) * ld + (H + kvh) * hd, dk, hd, sub, 1.f);
     store_row<T, HDP>(dqkv + (size_t)(b * S + j) * ld + (H + Hkv + kvh) * hd, dv, hd, sub, 1.f);
   }
 }
 
-template <typename T, int HDP>
+template <typename T, int HDP, bool ROPE = false>
 void cuda_core_fwd(const void* qkv, void* out, float* lse, int B, int S, int H, int Hkv, int hd, float scale,
-                   cudaStream_t s) {
+                   cudaStream_t s, const float* cs = nullptr) {
   const int nt = (S + AR - 1) / AR;
   const bool vec = std::is_same<T, float>::value && hd % 4 == 0 && ((uintptr_t)qkv & 15u) == 0;
-  launch_pdl(attn_fwd_k<T, HDP>, dim3((unsigned)H * nt, B), AR * kLpr<HDP>, 0, s, (const T*)qkv, (T*)out, lse, S, H, Hkv, hd, scale,
-             nt, vec);
+  launch_pdl(attn_fwd_k<T, HDP, ROPE>, dim3((unsigned)H * nt, B), AR * kLpr<HDP>, 0, s, (const T*)qkv, (T*)out, lse, S, H,
+             Hkv, hd, scale, nt, vec, (const float2*)cs);
 }
-template <typename T, int HDP>
+template <typename T, int HDP, bool ROPE = false>
 void cuda_core_bwd(const void* qkv, const void* out, const void* dout, const float* lse, void* dqkv, int B, int S, int H,
-                   int Hkv, int hd, float scale, cudaStream_t s) {
+                   int Hkv, int hd, float scale, cudaStream_t s, const float* cs = nullptr) {
   const int nt = (S + AR - 1) / AR;
   const bool vec = std::is_same<T, float>::value && hd % 4 == 0 &&
                    (((uintptr_t)qkv | (uintptr_t)out | (uintptr_t)dout) & 15u) == 0;
-  launch_pdl(attn_bwd_k<T, HDP>, dim3((unsigned)H * 2 * nt, B), AR * kLpr<HDP>, 0, s, (const T*)qkv, (const T*)out, (const T*)dout, lse,
-             (T*)dqkv, S, H, Hkv, hd, scale, nt, vec);
+  launch_pdl(attn_bwd_k<T, HDP, ROPE>, dim3((unsigned)H * 2 * nt, B), AR * kLpr<HDP>, 0, s, (const T*)qkv, (const T*)out,
+             (const T*)dout, lse, (T*)dqkv, S, H, Hkv, hd, scale, nt, vec, (const float2*)cs);
 }
 
 // Head padding for the tcgen05 kernels (head dims 64 and 128): dst [N, nh * hp] from src [N, nh * hd] with
@@ -407,9 +451,19 @@ bool attn_bwd_padded(const void* qkv, const void* out, const void* dout, const f
 }
 }  // namespace
 
+// A rotation pass of its own is a launch forward and one backward per layer, all latency on small shapes (eight steps
+// of the tiny fp32 model: 3920 us with the passes, 3810 without). Heads of 64 and 128 keep the pass: the table beside
+// two rows' registers spills in the backward, 330 bytes.
+bool attn_rotates(int dt, int hd) { return dt != BF16 && hd == 32; }
+
 void attn_fwd(int dt, const void* qkv, void* out, float* lse, int B, int S, int H, int Hkv, int hd, cudaStream_t s,
-              unsigned* err, cudaMemPool_t pool) {
+              unsigned* err, cudaMemPool_t pool, const float* cs) {
   const float scale = 1.f / sqrtf((float)hd);
+  if (cs) {
+    note_launch(1);
+    cuda_core_fwd<float, 32, true>(qkv, out, lse, B, S, H, Hkv, hd, scale, s, cs);
+    return;
+  }
   if (dt == BF16 && attn_fwd_tcgen05(qkv, out, lse, B, S, H, Hkv, hd, s, err, scale)) return;
   if (dt == BF16 && attn_fwd_padded(qkv, out, lse, B, S, H, Hkv, hd, s, err, pool)) return;
   note_launch(1);
@@ -423,9 +477,13 @@ void attn_fwd(int dt, const void* qkv, void* out, float* lse, int B, int S, int 
 }
 
 void attn_bwd(int dt, const void* qkv, const void* out, const void* dout, const float* lse, float* Dbuf, void* dqkv,
-              int B, int S, int H, int Hkv, int hd, cudaStream_t s, cudaMemPool_t pool, unsigned* err) {
+              int B, int S, int H, int Hkv, int hd, cudaStream_t s, cudaMemPool_t pool, unsigned* err, const float* cs) {
   note_launch(dt == BF16 ? (H > Hkv ? 3 : 2) : 1);
   const float scale = 1.f / sqrtf((float)hd);
+  if (cs) {
+    cuda_core_bwd<float, 32, true>(qkv, out, dout, lse, dqkv, B, S, H, Hkv, hd, scale, s, cs);
+    return;
+  }
   if (dt == BF16 && attn_bwd_tcgen05(qkv, out, dout, lse, Dbuf, dqkv, B, S, H, Hkv, hd, s, pool, err, scale)) return;
   if (dt == BF16 && attn_bwd_padded(qkv, out, dout, lse, Dbuf, dqkv, B, S, H, Hkv, hd, s, pool, err)) return;
   if (dt == BF16 && attn_bwd_tc(qkv, out, dout, lse, Dbuf, dqkv, B, S, H, Hkv, hd, s, pool)) return;

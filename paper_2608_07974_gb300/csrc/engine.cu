@@ -378,16 +378,18 @@ void GW(zl_ctx* c, cudaStream_t s, Chunk& k, int li, PK p, int M, int N, int K, 
   pfree(tmp, s);
 }
 
+// The rotation table where the attention kernels rotate queries and keys (the saved qkv is then unrotated).
+const float* attn_rope(const zl_ctx* c) { return c->llama && attn_rotates(c->dt, c->hd) ? c->rope_cs : nullptr; }
 void AF(zl_ctx* c, cudaStream_t s, const void* qkv, void* out, float* lse, int B, int S) {
   const double e = (double)esz(c), N = (double)B * S;
   ProfScope p(c, s, PC_ATTN_F, 2.0 * B * c->H * (double)S * S * c->hd, e * N * (c->qkvw + c->ad));
-  attn_fwd(c->dt, qkv, out, lse, B, S, c->H, c->Hkv, c->hd, s, c->d_err, c->pool);
+  attn_fwd(c->dt, qkv, out, lse, B, S, c->H, c->Hkv, c->hd, s, c->d_err, c->pool, attn_rope(c));
 }
 void AB(zl_ctx* c, cudaStream_t s, const void* qkv, const void* out, const void* dout, const float* lse, float* D,
         void* dqkv, int B, int S) {
   const double e = (double)esz(c), N = (double)B * S;
   ProfScope p(c, s, PC_ATTN_B, 4.0 * B * c->H * (double)S * S * c->hd, e * N * (2.0 * c->qkvw + 2.0 * c->ad), 3);
-  attn_bwd(c->dt, qkv, out, dout, lse, D, dqkv, B, S, c->H, c->Hkv, c->hd, s, c->pool, c->d_err);
+  attn_bwd(c->dt, qkv, out, dout, lse, D, dqkv, B, S, c->H, c->Hkv, c->hd, s, c->pool, c->d_err, attn_rope(c));
 }
 void NF(zl_ctx* c, cudaStream_t s, const void* x, const float* g, const float* b, void* y, float* rstd, float* mean,
         int N) {
@@ -504,8 +506,8 @@ void layer_fwd(zl_ctx* c, Chunk& k, int li, LayerSave& sv, const void* x, void* 
   const int N = B * S, dt = c->dt;
   sv.x = x;
   NF(c, s, x, Wm(k, li, P_N1W), Wm(k, li, P_N1B), sv.xn1, sv.rstd1, sv.mean1, N);
-  // Llama: RoPE in the QKV product's epilogue (after the LoRA term, which is part of the product); otherwise a RoPE
-  // pass after the product
+  // Llama: RoPE in the QKV product's epilogue (bf16; after the LoRA term, which is part of the product) or as the
+  // attention kernels load queries and keys (fp32); otherwise a RoPE pass after the product
   bool rotated = false;
   if (c->llama && dt == BF16) {
     const int r16 = lora_r16(c->cfg.lora_rank);
@@ -522,7 +524,7 @@ void layer_fwd(zl_ctx* c, Chunk& k, int li, LayerSave& sv, const void* x, void* 
   }
   if (!rotated) {
     linear_fwd(c, k, li, 0, sv.xn1, sv.qkv, Wm(k, li, P_BQKV), nullptr, sv.u[0], N, s);
-    if (c->llama) {
+    if (c->llama && !attn_rope(c)) {
       ProfScope p(c, s, PC_ELEM, 0, 2.0 * esz(c) * (double)N * (c->H + c->Hkv) * c->hd);
       launch_rope(dt, sv.qkv, c->rope_cs, N, S, c->H, c->Hkv, c->hd, 0, s);
     }
@@ -657,7 +659,7 @@ void layer_bwd(zl_ctx* c, Chunk& k, int li, LayerSave& sv, const void* dy, void*
   GW(c, s, k, li, P_WO, c->d, c->ad, N, w.dx2, sv.att);
   bias_grad(c, w.dx2, N, c->d, Gm(k, li, P_BO), w, q);
   AB(c, s, sv.qkv, sv.att, w.datt, sv.lse, w.D, w.dqkv, B, S);
-  if (c->llama) {
+  if (c->llama && !attn_rope(c)) {
     ProfScope p(c, s, PC_ELEM, 0, 2.0 * esz(c) * (double)N * (c->H + c->Hkv) * c->hd);
     launch_rope(dt, w.dqkv, c->rope_cs, N, S, c->H, c->Hkv, c->hd, 1, s);
   }

@@ -154,13 +154,17 @@ void gemm_simt(int dt, int mode, int M, int N, int K, const void* A, const void*
 // where the copies come from, NULL = the device's default pool), mma.sync if they cannot be had; fp32:
 // CUDA cores.
 void attn_fwd(int dt, const void* qkv, void* out, float* lse, int B, int S, int H, int Hkv, int hd,
-              cudaStream_t s, unsigned* err = nullptr, cudaMemPool_t pool = nullptr);
+              cudaStream_t s, unsigned* err = nullptr, cudaMemPool_t pool = nullptr, const float* cs = nullptr);
+// Whether attn_fwd and attn_bwd can rotate (rotate-half RoPE, (cos, sin) table cs [S, hd / 2]) queries and keys
+// themselves: given cs they take qkv unrotated and return dqkv of the unrotated one. fp32 heads of 32, where a
+// rotation's pairs lie in one thread.
+bool attn_rotates(int dt, int hd);
 // Gradients into dqkv (same layout as qkv). Dbuf: [B, H, S] scratch. bf16 with head dim 64 or 128: the
 // tcgen05 kernels (err as for attn_fwd); other even bf16 head dims up to 128: the tcgen05 kernels on
 // zero-padded copies; else mma.sync; fp32: CUDA cores.
 void attn_bwd(int dt, const void* qkv, const void* out, const void* dout, const float* lse, float* Dbuf,
               void* dqkv, int B, int S, int H, int Hkv, int hd, cudaStream_t s, cudaMemPool_t pool = nullptr,
-              unsigned* err = nullptr);
+              unsigned* err = nullptr, const float* cs = nullptr);
 // dK, dV of each KV head (bf16, into dqkv) = fixed-order sums over its `rep` shares of the fp32 partials
 // part[2][Hkv * rep][NS][hd] (dK unscaled; times scale here).
 void launch_reduce_dkv(const float* part, void* dqkv, int NS, int H, int Hkv, int rep, int hd, float scale,

@@ -79,3 +79,23 @@ def test_fp32_attention_alignment(B, S, H, Hkv, hd):
         res.append((out.clone(), lse, dqkv.clone()))
     for a, b in zip(*res):
         assert torch.equal(a, b)
+
+
+# Heads of 32 are rotated inside the fp32 attention kernels: training steps against the float64 oracle, with the
+# loss and per-tensor tolerances of the other fp32 parity tests (1e-4).
+@pytest.mark.parametrize("seq,kv", [(50, 2), (33, 1), (31, 4)])
+def test_fp32_rotated_attention(seq, kv):
+    import synth
+    from tests.gpu_common import engine_for, fro_rel, oracle_for, rel
+    w = synth.Workload("rot-f32", synth.ModelDims(synth.ARCH_LLAMA, 2, 128, 4, kv, 344, 300, 64), "f32", batch=3, seq=seq, K=2,
+                       steps=2, lr=1e-4, seed=seq)
+    P = synth.make_params(w.dims, w.seed)
+    eng, orc = engine_for(w), oracle_for(w, P)
+    eng.load(P)
+    for s in range(w.steps):
+        ids, labels = synth.make_batch(w, s)
+        for a, b in zip(eng.step(ids.cuda(), labels.cuda()), orc.step(ids, labels)):
+            assert rel(a, b) <= 1e-4
+    for n in orc.trainable_names():
+        assert fro_rel(eng.get(n), orc.P[n]) <= 1e-4, n
+    eng.close()
