@@ -449,10 +449,22 @@ void lora_down(zl_ctx* c, const void* X, const void* A, void* u, int N, int in, 
   if (c->dt == BF16 && r == 16 && in % 8 == 0) {
     const double e = (double)esz(c);
     ProfScope p(c, s, PC_GEMM, 2.0 * N * r * (double)in, e * ((double)N * in + (double)r * in + (double)N * r));
-    launch_rank16(X, A, u, N, in, scale, s);
-    return;
+    if (rank16_down(X, A, u, N, in, scale, s)) return;
+    p.keep = false;
   }
   G(c, s, 0, N, r, in, X, A, u, nullptr, nullptr, scale);
+}
+
+// grad [r16, w] += u^T Y, the gradient of a LoRA factor from u [N, r16] and Y [N, w].
+void lora_grad(zl_ctx* c, const void* u, const void* Y, float* grad, int N, int w, cudaStream_t s) {
+  const int r = lora_r16(c->cfg.lora_rank);
+  if (c->dt == BF16 && r == 16) {
+    const double e = (double)esz(c);
+    ProfScope p(c, s, PC_GEMM, 2.0 * N * r * (double)w, e * ((double)N * w + (double)N * r) + 8.0 * r * w);
+    if (rank16_grad(u, Y, grad, N, w, s)) return;
+    p.keep = false;
+  }
+  G(c, s, 2, r, w, N, u, Y, grad, nullptr, nullptr);
 }
 
 // C = A op(B) (+ bias) (+ R) + u F for a LoRA term u [M, r16], F [r16, N]: one product with further k blocks where the
@@ -491,15 +503,15 @@ void linear_bwd_dx(zl_ctx* c, Chunk& k, int li, int i, const void* X, const void
                    int N, cudaStream_t s) {
   const Layer& L = k.layers[li];
   const void* W = Wc(c, k, li, (PK)kLoraP[i]);
-  const int in = L.lin_in[i], o = L.lin_out[i], r = lora_r16(c->cfg.lora_rank);
-  if (r <= 0) {
+  const int in = L.lin_in[i], o = L.lin_out[i];
+  if (lora_r16(c->cfg.lora_rank) <= 0) {
     G(c, s, 1, N, in, o, dY, W, dX, nullptr, nullptr);
     return;
   }
   lora_down(c, dY, TrainC(c, k, L.lb[i]), du, N, o, c->cfg.lora_scale, s);
   G_lora(c, s, 1, N, in, o, dY, W, dX, nullptr, nullptr, du, TrainC(c, k, L.la[i]));
-  G(c, s, 2, r, o, N, u, dY, k.grad + L.lb[i], nullptr, nullptr);
-  G(c, s, 2, r, in, N, du, X, k.grad + L.la[i], nullptr, nullptr);
+  lora_grad(c, u, dY, k.grad + L.lb[i], N, o, s);
+  lora_grad(c, du, X, k.grad + L.la[i], N, in, s);
 }
 
 void layer_fwd(zl_ctx* c, Chunk& k, int li, LayerSave& sv, const void* x, void* y, int B, int S, cudaStream_t s) {

@@ -140,8 +140,10 @@ struct GemmExt {
 };
 bool gemm_tc_ext(int mode, int M, int N, int K, const void* A, const void* B, void* C, const float* bias, const void* R,
                  const GemmExt& e, const GemmRope* rope, unsigned* err, cudaStream_t s, cudaMemPool_t pool);
-// U [N, 16] = scale * X [N, K] W [16, K]^T in bf16 (K % 8 == 0, 16-byte aligned rows): the rank-16 products of LoRA.
-void launch_rank16(const void* X, const void* W, void* U, int N, int K, float scale, cudaStream_t s);
+// The rank-16 products of LoRA, bf16: U [N, 16] = scale * X [N, K] W [16, K]^T, and G [16, C] += U [N, 16]^T Y [N, C]
+// (fp32). False, with nothing launched, unless the row lengths are multiples of 8 and the operands 16-byte aligned.
+bool rank16_down(const void* X, const void* W, void* U, int N, int K, float scale, cudaStream_t s);
+bool rank16_grad(const void* U, const void* Y, float* G, int N, int C, cudaStream_t s);
 bool gemm_tc_available();
 bool gemm_tc(int mode, int M, int N, int K, const void* A, const void* B, void* C, const float* bias, const void* R,
              unsigned* err, cudaStream_t s, cudaMemPool_t pool, float alpha, int rmode = 0);

@@ -34,3 +34,10 @@ def test_lora_gradients(arch, rank, heads, kv, hd, batch, seq):
         h = eng.forward_chunk(k, h.view(batch * seq, -1).to(torch.bfloat16).cuda(), None, batch, seq)
         h = h.float().cpu().view(batch, seq, -1)
     eng.close()
+
+
+# Token counts on the other side of the rank-16 kernels' lines: 32 rows a CTA (the last one ragged), and the tokens
+# shared by clusters of eight and of four.
+@pytest.mark.parametrize("batch,seq", [(10, 251), (5, 255), (3, 200)])
+def test_lora_gradients_many_tokens(batch, seq):
+    test_lora_gradients(synth.ARCH_LLAMA, 16, 2, 1, 64, batch, seq)
