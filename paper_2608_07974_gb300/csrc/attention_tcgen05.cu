@@ -61,32 +61,35 @@ __device__ __forceinline__ void tmem_release(uint64_t* fin, uint32_t tmem, uint3
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols) : "memory");
 }
 
-// 128 rows x HD columns of one head from `m` into a tile of HD / 64 blocks of [128 rows][64 columns].
-template <int HD>
+// ROWS rows x HD columns of one head from `m` (boxes of BOX rows) into a tile of HD / 64 blocks of [ROWS][64 columns].
+template <int HD, int ROWS = 128, int BOX = 128>
 __device__ __forceinline__ void load_tile(uint8_t* dst, const CUtensorMap* m, uint64_t* bar, int col, int row, int b) {
 #pragma unroll
-  for (int c = 0; c < HD / 64; ++c) tma3d(dst + c * 16384, m, bar, col + 64 * c, row, b);
+  for (int c = 0; c < HD / 64; ++c)
+#pragma unroll
+    for (int r = 0; r < ROWS; r += BOX) tma3d(dst + (c * ROWS + r) * 128, m, bar, col + 64 * c, row + r, b);
 }
 
-// D[128 x 128] = A[128 x HD] B[128 x HD]^T, both K-major tiles of load_tile.
-template <int HD>
+// D[128 x NB] = A[128 x HD] B[NB x HD]^T, both K-major tiles of load_tile.
+template <int HD, int NB = 128>
 __device__ __forceinline__ void mma_nt(uint32_t d, uint32_t a, uint32_t b) {
-  constexpr uint32_t id = idesc_f16(128, 128, false, false);
+  constexpr uint32_t id = idesc_f16(128, NB, false, false);
 #pragma unroll
   for (int ks = 0; ks < HD / 16; ++ks) {
-    const uint32_t o = (ks / 4) * 16384 + (ks % 4) * 32;
-    mma_bf16(d, sdesc(a + o, 16, 1024), sdesc(b + o, 16, 1024), id, ks > 0 ? 1u : 0u);
+    const uint32_t o = (ks % 4) * 32;
+    mma_bf16(d, sdesc(a + (ks / 4) * 16384 + o, 16, 1024), sdesc(b + (ks / 4) * NB * 128 + o, 16, 1024), id,
+             ks > 0 ? 1u : 0u);
   }
 }
 
-// D[128 x HD] (+)= A[128 x 128] B[128 x HD]: A in TMEM, each group of CW score columns holding its bf16
+// D[128 x HD] (+)= A[128 x NB] B[NB x HD]: A in TMEM, each group of CW score columns holding its bf16
 // pairs in the group's first CW / 2 columns; B a tile of load_tile read MN-major (16-row steps 2 KB apart).
-template <int HD, int CW>
+template <int HD, int CW, int NB = 128>
 __device__ __forceinline__ void mma_ta(uint32_t d, uint32_t a, uint32_t b, bool acc) {
   constexpr uint32_t id = idesc_f16(128, HD, false, true);
 #pragma unroll
-  for (int ks = 0; ks < 8; ++ks)
-    mma_bf16_ta(d, a + (ks * 16 / CW) * CW + (ks * 16 % CW) / 2, sdesc(b + ks * 2048, 16384, 1024), id,
+  for (int ks = 0; ks < NB / 16; ++ks)
+    mma_bf16_ta(d, a + (ks * 16 / CW) * CW + (ks * 16 % CW) / 2, sdesc(b + ks * 2048, NB * 128, 1024), id,
                 (acc || ks > 0) ? 1u : 0u);
 }
 
@@ -118,31 +121,31 @@ __device__ __forceinline__ void store_rows(uint32_t t, float f, uint8_t* st, con
 }
 
 // ==============================================================================================
-// Forward, one pass with lazy rescaling. Per 128-key block j: S = Q K_j^T (TMEM), the softmax warps (half
-// a query row per thread, the two halves' maxima exchanged through shared memory) turn S into P =
-// 2^(s - m) in place, O += P V_j. The running maximum m moves only
+// Forward, one pass with lazy rescaling. Per 64-key block j: S = Q K_j^T (TMEM), the softmax warps (a query
+// row per thread) turn S into P = 2^(s - m) in place, O += P V_j. The running maximum m moves only
 // when the block maximum exceeds it by more than 8 (log2 units): P then stays at most 256 (exact in fp32
 // sums, the usual bf16 rounding), and O and the row sum l are rescaled (in TMEM / registers) only on such
 // a move. At the end O / l is the softmax-weighted sum and m + log2 l the row's log-sum-exp.
 //
-// One block's chain S -> softmax -> P V is serial (S, P and O share 256 TMEM columns), and two CTAs per SM
-// (256 columns and at most 113 KB of shared memory each) fill each other's gaps: while one is in its
-// softmax, the other's products run. What bounds it: the softmax phase (about 1,450 cycles a block with its
-// hand-offs, of which 512 are the exponentials) against 1,024 cycles of products at head dim 128. Measured
-// against one persistent CTA per SM with P in shared memory: B 2, S 1024, 32 heads of 128 36.8 -> 22.7 us
-// (755 TFLOP/s); B 1, S 4096 1,250 TFLOP/s; B 4, S 2048, 32 / 4 heads of 64 103 us (665 TFLOP/s). Four
-// softmax warps with whole rows (no exchange) measured 1-3% slower.
+// Two score buffers: S of the next block is formed under this block's softmax, and two CTAs per SM (256 TMEM
+// columns and at most 113 KB of shared memory each) fill each other's gaps. What bounds it: the softmax warps, two
+// an SM quarter, whose block (about 1,450 cycles, of which 256 are the exponentials) is a chain of TMEM read,
+// maximum, exponentials, TMEM write and hand-off. Measured against one score buffer of 128 keys and two softmax warps
+// per quadrant (which fit beside it): B 4, S 2048, 32 / 4 heads of 64 103 -> 92 us (743 TFLOP/s); B 2, S 1024, 32
+// heads of 128 22.7 -> 20.8 us (827 TFLOP/s); B 1, S 4096 1,250 -> 1,260 TFLOP/s. On the same blocks: three buffers
+// at head dim 64 93 us; two warps per quadrant, half a row each, 100 us; two groups of warps on alternate
+// blocks, each with an O of its own, 98 us; one buffer and three CTAs 95 us.
 // ==============================================================================================
 template <int HD>
 struct FCfg {
-  static constexpr int T = 128 * HD * 2;                // one tile
-  static constexpr int NST = HD == 64 ? 2 : 1;          // K and V buffers
-  static constexpr int XBYTES = (2 * 2 * 128 + 2 * 128) * 4;   // maxima [2 buffers][2 halves][rows], sums [2][rows]
-  static constexpr int SMEM = T + NST * 2 * T + XBYTES + 256 + 1024;
-  static constexpr int NSW = 8;                         // softmax warps: two per lane quadrant, 64 keys each
-  static constexpr int NTHR = 64 + 32 * NSW;            // TMA warp, MMA warp, softmax warps
-  static constexpr uint32_t OCOL = 128, COLS = 256;
-  static_assert(SMEM + 1024 <= 233472 / 2, "two CTAs per SM");
+  static constexpr int KB = 64;                              // keys per block
+  static constexpr int T = 128 * HD * 2, KT = KB * HD * 2;   // the Q tile, a K or V tile
+  static constexpr int NST = HD == 64 ? 4 : 2;               // K and V buffers
+  static constexpr int SMEM = T + NST * 2 * KT + 256 + 1024;
+  static constexpr int NSW = 4;                              // softmax warps, one per TMEM lane quadrant
+  static constexpr int NTHR = 64 + 32 * NSW;                 // TMA warp, MMA warp, softmax warps
+  static constexpr uint32_t OCOL = 2 * KB, COLS = 256;       // two score buffers, O
+  static_assert(2 * (SMEM + 1024) <= 233472, "two CTAs per SM");
   static_assert(OCOL + HD <= COLS, "TMEM columns");
 };
 
@@ -151,28 +154,27 @@ __global__ void __launch_bounds__(FCfg<HD>::NTHR, 2)
     attn_fwd_k(const __grid_constant__ CUtensorMap tqkv, const __grid_constant__ CUtensorMap tout,
                float* __restrict__ lse, int S, int H, int Hkv, float scale, unsigned* err) {
   using C_ = FCfg<HD>;
-  constexpr int NST = C_::NST;
+  constexpr int NST = C_::NST, KB = C_::KB;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* sq = smem;                       // Q, at the end the staging of the output
   uint8_t* sk = sq + C_::T;                 // [NST] K
-  uint8_t* sv = sk + NST * C_::T;           // [NST] V
-  float* xmax = (float*)(sv + NST * C_::T);   // [2][2][128]
-  float* xsum = xmax + 512;                   // [2][128]
-  uint64_t* kfull = (uint64_t*)(xsum + 256);
+  uint8_t* sv = sk + NST * C_::KT;           // [NST] V
+  uint64_t* kfull = (uint64_t*)(sv + NST * C_::KT);
   uint64_t* kempty = kfull + NST;
   uint64_t* vfull = kempty + NST;
   uint64_t* vempty = vfull + NST;
   uint64_t* qfull = vempty + NST;
-  uint64_t* sfull = qfull + 1;
-  uint64_t* pfull = sfull + 1;
-  uint64_t* ofull = pfull + 1;
-  uint64_t* fin = ofull + 1;
+  uint64_t* sfull = qfull + 1;    // [2], as pfull and pvdone: by block parity
+  uint64_t* pfull = sfull + 2;
+  uint64_t* pvdone = pfull + 2;
+  uint64_t* fin = pvdone + 2;
   uint32_t* tbase = (uint32_t*)(fin + 1);
   volatile int* abort_flag = (volatile int*)(tbase + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int h = blockIdx.x, b = blockIdx.y, qb = gridDim.z - 1 - blockIdx.z;   // longest first
-  const int kvh = h / (H / Hkv), q0 = qb * QB, nkb = qb + 1;
+  const int kvh = h / (H / Hkv), q0 = qb * QB;
+  const int nkb = (min(q0 + QB, S) + KB - 1) / KB;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NST; ++s) {
@@ -182,9 +184,11 @@ __global__ void __launch_bounds__(FCfg<HD>::NTHR, 2)
       mbar_init(&vempty[s], 1);
     }
     mbar_init(qfull, 1);
-    mbar_init(sfull, 1);
-    mbar_init(pfull, C_::NSW);
-    mbar_init(ofull, 1);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&sfull[s], 1);
+      mbar_init(&pfull[s], C_::NSW);
+      mbar_init(&pvdone[s], 1);
+    }
     mbar_init(fin, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -204,7 +208,7 @@ __global__ void __launch_bounds__(FCfg<HD>::NTHR, 2)
     const bool leader = elect_one();
     if (leader) {
       mbar_expect_tx(qfull, C_::T);
-      load_tile<HD>(sq, &tqkv, qfull, h * HD, q0, b);
+      load_tile<HD, 128, KB>(sq, &tqkv, qfull, h * HD, q0, b);
     }
     bool ok = true;
     int kp[NST], vp[NST];   // parity of the last fill of each buffer, -1 if none
@@ -216,15 +220,15 @@ __global__ void __launch_bounds__(FCfg<HD>::NTHR, 2)
       if (!uwait(&kempty[st], ph ^ 1u, abort_flag, err)) { ok = false; break; }
       kp[st] = (int)ph;
       if (leader) {
-        mbar_expect_tx(&kfull[st], C_::T);
-        load_tile<HD>(sk + st * C_::T, &tqkv, &kfull[st], xk, j * QB, b);
+        mbar_expect_tx(&kfull[st], C_::KT);
+        load_tile<HD, KB, KB>(sk + st * C_::KT, &tqkv, &kfull[st], xk, j * KB, b);
       }
       __syncwarp();
       if (!uwait(&vempty[st], ph ^ 1u, abort_flag, err)) { ok = false; break; }
       vp[st] = (int)ph;
       if (leader) {
-        mbar_expect_tx(&vfull[st], C_::T);
-        load_tile<HD>(sv + st * C_::T, &tqkv, &vfull[st], xv, j * QB, b);
+        mbar_expect_tx(&vfull[st], C_::KT);
+        load_tile<HD, KB, KB>(sv + st * C_::KT, &tqkv, &vfull[st], xv, j * KB, b);
       }
       __syncwarp();
     }
@@ -241,52 +245,57 @@ __global__ void __launch_bounds__(FCfg<HD>::NTHR, 2)
     const uint32_t q_addr = su32(sq), k_addr = su32(sk), v_addr = su32(sv);
     const bool leader = elect_one();
     bool ok = uwait(qfull, 0, abort_flag, err);
-    for (int j = 0; ok && j < nkb; ++j) {
+    // S of block j into its buffer, over P of block j - 2, which its P V product (issued before) reads first
+    auto scores = [&](int j) {
       const int st = j % NST;
-      const uint32_t ph = (uint32_t)(j / NST) & 1u;
-      if (!uwait(&kfull[st], ph, abort_flag, err)) { ok = false; break; }
+      if (!uwait(&kfull[st], (uint32_t)(j / NST) & 1u, abort_flag, err)) return false;
       fence_after();
-      if (leader) {   // over P of block j - 1, which its P V product (issued before) reads first
-        mma_nt<HD>(tmem, q_addr, k_addr + st * C_::T);
-        mma_commit(sfull);
+      if (leader) {
+        mma_nt<HD, KB>(tmem + (uint32_t)((j & 1) * KB), q_addr, k_addr + st * C_::KT);
+        mma_commit(&sfull[j & 1]);
         mma_commit(&kempty[st]);
       }
       __syncwarp();
-      if (!uwait(&vfull[st], ph, abort_flag, err) || !uwait(pfull, (uint32_t)j & 1u, abort_flag, err)) {
+      return true;
+    };
+    ok = ok && scores(0) && (nkb == 1 || scores(1));
+    for (int j = 0; ok && j < nkb; ++j) {
+      const int st = j % NST;
+      if (!uwait(&vfull[st], (uint32_t)(j / NST) & 1u, abort_flag, err) ||
+          !uwait(&pfull[j & 1], (uint32_t)(j >> 1) & 1u, abort_flag, err)) {
         ok = false;
         break;
       }
       fence_after();
       if (leader) {
-        mma_ta<HD, 32>(tmem + C_::OCOL, tmem, v_addr + st * C_::T, j > 0);
+        mma_ta<HD, 32, KB>(tmem + C_::OCOL, tmem + (uint32_t)((j & 1) * KB), v_addr + st * C_::KT, j > 0);
         mma_commit(&vempty[st]);
-        if (j == nkb - 1) mma_commit(ofull);
+        mma_commit(&pvdone[j & 1]);
       }
       __syncwarp();
+      if (j + 2 < nkb && !scores(j + 2)) ok = false;
     }
     if (leader) mma_commit(fin);   // every MMA of the leader completes before TMEM is released
     __syncwarp();
   } else {
-    // ---------------- softmax and output: warps 2..9, half a query row per thread ----------------
-    const int quad = warp & 3, half = (warp - 2) >> 2;    // TMEM lane quadrant; key half of every block
+    // ---------------- softmax and output: a query row per thread ----------------
+    const int quad = warp & 3;    // TMEM lane quadrant
     const int r = quad * 32 + lane, q = q0 + r;
     const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
-    const uint32_t ts = trow + (uint32_t)(64 * half);
     const float sl2 = scale * kL2e;
     const uint64_t SL2 = f2(sl2, sl2);
-    // After a failed wait the loop only runs on over whatever TMEM holds (both warps of a quadrant pass every
-    // named barrier); nothing is stored.
     bool ok = true;
     float m = -INFINITY;                                  // running maximum (log2 units)
-    uint64_t la = f2(0.f, 0.f), lb = la;                  // this half's row sum, in four parts
+    uint64_t la = f2(0.f, 0.f), lb = la;                  // the row sum, in four parts
     for (int j = 0; j < nkb; ++j) {
-      if (ok && !uwait(sfull, (uint32_t)j & 1u, abort_flag, err)) ok = false;
+      if (!uwait(&sfull[j & 1], (uint32_t)(j >> 1) & 1u, abort_flag, err)) { ok = false; break; }
+      const uint32_t ts = trow + (uint32_t)((j & 1) * KB);
       uint32_t v[64];
       float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
       fence_after();
       tmem_ld64u(ts, v);
-      if (j == nkb - 1) {   // the diagonal block: keys after the query (and past the end) are masked
-        const int kmax = min(q, S - 1) - j * QB - 64 * half;
+      if (j + 2 >= nkb) {   // the diagonal blocks: keys after the query (and past the end) are masked
+        const int kmax = min(q, S - 1) - j * KB;
 #pragma unroll
         for (int e = 0; e < 64; ++e)
           if (e > kmax) v[e] = 0xff800000u;
@@ -297,19 +306,16 @@ __global__ void __launch_bounds__(FCfg<HD>::NTHR, 2)
         for (int u = 0; u < 4; ++u) mx[u] = fmaxf(mx[u], __uint_as_float(v[e + u]));
       }
       const float mh = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sl2;
-      // the partner half's maximum (double-buffered by block parity; one barrier per block)
-      float* xm = xmax + (j & 1) * 256;
-      xm[half * 128 + r] = mh;
-      asm volatile("bar.sync %0, 64;" ::"r"(1 + quad) : "memory");
-      const float mnew = fmaxf(m, fmaxf(mh, xm[(1 - half) * 128 + r]));
+      const float mnew = fmaxf(m, mh);
       const bool move = mnew > m + 8.f;   // also true on the first block (m = -inf)
-      // the previous P V product completed before this S, which was issued after it
-      if (j > 0 && __any_sync(0xffffffffu, move)) {   // rescale this half of the O row (warp-wide TMEM access)
+      if (j > 0 && __any_sync(0xffffffffu, move)) {   // rescale the O row (warp-wide TMEM access), P V of j - 1 in it
+        if (!uwait(&pvdone[(j - 1) & 1], (uint32_t)((j - 1) >> 1) & 1u, abort_flag, err)) { ok = false; break; }
+        fence_after();
         const float a = move ? ex2(m - mnew) : 1.f;
         la = mul2(la, f2(a, a));
         lb = mul2(lb, f2(a, a));
 #pragma unroll 1
-        for (int c = half * (HD / 2); c < (half + 1) * (HD / 2); c += 32) {
+        for (int c = 0; c < HD; c += 32) {
           float o[32];
           tmem_ld32(trow + C_::OCOL + (uint32_t)c, o);
 #pragma unroll
@@ -337,21 +343,17 @@ __global__ void __launch_bounds__(FCfg<HD>::NTHR, 2)
       tmem_st_wait();
       fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(pfull);
+      if (lane == 0) mbar_arrive(&pfull[j & 1]);
     }
-    // output: both halves use the same m; O / (l_0 + l_1), log-sum-exp m + log2(l_0 + l_1)
+    // output: O / l, log-sum-exp m + log2 l
     const float2 ls = uf2(add2(la, lb));
-    xsum[half * 128 + r] = ls.x + ls.y;
-    asm volatile("bar.sync %0, 64;" ::"r"(1 + quad) : "memory");
-    const float lt = xsum[r] + xsum[128 + r];
+    const float lt = ls.x + ls.y;
     const float inv = lt > 0.f ? 1.f / lt : 0.f;
-    if (ok && uwait(ofull, 0, abort_flag, err)) {
+    if (ok && uwait(&pvdone[(nkb - 1) & 1], (uint32_t)((nkb - 1) >> 1) & 1u, abort_flag, err)) {
       fence_after();
-      // one 64-column box per warp (head dim 64: the first warp of a quadrant has the only one)
-      if (half < HD / 64)
-        store_rows(trow + C_::OCOL, inv, sq + quad * (HD / 64) * 4096, &tout, h * HD, q0 + quad * 32, b, S, half,
-                   half + 1, lane);
-      if (q < S && half == 0) lse[((size_t)b * H + h) * S + q] = (lt > 0.f ? m + log2f(lt) : INFINITY) * kLn2;
+      store_rows(trow + C_::OCOL, inv, sq + quad * (HD / 64) * 4096, &tout, h * HD, q0 + quad * 32, b, S, 0, HD / 64,
+                 lane);
+      if (q < S) lse[((size_t)b * H + h) * S + q] = (lt > 0.f ? m + log2f(lt) : INFINITY) * kLn2;
     }
   }
 
@@ -1210,7 +1212,7 @@ bool fwd_launch(const void* qkv, void* out, float* lse, int B, int S, int H, int
     attr = true;
   }
   CUtensorMap mq, mo;
-  if (!qkv_map(&mq, qkv, B, S, (H + 2 * Hkv) * HD, 128) || !qkv_map(&mo, out, B, S, H * HD, 32)) return false;
+  if (!qkv_map(&mq, qkv, B, S, (H + 2 * Hkv) * HD, C_::KB) || !qkv_map(&mo, out, B, S, H * HD, 32)) return false;
   return launch_pdl(kern, dim3(H, B, (S + QB - 1) / QB), C_::NTHR, C_::SMEM, s, mq, mo, lse, S, H, Hkv, scale, err) ==
          cudaSuccess;
 }

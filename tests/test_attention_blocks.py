@@ -44,3 +44,28 @@ def test_attention_block_edges(B, Bb, S, H, Hkv, hd):
     again = torch.empty_like(dqkv)
     B.zl_op_attention_bwd(B.ZL_DTYPE_BF16, qkv, out, dout, lse, again, Bb, S, H, Hkv, hd)
     assert torch.equal(again, dqkv)   # fixed summation order
+
+
+# The forward's 64-key blocks: two keys (with one dQ and dK are exactly zero and have no relative error), a block exactly, one key more and less, an odd and an even number of them.
+@pytest.mark.parametrize("S,hd", [(2, 64), (63, 128), (64, 64), (65, 128), (191, 64), (193, 64), (193, 128)])
+def test_attention_key_blocks(B, S, hd):
+    test_attention_block_edges(B, 2, S, 2, 1, hd)
+
+
+@pytest.mark.parametrize("S,hd", [(300, 64), (450, 128)])
+def test_attention_moving_maximum(B, S, hd):
+    """Scores that grow with the key's position: the running maximum moves, and O is rescaled, in every block."""
+    g = torch.Generator(device="cuda").manual_seed(S)
+    q, k, v = (torch.randn(S, 2, hd, device="cuda", generator=g) for _ in range(3))
+    q[..., 0] = 1.0
+    k[..., 0] = torch.arange(S, device="cuda").float()[:, None] * (0.4 * hd ** 0.5)   # 0.4 a key, 26 a block (> 8 in log2)
+    qkv = torch.cat([q, k, v], 1).reshape(S, 6 * hd).to(torch.bfloat16)
+    out, lse = torch.empty(S, 2 * hd, device="cuda", dtype=torch.bfloat16), torch.empty(1, 2, S, device="cuda")
+    B.zl_op_attention(B.ZL_DTYPE_BF16, qkv, out, lse, 1, S, 2, 2, hd)
+    t = qkv.double().view(S, 6, hd).transpose(0, 1)
+    s = (t[:2] @ t[2:4].transpose(-1, -2)) / hd ** 0.5
+    s = s.masked_fill(torch.ones(S, S, dtype=torch.bool, device="cuda").triu(1), float("-inf"))
+    ref = (torch.softmax(s, -1) @ t[4:]).transpose(0, 1).reshape(S, 2 * hd)
+    # fp32 scores of up to 0.4 S carry errors of 2^-24 of their terms; P and the result are rounded to bf16
+    assert float((lse[0].double() - torch.logsumexp(s, -1)).abs().max()) <= 0.4 * S * hd * 2.0 ** -23
+    assert float((out.double() - ref).norm() / ref.norm()) <= 1e-2
