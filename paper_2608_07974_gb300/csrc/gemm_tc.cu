@@ -630,7 +630,7 @@ __global__ void __launch_bounds__(UPD ? kThreadsUpd : kThreads, 1)
 }
 
 // Sums the split-K partials in split order (deterministic) and applies the epilogue (mode 4: the fused
-// optimizer step of `u`, as update_row32 does it).
+// optimizer step of `u`, as the fused epilogue does it).
 __global__ void splitk_reduce_k(const float* __restrict__ ws, int splits, int M, int N, int mode, void* C,
                                 const float* __restrict__ bias, const bf16* R, float alpha, int rmode,
                                 const GemmUpdate u) {

@@ -1,3 +1,4 @@
+import gc
 import os
 import sys
 
@@ -25,3 +26,9 @@ def pytest_collection_modifyitems(config, items):
     for it in items:
         if "gpu" in it.keywords:
             it.add_marker(skip)
+
+
+@pytest.fixture(autouse=True, scope="module")
+def _no_garbage_from_earlier_modules():
+    """Tensors that an earlier module left in reference cycles go now, not inside a region whose allocations a test counts."""
+    gc.collect()
