@@ -849,7 +849,9 @@ struct Plan {
 // The plan with the least predicted time (us): a fixed cost (launch, set-up, first loads), then waves of units
 // (a tile, or a pair's two, times K / splits) on 152 SMs (76 pairs, or 304 slots of width 64), each 64-deep k
 // block of a unit at the rate measured for its kernel and no wave shorter than a tile's epilogue, the last
-// wave's epilogue, and for splits the fp32 partials through HBM and the reduction. Fitted to every plan on 53
+// wave's epilogue, and for splits the fp32 partials through HBM and 4 us for the reduction with its launch and the
+// workspace's allocation (2 us, the reduction alone, lost where a small product is one of a sequence: a linear of 412
+// tokens, 2176 x 800, forward, dX and dW 36.4 us against 30.9; 694, 1728 x 5504 66 against 59). Fitted to every plan on 53
 // shapes (4096^3, the GPT-2, 1.1B and 7B layer and head shapes, ragged ones from 203 rows): 8% off at the
 // median of both sides, the chosen plan within 4% of the fastest one on all but a few small shapes. Pairs win wherever
 // their 256-row tiles fill the SMs (7B QKV forward 117 us against 131 alone; 4096^3 79.5 against 94); single
@@ -885,7 +887,7 @@ Plan choose(int mode, int M, int N, int K) {
       const long waves = (tiles * sp + slots - 1) / slots;
       const double e = sp > 1 ? c.epi : epi;
       double t = 2.8 + waves * std::max(kps * c.kb * (dw ? 1.06 : 1.0), e) + e;
-      if (sp > 1) t += (8.0 * sp * M * N + state) / hbm + 2.0;
+      if (sp > 1) t += (8.0 * sp * M * N + state) / hbm + 4.0;
       else t = std::max(t, state / hbm + 2.8);
       if (t < best * 0.98) { best = t; p = Plan{c.bn, sp, c.pair}; }
     }
