@@ -69,3 +69,30 @@ def test_attention_moving_maximum(B, S, hd):
     # fp32 scores of up to 0.4 S carry errors of 2^-24 of their terms; P and the result are rounded to bf16
     assert float((lse[0].double() - torch.logsumexp(s, -1)).abs().max()) <= 0.4 * S * hd * 2.0 ** -23
     assert float((out.double() - ref).norm() / ref.norm()) <= 1e-2
+
+
+@pytest.mark.parametrize("S,hd", [(100, 64), (128, 128), (129, 128), (300, 64)])
+def test_attention_first_maximum(B, S, hd):
+    """A row's largest probability among its first 128 keys is 1, which bf16 holds, also where the key lies in the second 64: one
+    key there outweighs the first by 2^0.1 to 2^7.6, less than what moves the running maximum."""
+    key, D = 64 + (S - 64) // 2 if S < 128 else 90, 16
+    g = torch.Generator(device="cuda").manual_seed(S)
+    q, k = torch.zeros(S, 2, hd, device="cuda"), torch.zeros(S, 2, hd, device="cuda")
+    q[..., 0] = torch.linspace(0.1, 7.6, S, device="cuda")[:, None] * 0.6931 * hd ** 0.5 / D   # log2 units over the first key
+    k[key, :, 0] = D
+    q[..., 1], k[..., 1] = -30.0, hd ** 0.5       # every key but two: e^-30 of the first
+    k[0, :, 1] = k[key, :, 1] = 0.0
+    v = 1.0 + torch.rand(S, 2, hd, device="cuda", generator=g)
+    qkv = torch.cat([q, k, v], 1).reshape(S, 6 * hd).to(torch.bfloat16)
+    out, lse = torch.empty(S, 2 * hd, device="cuda", dtype=torch.bfloat16), torch.empty(1, 2, S, device="cuda")
+    B.zl_op_attention(B.ZL_DTYPE_BF16, qkv, out, lse, 1, S, 2, 2, hd)
+    t = qkv.double().view(S, 6, hd).transpose(0, 1)
+    s = (t[:2] @ t[2:4].transpose(-1, -2)) / hd ** 0.5
+    s = s.masked_fill(torch.ones(S, S, dtype=torch.bool, device="cuda").triu(1), float("-inf"))
+    ref = (torch.softmax(s, -1) @ t[4:]).transpose(0, 1)[key:]
+    # bf16 rounds by at most 2^-8 of a value's power of two: the result once, and the first key's probability once, a share w2 of
+    # the result (times a value of at most 2); fp32 sums and exponentials stay below 1e-5
+    w2 = torch.softmax(s, -1)[:, key:, 0].transpose(0, 1)[..., None]
+    got = out.double().view(S, 2, hd)[key:]
+    bound = 2.0 ** (torch.floor(torch.log2(ref)) - 8) + 2.0 ** -8 * w2 * 2.0 + 1e-5
+    assert bool(((got - ref).abs() <= bound).all()), float(((got - ref).abs() / bound).max())
