@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_fwd_k(const T* __restrict
       float mn = m;
 #pragma unroll
       for (int u = 0; u < AF; ++u) mn = fmaxf(mn, s[u]);
-      if (mn > -INFINITY) {   // (past the row's last key a warp still runs for its other rows)
+      if (j0 + j <= i) {   // past the row's last key a warp still runs for its other rows (a group of NaN scores has no maximum)
         const float corr = expf(m - mn);
 #pragma unroll
         for (int u = 0; u < AF; ++u) s[u] = expf(s[u] - mn);

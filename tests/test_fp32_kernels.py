@@ -81,6 +81,25 @@ def test_fp32_attention_alignment(B, S, H, Hkv, hd):
         assert torch.equal(a, b)
 
 
+def _f32_attention(B, qkv, dout, S, H, Hkv, hd):
+    out, dqkv, lse = torch.empty_like(dout), torch.empty_like(qkv), torch.empty(1, H, S, device="cuda")
+    B.zl_op_attention(0, qkv, out, lse, 1, S, H, Hkv, hd)
+    B.zl_op_attention_bwd(0, qkv, out, dout, lse, dqkv, 1, S, H, Hkv, hd)
+    return out.view(S, H, hd), lse[0].T, dqkv.view(S, H + 2 * Hkv, hd)
+
+
+# A row whose first keys all have NaN scores (a whole group of eight, or of the row's length) is NaN, whatever follows.
+@pytest.mark.parametrize("nan_keys", [1, 8, 16, 40])
+@pytest.mark.parametrize("hd", [32, 66, 128])
+def test_fp32_attention_keeps_nan(B, nan_keys, hd):
+    S, H, Hkv = 70, 2, 1
+    g = torch.Generator(device="cuda").manual_seed(hd)
+    qkv, dout = torch.randn(S, (H + 2) * hd, device="cuda", generator=g), torch.randn(S, H * hd, device="cuda", generator=g)
+    qkv[:nan_keys, H * hd] = float("nan")
+    out, lse, _ = _f32_attention(B, qkv, dout, S, H, Hkv, hd)
+    assert bool(out.isnan().all()) and bool(lse.isnan().all())
+
+
 # Heads of 32 are rotated inside the fp32 attention kernels: training steps against the float64 oracle, with the
 # loss and per-tensor tolerances of the other fp32 parity tests (1e-4).
 @pytest.mark.parametrize("seq,kv", [(50, 2), (33, 1), (31, 4)])
