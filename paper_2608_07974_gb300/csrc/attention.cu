@@ -20,7 +20,10 @@ namespace {
 // in flight together. A tile's rows are loaded into registers during the tile before, 16 bytes a load, because on
 // small shapes the loads' latency is the kernel: with scalar loads between the barriers 4 x 64 tokens, 4 heads of
 // 32 took 9.2 us forward and 14.4 us backward, with these 5.7 and 10.1 (2 x 512 tokens, 16 heads of 64 over 4: 139
-// and 713, now 137 and 581: there shared-memory reads, one per four multiply-adds, are the bound).
+// and 713, then 137 and 581: there shared-memory reads, one per four multiply-adds, are the bound).
+// Masked rows of a diagonal tile (and, for dK and dV, rows past the end) are left out, not weighted with zero; the
+// other tiles run a loop without masks, which gives back more than that costs: 5.8 and 9.8 us with zero weights, now
+// 6.2 and 7.7 (137 and 569, now 137 and 400).
 // One warp per row with one key at a time, which these replace, waited for five shuffles and a global load per
 // key: 4 x 64 tokens, 4 heads of 32 (the tiny fp32 workload) is bound by that chain, not by its 17 MFLOP.
 // ------------------------------------------------------------------------------------------------
@@ -137,11 +140,13 @@ __device__ __forceinline__ void dot_tile(float* s, const RowV<HDP>& a, const flo
 #pragma unroll
     for (int u = 0; u < U; ++u) s[u] += __shfl_xor_sync(0xffffffffu, s[u], x);
 }
-// o += sum_u w[u] * tile row j + u
-template <int HDP, int U>
-__device__ __forceinline__ void axpy_tile(RowV<HDP>& o, const float* w, const float* tile, int j, int sub) {
+// o += sum_u w[u] * tile row j + u. EDGE: over u from lo to hi - 1 only (a weight of zero would still turn a masked
+// row's Inf or NaN into NaN).
+template <int HDP, int U, bool EDGE>
+__device__ __forceinline__ void axpy_tile(RowV<HDP>& o, const float* w, const float* tile, int j, int sub, int lo = 0, int hi = U) {
 #pragma unroll
   for (int u = 0; u < U; ++u) {
+    if (EDGE && (u < lo || u >= hi)) continue;
     const float* t = tile + (j + u) * (HDP + 4) + 4 * sub;
 #pragma unroll
     for (int c = 0; c < RowV<HDP>::NC; ++c) {
@@ -186,29 +191,37 @@ __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_fwd_k(const T* __restrict
     put_row<HDP>(vs, vn, row, sub);
     __syncthreads();
     if (j0 + AR <= i0) fetch(j0 + AR);
+    auto keys = [&](auto edge) {   // the tile's keys, on the diagonal (edge) those up to the query
+      constexpr bool EDGE = decltype(edge)::value;
 #pragma unroll 1
-    for (int j = 0; j < AR; j += AF) {
-      float s[AF];
-      dot_tile<HDP, AF>(s, q, ks, j, sub);
+      for (int j = 0; j < AR; j += AF) {
+        float s[AF];
+        dot_tile<HDP, AF>(s, q, ks, j, sub);
+        const int n = i + 1 - j0 - j;   // visible keys from j on
+        if (EDGE) {
 #pragma unroll
-      for (int u = 0; u < AF; ++u)
-        if (j0 + j + u > i) s[u] = -INFINITY;
-      float mn = m;
+          for (int u = 0; u < AF; ++u)
+            if (u >= n) s[u] = -INFINITY;
+        }
+        float mn = m;
 #pragma unroll
-      for (int u = 0; u < AF; ++u) mn = fmaxf(mn, s[u]);
-      if (j0 + j <= i) {   // past the row's last key a warp still runs for its other rows (a group of NaN scores has no maximum)
-        const float corr = expf(m - mn);
+        for (int u = 0; u < AF; ++u) mn = fmaxf(mn, s[u]);
+        if (!EDGE || n > 0) {   // past the row's last key a warp still runs for its other rows (a group of NaN scores has no maximum)
+          const float corr = expf(m - mn);
 #pragma unroll
-        for (int u = 0; u < AF; ++u) s[u] = expf(s[u] - mn);
-        float ls = 0.f;
+          for (int u = 0; u < AF; ++u) s[u] = expf(s[u] - mn);
+          float ls = 0.f;
 #pragma unroll
-        for (int u = 0; u < AF; u += 2) ls += s[u] + s[u + 1];
-        l = l * corr + ls;
-        scale_row<HDP>(o, corr);
-        axpy_tile<HDP, AF>(o, s, vs, j, sub);
-        m = mn;
+          for (int u = 0; u < AF; u += 2) ls += s[u] + s[u + 1];
+          l = l * corr + ls;
+          scale_row<HDP>(o, corr);
+          axpy_tile<HDP, AF, EDGE>(o, s, vs, j, sub, 0, n);
+          m = mn;
+        }
       }
-    }
+    };
+    if (j0 < i0) keys(std::false_type{});
+    else keys(std::true_type{});
   }
   if (i >= S) return;
   store_row<T, HDP>(out + (size_t)(b * S + i) * H * hd + h * hd, o, hd, sub, 1.f / l);
@@ -259,15 +272,20 @@ __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_bwd_k(const T* __restrict
       put_row<HDP>(tb, vn, row, sub);
       __syncthreads();
       if (j0 + AR <= i0) fetch(j0 + AR);
+      auto keys = [&](auto edge) {   // as in the forward
+        constexpr bool EDGE = decltype(edge)::value;
 #pragma unroll 1
-      for (int j = 0; j < AR; j += AB) {
-        float s[AB], dp[AB];
-        dot_tile<HDP, AB>(s, q, ta, j, sub);
-        dot_tile<HDP, AB>(dp, g, tb, j, sub);
+        for (int j = 0; j < AR; j += AB) {
+          float s[AB], dp[AB];
+          dot_tile<HDP, AB>(s, q, ta, j, sub);
+          dot_tile<HDP, AB>(dp, g, tb, j, sub);
 #pragma unroll
-        for (int u = 0; u < AB; ++u) s[u] = j0 + j + u <= i ? expf(s[u] - L) * (dp[u] - D) : 0.f;
-        axpy_tile<HDP, AB>(dq, s, ta, j, sub);
-      }
+          for (int u = 0; u < AB; ++u) s[u] = expf(s[u] - L) * (dp[u] - D);
+          axpy_tile<HDP, AB, EDGE>(dq, s, ta, j, sub, 0, i + 1 - j0 - j);
+        }
+      };
+      if (j0 < i0) keys(std::false_type{});
+      else keys(std::true_type{});
     }
     scale_row<HDP>(dq, scale);
     if (ROPE) rotate_row<HDP>(dq, tq, -1.f);
@@ -311,19 +329,24 @@ __global__ void __launch_bounds__(AR * kLpr<HDP>) attn_bwd_k(const T* __restrict
       __syncthreads();
       if (i0 + AR < S) fetch(h, i0 + AR);
       else if (hh + 1 < rep) fetch(h + 1, j0);
+      auto queries = [&](auto edge) {   // the tile's queries, on the diagonal and at the end (edge) those from the key on that exist
+        constexpr bool EDGE = decltype(edge)::value;
 #pragma unroll 1
-      for (int i = 0; i < AR; i += AB) {
-        float s[AB], dp[AB];
-        dot_tile<HDP, AB>(s, k, ta, i, sub);
-        dot_tile<HDP, AB>(dp, v, tb, i, sub);
+        for (int i = 0; i < AR; i += AB) {
+          float s[AB], dp[AB];
+          dot_tile<HDP, AB>(s, k, ta, i, sub);
+          dot_tile<HDP, AB>(dp, v, tb, i, sub);
 #pragma unroll
-        for (int u = 0; u < AB; ++u) {
-          s[u] = i0 + i + u >= j ? expf(s[u] - sl[i + u]) : 0.f;
-          dp[u] = s[u] * (dp[u] - sd[i + u]);
+          for (int u = 0; u < AB; ++u) {
+            s[u] = expf(s[u] - sl[i + u]);
+            dp[u] = s[u] * (dp[u] - sd[i + u]);
+          }
+          axpy_tile<HDP, AB, EDGE>(dv, s, tb, i, sub, j - i0 - i, S - i0 - i);
+          axpy_tile<HDP, AB, EDGE>(dk, dp, ta, i, sub, j - i0 - i, S - i0 - i);
         }
-        axpy_tile<HDP, AB>(dv, s, tb, i, sub);
-        axpy_tile<HDP, AB>(dk, dp, ta, i, sub);
-      }
+      };
+      if (j0 < i0 && i0 + AR <= S) queries(std::false_type{});
+      else queries(std::true_type{});
     }
   }
   scale_row<HDP>(dk, scale);

@@ -100,6 +100,37 @@ def test_fp32_attention_keeps_nan(B, nan_keys, hd):
     assert bool(out.isnan().all()) and bool(lse.isnan().all())
 
 
+# NaN or Inf in one token's query, key, value or output gradient reaches the rows that read it and, causally, no others: the
+# rest is what it is without (first and last rows of 32-row tiles and of the sequence).
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("S,t,hd", [(70, 3, 32), (70, 31, 30), (70, 32, 64), (70, 69, 32), (64, 63, 128), (33, 32, 66)])
+@pytest.mark.parametrize("where", ["q", "k", "v", "dout"])
+def test_fp32_attention_causal_nonfinite(B, where, S, t, hd, bad):
+    H, Hkv, h = 4, 2, 1   # query head 1 and KV head 0, which heads 0 and 1 read
+    g = torch.Generator(device="cuda").manual_seed(S + t + hd)
+    qkv, dout = torch.randn(S, (H + 2 * Hkv) * hd, device="cuda", generator=g), torch.randn(S, H * hd, device="cuda", generator=g)
+    clean = [x.clone() for x in _f32_attention(B, qkv, dout, S, H, Hkv, hd)]
+    if where == "dout":
+        dout[t, h * hd + 1] = bad
+    else:
+        qkv[t, {"q": h, "k": H, "v": H + Hkv}[where] * hd + 1] = bad
+    out, lse, dqkv = _f32_attention(B, qkv, dout, S, H, Hkv, hd)
+    i = torch.arange(S, device="cuda")
+    # rows of (out, lse, dQ) of the heads, and of (dK, dV) of the KV heads, that the bad row may reach
+    none, later, own, upto = i < 0, i >= t, i == t, i <= t
+    heads = [h] if where in ("q", "dout") else [0, 1]
+    o, l, dq, dk, dv = {"q": (own, own, own, upto, upto), "k": (later, later, later, i >= 0, i >= 0), "v": (later, none, later, i >= 0, none),
+                        "dout": (none, none, own, upto, upto)}[where]
+    for name, got, ref, hs, rows in (("out", out, clean[0], heads, o), ("lse", lse, clean[1], heads, l), ("dq", dqkv[:, :H], clean[2][:, :H], heads, dq),
+                                     ("dk", dqkv[:, H:H + Hkv], clean[2][:, H:H + Hkv], [0], dk),
+                                     ("dv", dqkv[:, H + Hkv:], clean[2][:, H + Hkv:], [0], dv)):
+        may = torch.zeros(got.shape[:2], dtype=torch.bool, device="cuda")
+        may[:, hs] = rows[:, None]
+        assert torch.equal(got[~may], ref[~may]), name
+    if bad != bad:   # (an infinite key may also be a score of -inf, a weight of zero)
+        assert bool(out[o][:, heads].isnan().any(-1).all()) and bool(dqkv[dq][:, heads].isnan().any(-1).all())
+
+
 # Heads of 32 are rotated inside the fp32 attention kernels: training steps against the float64 oracle, with the
 # loss and per-tensor tolerances of the other fp32 parity tests (1e-4).
 @pytest.mark.parametrize("seq,kv", [(50, 2), (33, 1), (31, 4)])
