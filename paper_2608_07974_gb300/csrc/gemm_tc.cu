@@ -909,7 +909,7 @@ bool run_tc(int mode, int M, int N, int K, const void* A, const void* B, void* C
   if (!tc::init()) return false;
   if (M < 16 || N < 16 || K < 16) return false;
   auto al16 = [](const void* p) { return ((uintptr_t)p & 15u) == 0; };
-  if (!al16(A) || !al16(B) || !al16(C) || (R && !al16(R))) return false;
+  if (!al16(A) || !al16(B) || !al16(C) || (R && !al16(R)) || (bias && !al16(bias))) return false;   // all read 16 bytes at a time
   // the fused update: 16-byte aligned state rows, a compute copy, no accumulated gradient
   if (u && (!al16(u->theta) || !al16(u->m) || !al16(u->v) || u->g || !u->comp || !al16(u->comp) || N % 8 != 0 ||
             (u->blk && (M % 16 != 0 || N % 32 != 0))))

@@ -134,6 +134,22 @@ def test_gemm_fused_epilogue(B, monkeypatch, dtype, mode, r_mode, with_bias, til
     assert err <= (1e-2 if dtype == "bf16" else 1e-5), err
 
 
+# A bias that does not start on 16 bytes (part of a larger tensor) runs on the CUDA-core kernel, also where the plan has splits.
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("off", [1, 2, 3])
+def test_gemm_bias_off_16_bytes(B, mode, off):
+    M, N, K = 130, 136, 200
+    g = torch.Generator(device="cuda").manual_seed(off)
+    a = torch.randn(M, K, device="cuda", generator=g).bfloat16()
+    b = torch.randn(*((N, K) if mode == 0 else (K, N)), device="cuda", generator=g).bfloat16()
+    bias = torch.randn(N + off, device="cuda", generator=g)[off:]
+    ref = a.double() @ (b.double().T if mode == 0 else b.double()) + bias.double()
+    c = torch.full((M, N), float("nan"), device="cuda", dtype=torch.bfloat16)
+    B.zl_op_gemm_ex(1, mode, M, N, K, a, b, c, bias=bias)
+    # one rounding to bf16 (2^-8 of a value's power of two) over fp32 sums of K products
+    assert bool(((c.double() - ref).abs() <= 2.0 ** -8 * ref.abs() + 1e-4).all())
+
+
 # dW with the bias gradient: C += A^T B (tensor-core GEMM for bf16 under the default and forced tiles,
 # CUDA cores for fp32) and db += column sums of A (the column-sum kernel of the bias gradients).
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
