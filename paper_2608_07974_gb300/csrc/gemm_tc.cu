@@ -915,8 +915,8 @@ bool run_tc(int mode, int M, int N, int K, const void* A, const void* B, void* C
             (u->blk && (M % 16 != 0 || N % 32 != 0))))
     return false;
   if (N % 8 != 0) return false;
-  // the rotation: bf16 C without residual, whole heads of 64 or 128 columns from column 0
-  if (rope && (mode != 0 || R || !rope->cs || ((uintptr_t)rope->cs & 7u) || (rope->hd != 64 && rope->hd != 128) ||
+  // the rotation: bf16 C without residual, whole heads of 64 or 128 columns from column 0, a table read 16 bytes at a time
+  if (rope && (mode != 0 || R || !rope->cs || !al16(rope->cs) || (rope->hd != 64 && rope->hd != 128) ||
                rope->S < 1 || rope->cols < 0 || rope->cols % rope->hd != 0 || rope->cols > N))
     return false;
   if ((mode == 0 || mode == 1) && K % 8 != 0) return false;

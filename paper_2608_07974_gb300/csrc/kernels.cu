@@ -540,7 +540,7 @@ void launch_partials_add(const float* part, int nb, int d, float* out, cudaStrea
 // RoPE (rotate-half), SwiGLU, GELU(tanh)
 // ------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void rope_k(T* __restrict__ qkv, const float2* __restrict__ cs, int N, int S, int nh, int hd,
+__global__ void rope_k(T* __restrict__ qkv, const float* __restrict__ cs, int N, int S, int nh, int hd,
                        int ld, int inverse) {
   pdl_wait();
   pdl_trigger();
@@ -551,19 +551,19 @@ __global__ void rope_k(T* __restrict__ qkv, const float2* __restrict__ cs, int N
     const int i = (int)(idx % half);
     const int hh = (int)((idx / half) % nh);
     const int n = (int)(idx / ((long)half * nh));
-    const float2 c = cs[(size_t)(n % S) * half + i];
-    const float sn = inverse ? -c.y : c.y;
+    const float* c = cs + 2 * ((size_t)(n % S) * half + i);
+    const float sn = inverse ? -c[1] : c[1];
     T* p = qkv + (size_t)n * ld + (size_t)hh * hd;
     const float x1 = to_f(p[i]), x2 = to_f(p[i + half]);
     float y1, y2;
-    rope_rot(x1, x2, c.x, sn, y1, y2);
+    rope_rot(x1, x2, c[0], sn, y1, y2);
     p[i] = from_f<T>(y1);
     p[i + half] = from_f<T>(y2);
   }
 }
 
-// Head dims with hd / 2 a multiple of 8: one thread per 8 rotation pairs (16-byte loads of both halves and
-// 64 bytes of the (cos, sin) table), blocks striding over token rows, no 64-bit index divisions.
+// Head dims with hd / 2 a multiple of 8, rows and table on 16 bytes: one thread per 8 rotation pairs (16-byte loads of
+// both halves and 64 bytes of the (cos, sin) table), blocks striding over token rows, no 64-bit index divisions.
 template <typename T>
 __global__ void rope8_k(T* __restrict__ qkv, const float2* __restrict__ cs, int N, int S, int nh, int hd, int ld,
                         int inverse) {
@@ -605,15 +605,15 @@ void launch_rope(int dt, void* qkv, const float* cs, int N, int S, int H, int Hk
 void launch_rope_heads(int dt, void* qkv, const float* cs, int N, int S, int nh, int hd, int ld, int inverse,
                        cudaStream_t s) {
   note_launch(1);
-  if (hd % 16 == 0) {
+  if (hd % 16 == 0 && (((uintptr_t)qkv | (uintptr_t)cs | (uintptr_t)ld * dt_size(dt)) & 15u) == 0) {
     const int th = 128, g = std::min(N, 152 * 16);
     if (dt == BF16) launch_pdl(rope8_k<bf16>, g, th, 0, s, (bf16*)qkv, (const float2*)cs, N, S, nh, hd, ld, inverse);
     else launch_pdl(rope8_k<float>, g, th, 0, s, (float*)qkv, (const float2*)cs, N, S, nh, hd, ld, inverse);
     return;
   }
   const int th = 256, g = grid_for((size_t)N * nh * (hd / 2), th);
-  if (dt == BF16) launch_pdl(rope_k<bf16>, g, th, 0, s, (bf16*)qkv, (const float2*)cs, N, S, nh, hd, ld, inverse);
-  else launch_pdl(rope_k<float>, g, th, 0, s, (float*)qkv, (const float2*)cs, N, S, nh, hd, ld, inverse);
+  if (dt == BF16) launch_pdl(rope_k<bf16>, g, th, 0, s, (bf16*)qkv, cs, N, S, nh, hd, ld, inverse);
+  else launch_pdl(rope_k<float>, g, th, 0, s, (float*)qkv, cs, N, S, nh, hd, ld, inverse);
 }
 
 __device__ __forceinline__ float sigmoidf_(float x) { return 1.f / (1.f + expf(-x)); }

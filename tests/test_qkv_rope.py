@@ -113,6 +113,28 @@ def test_qkv_rope_matches_two_pass_and_oracle(B, monkeypatch, dts, Bt, S, H, Hkv
     assert not bad.any(), f"{bad.sum().item()} elements off the oracle; worst {(err - u * scale).max().item():.3g}"
 
 
+# A (cos, sin) table or an output that does not start on 16 bytes (or an output row length that is not a multiple of them)
+# takes a path that reads single values; the result is that of aligned ones.
+@pytest.mark.parametrize("dts,hd,cs_off,c_off,extra", [("bf16", 128, 2, 0, 0), ("bf16", 64, 1, 0, 0), ("bf16", 64, 0, 1, 0), ("bf16", 32, 2, 0, 3),
+                                                       ("f32", 32, 1, 0, 0), ("f32", 64, 0, 1, 0), ("f32", 32, 0, 0, 2)])
+def test_qkv_rope_off_16_bytes(B, dts, hd, cs_off, c_off, extra):
+    torch.manual_seed(11)
+    dt, code = (torch.bfloat16, B.ZL_DTYPE_BF16) if dts == "bf16" else (torch.float32, B.ZL_DTYPE_F32)
+    S, H, K = 37, 3, 64
+    M, N, rot = 2 * S, 3 * H * hd + extra, 2 * H * hd
+    A, W = (torch.randn(M, K, device="cuda") / 8).to(dt), torch.randn(N, K, device="cuda").to(dt)
+
+    def off(t, n):
+        b = torch.empty(t.numel() + n, device="cuda", dtype=t.dtype)
+        b[n:] = t.flatten()
+        return b[n:].view(t.shape)
+    cs = off(_table(S, hd).cuda(), cs_off)
+    C0, C = (off(torch.zeros(M, N, device="cuda", dtype=dt), c_off) for _ in range(2))
+    B.zl_op_gemm_ex(code, 0, M, N, K, A, W, C0)
+    B.zl_op_qkv_rope(code, M, N, K, A, W, C, cs, S, hd, rot)
+    assert torch.equal(C, _two_pass(C0, cs, S, hd, rot, dt))   # the same product under both calls
+
+
 def test_qkv_rope_llama7b_projection(B, monkeypatch):
     """The 7B-shaped projection (2 x 1024 tokens, d 4096, 32 + 32 + 32 heads of 128) in one launch,
     bit for bit the two-pass composition; the oracle on 48 sampled rows (both sequences, early and late
