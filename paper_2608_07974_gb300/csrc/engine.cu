@@ -1521,6 +1521,17 @@ zl_status zl_load_weights(zl_ctx* c, const char* name, const void* src, size_t b
   return zl_set_param(c, name, src, bytes, on_device);
 }
 
+// Memory of the current device, which a kernel may write (a copy also reaches another device's and the host's).
+static bool on_current_device(const void* p) {
+  cudaPointerAttributes a = {};
+  int dev = 0;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
 zl_status zl_get_param(zl_ctx* c, const char* name, int which, void* dst, size_t bytes, int on_device) {
   if (!c || !name || !dst) { g_err = "NULL argument"; return ZL_ERR_ARG; }
   return guarded(c, [&]() -> zl_status {
@@ -1546,7 +1557,7 @@ zl_status zl_get_param(zl_ctx* c, const char* name, int which, void* dst, size_t
       for (int j = 0; j < f.trows; ++j)
         for (int o = 0; o < f.tcols; ++o) t[(size_t)o * f.trows + j] = h[(size_t)j * f.tcols + o];
       CK(cudaMemcpy(dst, t.data(), bytes, on_device ? cudaMemcpyHostToDevice : cudaMemcpyHostToHost));
-    } else if (f.brows > 0 && on_device && ((uintptr_t)dst & 15u) == 0) {   // blocked -> row-major, straight there
+    } else if (f.brows > 0 && on_device && ((uintptr_t)dst & 15u) == 0 && on_current_device(dst)) {   // blocked -> row-major
       launch_blk_permute((const float*)srcp, (float*)dst, f.brows, f.bcols, 0, 0);
       CHECK_LAUNCH();
       CK(cudaStreamSynchronize(0));

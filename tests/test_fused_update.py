@@ -132,3 +132,28 @@ def test_checkpoints_move_between_blocked_and_row_major_state():
         assert losses == ref[0], (src_kw, dst_kw)
         for key in ref[1]:
             assert torch.equal(st[key], ref[1][key]), (src_kw, dst_kw, key)
+
+
+@pytest.mark.parametrize("where", ["device", "device + 4 bytes", "pinned"])
+def test_get_param_to_device(where):
+    """zl_get_param with on_device: masters and moments, blocked and row-major, straight into this device's memory or through a copy
+    (off 16 bytes, or not device memory), the same bits as the read into host memory."""
+    import ctypes
+    from paper_2608_07974_gb300 import binding
+    w = MIXED
+    eng = engine_for(w)
+    eng.load(_params(w))
+    ids, labels = synth.make_batch(w, 0)
+    eng.step(ids.cuda(), labels.cuda())
+    fn = ctypes.CDLL(binding.LIB_PATH).zl_get_param
+    fn.argtypes = [ctypes.c_void_p, ctypes.c_char_p, ctypes.c_int, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_int]
+    for n in ("layers.0.wqkv", "layers.0.w2", "layers.1.w1", "layers.1.attn_norm.weight"):
+        for which in (0, 2, 3):
+            ref = eng.get(n, which).flatten()
+            buf = torch.full((ref.numel() + 8,), float("nan"), device="cpu" if where == "pinned" else "cuda")
+            buf = buf.pin_memory() if where == "pinned" else buf
+            off = 1 if where.endswith("bytes") else 0
+            assert fn(eng.ctx, n.encode(), which, buf[off:].data_ptr(), ref.numel() * 4, 1) == binding.ZL_OK, (n, binding.last_error())
+            assert torch.equal(buf[off:off + ref.numel()].cpu(), ref), (n, which)
+            assert bool(buf[off + ref.numel():].isnan().all()) and bool(buf[:off].isnan().all())   # and nothing beside it
+    eng.close()
