@@ -489,7 +489,7 @@ void attn_fwd(int dt, const void* qkv, void* out, float* lse, int B, int S, int 
   }
   if (dt == BF16 && attn_fwd_tcgen05(qkv, out, lse, B, S, H, Hkv, hd, s, err, scale)) return;
   if (dt == BF16 && attn_fwd_padded(qkv, out, lse, B, S, H, Hkv, hd, s, err, pool)) return;
-  note_launch(1);
+  note_launch(1);   // of the two kernels left
   if (dt == BF16 && attn_fwd_tc(qkv, out, lse, B, S, H, Hkv, hd, s)) return;
 #define CC(T)                                                                                  \
   if (hd <= 32) cuda_core_fwd<T, 32>(qkv, out, lse, B, S, H, Hkv, hd, scale, s);               \
@@ -501,15 +501,16 @@ void attn_fwd(int dt, const void* qkv, void* out, float* lse, int B, int S, int 
 
 void attn_bwd(int dt, const void* qkv, const void* out, const void* dout, const float* lse, float* Dbuf, void* dqkv,
               int B, int S, int H, int Hkv, int hd, cudaStream_t s, cudaMemPool_t pool, unsigned* err, const float* cs) {
-  note_launch(dt == BF16 ? (H > Hkv ? 3 : 2) : 1);
   const float scale = 1.f / sqrtf((float)hd);
   if (cs) {
+    note_launch(1);
     cuda_core_bwd<float, 32, true>(qkv, out, dout, lse, dqkv, B, S, H, Hkv, hd, scale, s, cs);
     return;
   }
   if (dt == BF16 && attn_bwd_tcgen05(qkv, out, dout, lse, Dbuf, dqkv, B, S, H, Hkv, hd, s, pool, err, scale)) return;
   if (dt == BF16 && attn_bwd_padded(qkv, out, dout, lse, Dbuf, dqkv, B, S, H, Hkv, hd, s, pool, err)) return;
   if (dt == BF16 && attn_bwd_tc(qkv, out, dout, lse, Dbuf, dqkv, B, S, H, Hkv, hd, s, pool)) return;
+  note_launch(1);
 #define CC(T)                                                                                        \
   if (hd <= 32) cuda_core_bwd<T, 32>(qkv, out, dout, lse, dqkv, B, S, H, Hkv, hd, scale, s);         \
   else if (hd <= 64) cuda_core_bwd<T, 64>(qkv, out, dout, lse, dqkv, B, S, H, Hkv, hd, scale, s);    \

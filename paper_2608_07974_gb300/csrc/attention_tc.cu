@@ -627,6 +627,7 @@ void bwd_t(const void* qkv, const void* out, const void* dout, const float* lse,
   dim3 gk(part ? H : Hkv, B, (S + BR - 1) / BR);
   launch_pdl(bwd_dkv_k<HDP>, gk, NT, smem, s, (const bf16*)qkv, (const bf16*)dout, lse, D, (bf16*)dqkv, S, H, Hkv, hd, scale,
                                       part);
+  note_launch(part ? 3 : 2);
   if (part) {
     const size_t total = (size_t)B * S * Hkv * (hd / 2);
     const int blocks = (int)std::min<size_t>((total + 255) / 256, 152 * 16);

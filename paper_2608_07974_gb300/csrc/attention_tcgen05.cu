@@ -1221,7 +1221,9 @@ bool bwd_launch(const void* qkv, const void* out, const void* dout, const float*
     if (e == cudaSuccess) launch_reduce_dkv(part, dqkv, B * S, H, Hkv, shares, HD, scale, s);
     cudaFreeAsync(part, s);
   }
-  return e == cudaSuccess;
+  if (e != cudaSuccess) return false;
+  note_launch(part ? 3 : 2);
+  return true;
 }
 
 template <int HD>
@@ -1236,8 +1238,10 @@ bool fwd_launch(const void* qkv, void* out, float* lse, int B, int S, int H, int
   }
   CUtensorMap mq, mo;
   if (!qkv_map(&mq, qkv, B, S, (H + 2 * Hkv) * HD, C_::KB) || !qkv_map(&mo, out, B, S, H * HD, 32)) return false;
-  return launch_pdl(kern, dim3(H, B, (S + QB - 1) / QB), C_::NTHR, C_::SMEM, s, mq, mo, lse, S, H, Hkv, scale, err) ==
-         cudaSuccess;
+  if (launch_pdl(kern, dim3(H, B, (S + QB - 1) / QB), C_::NTHR, C_::SMEM, s, mq, mo, lse, S, H, Hkv, scale, err) != cudaSuccess)
+    return false;
+  note_launch(1);
+  return true;
 }
 
 }  // namespace tg
@@ -1250,7 +1254,6 @@ bool attn_fwd_tcgen05(const void* qkv, void* out, float* lse, int B, int S, int 
   if (hd != 64 && hd != 128) return false;
   if ((((uintptr_t)qkv | (uintptr_t)out) & 15u) || B > 65535 || (S + 127) / 128 > 65535) return false;
   if (!tg::enc_init()) return false;
-  note_launch(1);
   return hd == 64 ? tg::fwd_launch<64>(qkv, out, lse, B, S, H, Hkv, s, err, scale)
                   : tg::fwd_launch<128>(qkv, out, lse, B, S, H, Hkv, s, err, scale);
 }

@@ -14,7 +14,7 @@ def B():
 
 
 # One block exactly, one row more and one less, a last block of one row; grouped heads whose dK / dV kernel takes
-# one, several or all query heads of a KV head in one CTA (with 152 SMs: 1 of 2, 2 of 4, 4 of 4, 2 of 8, 8 of 8).
+# all query heads of a KV head in one CTA.
 @pytest.mark.parametrize("Bb,S,H,Hkv,hd", [(2, 127, 2, 2, 64), (2, 128, 2, 2, 128), (1, 129, 2, 1, 128), (3, 256, 3, 3, 64),
                                            (1, 257, 2, 2, 64), (1, 385, 2, 2, 128), (16, 200, 32, 8, 64),
                                            (40, 129, 32, 8, 128), (16, 257, 32, 4, 128), (8, 641, 64, 8, 64)])
@@ -50,6 +50,13 @@ def test_attention_block_edges(B, Bb, S, H, Hkv, hd):
 @pytest.mark.parametrize("S,hd", [(2, 64), (63, 128), (64, 64), (65, 128), (191, 64), (193, 64), (193, 128)])
 def test_attention_key_blocks(B, S, hd):
     test_attention_block_edges(B, 2, S, 2, 1, hd)
+
+
+# Grouped heads whose dK / dV kernel takes one or several query heads of a KV head in one CTA and sums the partials afterwards
+# (with 152 SMs: 1 of 2, 2 of 4, 2 of 8, 4 of 8).
+@pytest.mark.parametrize("Bb,S,H,Hkv,hd", [(1, 257, 2, 1, 128), (16, 385, 8, 2, 64), (8, 513, 16, 2, 64), (8, 641, 16, 2, 128)])
+def test_attention_head_shares(B, Bb, S, H, Hkv, hd):
+    test_attention_block_edges(B, Bb, S, H, Hkv, hd)
 
 
 @pytest.mark.parametrize("S,hd", [(300, 64), (450, 128)])
@@ -96,3 +103,18 @@ def test_attention_first_maximum(B, S, hd):
     got = out.double().view(S, 2, hd)[key:]
     bound = 2.0 ** (torch.floor(torch.log2(ref)) - 8) + 2.0 ** -8 * w2 * 2.0 + 1e-5
     assert bool(((got - ref).abs() <= bound).all()), float(((got - ref).abs() / bound).max())
+
+
+# The launch counter: one kernel forward and two backward (one each in fp32), a reduction where a KV head's query heads lie in
+# several CTAs, two and four copies more where heads are padded to 64 or 128.
+@pytest.mark.parametrize("dt,Bb,S,H,Hkv,hd,fwd,bwd", [(1, 2, 100, 4, 4, 64, 1, 2), (1, 1, 257, 2, 1, 128, 1, 3), (1, 40, 129, 32, 8, 128, 1, 2),
+                                                      (1, 8, 513, 16, 2, 64, 1, 3), (1, 2, 100, 4, 4, 50, 3, 6), (0, 2, 100, 4, 2, 64, 1, 1)])
+def test_attention_launch_count(B, dt, Bb, S, H, Hkv, hd, fwd, bwd):
+    td = torch.bfloat16 if dt else torch.float32
+    qkv, out = torch.randn(Bb * S, (H + 2 * Hkv) * hd, device="cuda").to(td), torch.empty(Bb * S, H * hd, device="cuda", dtype=td)
+    lse, n0 = torch.empty(Bb, H, S, device="cuda"), B.zl_kernel_launches()
+    B.zl_op_attention(dt, qkv, out, lse, Bb, S, H, Hkv, hd)
+    n1 = B.zl_kernel_launches()
+    B.zl_op_attention_bwd(dt, qkv, out, torch.randn_like(out), lse, torch.empty_like(qkv), Bb, S, H, Hkv, hd)
+    torch.cuda.synchronize()
+    assert (n1 - n0, B.zl_kernel_launches() - n1) == (fwd, bwd)
