@@ -339,9 +339,9 @@ void G(zl_ctx* c, cudaStream_t s, int mode, int M, int N, int K, const void* A, 
 }
 // Weight gradient of matrix p of layer li: C += A^T B into its gradient accumulator, or, with the fused
 // update on (k.fuse: one micro-batch per window), the AdamW step of the matrix in the product's epilogue,
-// with no gradient stored. Where the tensor-core product does not apply (fp32, or a shape outside its
-// rules) the gradient is formed with gemm() in the accumulator and the step applied to the matrix's
-// range right after it: the same arithmetic either way.
+// with no gradient stored (bf16: gemm_tc_update, fp32: gemm_f32_update). Where neither takes the shape or the
+// alignment the gradient is formed with gemm() in the accumulator and the step applied to the matrix's range
+// right after it: the same arithmetic either way.
 void GW(zl_ctx* c, cudaStream_t s, Chunk& k, int li, PK p, int M, int N, int K, const void* A, const void* B) {
   if (!trainable(k, li, p)) return;   // frozen
   float* g = Gm(k, li, p);
@@ -483,9 +483,9 @@ void G_lora(zl_ctx* c, cudaStream_t s, int mode, int M, int N, int K, const void
 }
 
 // One linear of the layer forward, out = X W^T (+ bias) (+ R), with LoRA on it (Delta w = s B A, Section II-A): u = s X
-// A^T is kept for the backward, out += u B^T.
+// A^T is kept for the backward (have_u: it is there already), out += u B^T.
 void linear_fwd(zl_ctx* c, Chunk& k, int li, int i, const void* X, void* out, const float* bias, const void* R, void* u,
-                int N, cudaStream_t s) {
+                int N, cudaStream_t s, bool have_u = false) {
   const Layer& L = k.layers[li];
   const void* W = Wc(c, k, li, (PK)kLoraP[i]);
   const int in = L.lin_in[i], o = L.lin_out[i];
@@ -493,7 +493,7 @@ void linear_fwd(zl_ctx* c, Chunk& k, int li, int i, const void* X, void* out, co
     G(c, s, 0, N, o, in, X, W, out, bias, R);
     return;
   }
-  lora_down(c, X, TrainC(c, k, L.la[i]), u, N, in, c->cfg.lora_scale, s);
+  if (!have_u) lora_down(c, X, TrainC(c, k, L.la[i]), u, N, in, c->cfg.lora_scale, s);
   G_lora(c, s, 0, N, o, in, X, W, out, bias, R, u, TrainC(c, k, L.lb[i]));
 }
 
@@ -521,7 +521,8 @@ void layer_fwd(zl_ctx* c, Chunk& k, int li, LayerSave& sv, const void* x, void* 
   // Llama: RoPE in the QKV product's epilogue (bf16; after the LoRA term, which is part of the product) or as the
   // attention kernels load queries and keys (fp32); otherwise a RoPE pass after the product
   bool rotated = false;
-  if (c->llama && dt == BF16) {
+  const bool try_rot = c->llama && dt == BF16;
+  if (try_rot) {
     const int r16 = lora_r16(c->cfg.lora_rank);
     const Layer& L = k.layers[li];
     if (r16 > 0) lora_down(c, sv.xn1, TrainC(c, k, L.la[0]), sv.u[0], N, c->d, c->cfg.lora_scale, s);
@@ -535,7 +536,7 @@ void layer_fwd(zl_ctx* c, Chunk& k, int li, LayerSave& sv, const void* x, void* 
     p.keep = rotated;
   }
   if (!rotated) {
-    linear_fwd(c, k, li, 0, sv.xn1, sv.qkv, Wm(k, li, P_BQKV), nullptr, sv.u[0], N, s);
+    linear_fwd(c, k, li, 0, sv.xn1, sv.qkv, Wm(k, li, P_BQKV), nullptr, sv.u[0], N, s, try_rot);
     if (c->llama && !attn_rope(c)) {
       ProfScope p(c, s, PC_ELEM, 0, 2.0 * esz(c) * (double)N * (c->H + c->Hkv) * c->hd);
       launch_rope(dt, sv.qkv, c->rope_cs, N, S, c->H, c->Hkv, c->hd, 0, s);

@@ -41,3 +41,23 @@ def test_lora_gradients(arch, rank, heads, kv, hd, batch, seq):
 @pytest.mark.parametrize("batch,seq", [(10, 251), (5, 255), (3, 200)])
 def test_lora_gradients_many_tokens(batch, seq):
     test_lora_gradients(synth.ARCH_LLAMA, 16, 2, 1, 64, batch, seq)
+
+
+# Where the product does not rotate (head dim 50) the forward forms the same products as where it does (64): a RoPE pass and the
+# head padding's two copies more, and nothing twice.
+def test_lora_forward_launches():
+    from paper_2608_07974_gb300 import binding
+    counts = []
+    for hd in (64, 50):
+        d = synth.ModelDims(synth.ARCH_LLAMA, 1, 4 * hd, 4, 4, 328, 640, 64)
+        w = synth.Workload("lora-launches", d, "bf16", batch=2, seq=64, K=1, steps=1, seed=7)
+        P = synth.make_params(d, w.seed)
+        P.update(synth.make_lora_params(d, w.seed, 8, b_std=0.05))
+        eng = engine_for(w, lora_rank=8, lora_scale=2.0)
+        eng.load({n: (synth.round_bf16(t) if t.dim() == 2 else t) for n, t in P.items()})
+        h = torch.randn(128, 4 * hd, device="cuda").to(torch.bfloat16)
+        n0 = binding.zl_kernel_launches()
+        eng.forward_chunk(1, h, None, 2, 64)
+        counts.append(binding.zl_kernel_launches() - n0)
+        eng.close()
+    assert counts[1] - counts[0] == 3, counts
