@@ -849,13 +849,18 @@ struct Plan {
 // The plan with the least predicted time (us): a fixed cost (launch, set-up, first loads), then waves of units
 // (a tile, or a pair's two, times K / splits) on 152 SMs (76 pairs, or 304 slots of width 64), each 64-deep k
 // block of a unit at the rate measured for its kernel and no wave shorter than a tile's epilogue, the last
-// wave's epilogue, and for splits the fp32 partials through HBM and 4 us for the reduction with its launch and the
-// workspace's allocation (2 us, the reduction alone, lost where a small product is one of a sequence: a linear of 412
-// tokens, 2176 x 800, forward, dX and dW 36.4 us against 30.9; 694, 1728 x 5504 66 against 59). Fitted to every plan on 53
+// wave's epilogue, and for splits the fp32 partials through HBM and 3 us for the reduction with its launch and the
+// workspace's allocation. Fitted to every plan on 53
 // shapes (4096^3, the GPT-2, 1.1B and 7B layer and head shapes, ragged ones from 203 rows): 8% off at the
 // median of both sides, the chosen plan within 4% of the fastest one on all but a few small shapes. Pairs win wherever
 // their 256-row tiles fill the SMs (7B QKV forward 117 us against 131 alone; 4096^3 79.5 against 94); single
-// CTAs win where those tiles would leave SMs idle (4096 x 768 x 768 9.3 against 9.9). mode 4 (fused update):
+// CTAs win where those tiles would leave SMs idle (4096 x 768 x 768 9.3 against 9.9). An operand whose rows are not
+// whole 128-byte lines (an extent that is no multiple of 64 along memory) makes a k block 15 to 35% slower, by the
+// share of the block's bytes that it has; pairs, which copy half as much of B, lose least. Forward, dX and dW of a
+// linear in one sequence, us: 282 tokens, 2400 -> 1624 40.4 -> 32.3 (the term and the 3 us for a split; 4 us, fitted
+// where the host's launches were the bound, kept such products whole), 312, 1768 -> 928 32.5 -> 26.8, 375, 1576 -> 1336
+// 36.8 -> 35.7, 1498, 840 -> 2144 49.7 -> 48.6; 70, 2384 -> 1016, whose launches are the bound, 25.9 -> 29.3; 130
+// linears and heads 0.6% faster. mode 4 (fused update):
 // a unit's epilogue streams its optimizer state, which is its time when the products are short. Its split count is
 // mode 2's, so the fused and the unfused update sum the gradient in the same order (the tile does not matter).
 Plan choose(int mode, int M, int N, int K) {
@@ -868,6 +873,7 @@ Plan choose(int mode, int M, int N, int K) {
                                {64, 0, 0.330, 0.6}};
   const double hbm = 6.0e6;                  // bytes / us
   const bool dw = mode == 2 || mode == 4;    // both operands MN-major
+  const double off_a = (dw ? M : K) % 64 != 0, off_b = (mode == 0 ? K : N) % 64 != 0;   // rows off 128-byte lines
   const int nk = (K + BK - 1) / BK;
   const double state = mode == 4 ? 26.0 * M * N : 0.0;
   double best = 1e30;
@@ -879,6 +885,8 @@ Plan choose(int mode, int M, int N, int K) {
     const long tiles = c.pair ? (tm + 1) / 2 * tn : tm * tn;
     const long slots = c.pair ? g_sms / 2 : (long)g_sms * (c.bn == 64 ? 2 : 1);
     // the update's epilogue per unit: 26 bytes for each element of a CTA's tile at about 85 bytes per ns and SM
+    const double nb = c.pair ? c.bn / 2 : c.bn;   // a CTA copies 128 rows of A and these of B per k block
+    const double kb = c.kb * (dw ? 1.06 : 1.0) * (1.0 + 0.3 * (BM * off_a + nb * off_b) / (BM + nb));
     const double epi = c.epi + (mode == 4 ? 26.0 * BM * c.bn / 85e3 : 0.0);
     for (int sp : {1, 2, 3, 4, 6, 8}) {
       if (sp > 1 && nk / sp < 4) continue;
@@ -886,8 +894,8 @@ Plan choose(int mode, int M, int N, int K) {
       const int kps = (nk + sp - 1) / sp;
       const long waves = (tiles * sp + slots - 1) / slots;
       const double e = sp > 1 ? c.epi : epi;
-      double t = 2.8 + waves * std::max(kps * c.kb * (dw ? 1.06 : 1.0), e) + e;
-      if (sp > 1) t += (8.0 * sp * M * N + state) / hbm + 4.0;
+      double t = 2.8 + waves * std::max(kps * kb, e) + e;
+      if (sp > 1) t += (8.0 * sp * M * N + state) / hbm + 3.0;
       else t = std::max(t, state / hbm + 2.8);
       if (t < best * 0.98) { best = t; p = Plan{c.bn, sp, c.pair}; }
     }
