@@ -300,9 +300,10 @@ bool run_f32(int M, int N, int K, const float* A, const float* B, float* C, cons
   const bool rows_ok = MODE == 0 ? K % 4 == 0 : MODE == 1 ? K % 4 == 0 && N % 4 == 0 : M % 4 == 0 && N % 4 == 0;
   if (!rows_ok || !al16(A) || !al16(B) || M < 1 || N < 1 || K < 1 || (M + 31) / 32 > 65535) return false;
   const long t64 = (long)((M + 63) / 64) * ((N + 63) / 64), t32 = (long)((M + 31) / 32) * ((N + 31) / 32);
-  if (t64 >= 304) return launch_f32<MODE, 64, UPD>(M, N, K, A, B, C, ep, 1, s);
+  const long sms = sm_count();
+  if (t64 >= 2 * sms) return launch_f32<MODE, 64, UPD>(M, N, K, A, B, C, ep, 1, s);
   int ks = 1;
-  while (ks < 4 && t32 * ks * 2 <= 304 && K / (ks * 2) >= 64) ks *= 2;
+  while (ks < 4 && t32 * ks * 2 <= 2 * sms && K / (ks * 2) >= 64) ks *= 2;
   return launch_f32<MODE, 32, UPD>(M, N, K, A, B, C, ep, ks, s);
 }
 }  // namespace

@@ -12,6 +12,17 @@
 
 namespace zl {
 
+int sm_count() {
+  static const int n = [] {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      cudaGetLastError();
+    return std::max(v, 1);
+  }();
+  return n;
+}
+
 static inline int grid_for(size_t work, int threads, int max_blocks = 152 * 16) {
   size_t b = (work + threads - 1) / threads;
   if (b < 1) b = 1;

@@ -238,16 +238,6 @@ __global__ void __launch_bounds__(32 * RW) rank16_grad_k(const bf16* __restrict_
   if (nz > 1) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-int sm_count() {
-  static const int n = [] {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      cudaGetLastError();
-    return std::max(v, 1);
-  }();
-  return n;
-}
 bool al16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 template <int MT>

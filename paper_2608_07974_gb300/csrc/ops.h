@@ -17,6 +17,7 @@ inline void set_last_error(const std::string& msg) { set_last_error(msg.c_str())
 
 // Count of kernels launched by the library (process-wide).
 void note_launch(int n);
+int sm_count();   // of the device that is current at the first call
 unsigned long long launches_so_far();
 
 // h_0 = E[ids] (+ P[s]); bad ids set ZL_DEVERR_BAD_ID in *err and give a zero row.
