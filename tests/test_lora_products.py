@@ -5,7 +5,7 @@ import pytest
 import torch
 
 import synth
-from tests.gpu_common import cosine, engine_for, oracle_for, rel
+from tests.gpu_common import cosine, engine_for, fro_rel, oracle_for, rel
 
 pytestmark = pytest.mark.gpu
 
@@ -61,3 +61,35 @@ def test_lora_forward_launches():
         counts.append(binding.zl_kernel_launches() - n0)
         eng.close()
     assert counts[1] - counts[0] == 3, counts
+
+
+# The product with the LoRA term as further k blocks under every kind of plan (tiles of 64, 128, 256, CTA pairs with an odd tile row
+# at the end, splits whose last share is the term alone), both modes, with the rotation in the epilogue and without.
+@pytest.mark.parametrize("tile", ["64:1", "128:1:0", "128:1:1", "256:1:0", "256:1:1", "64:4", "128:4:0", "128:4:1", "256:3:1"])
+@pytest.mark.parametrize("rank,hd", [(16, 64), (70, 64), (16, 50), (70, 128)])
+def test_lora_every_plan(monkeypatch, tile, rank, hd):
+    batch, seq = 3, 107   # 321 tokens: three tile rows
+    d = synth.ModelDims(synth.ARCH_LLAMA, 1, 4 * hd, 4, 2, 328, 640, 128)
+    w = synth.Workload("lora-plans", d, "bf16", batch=batch, seq=seq, K=1, steps=1, seed=79)
+    P = synth.make_params(d, w.seed)
+    P.update(synth.make_lora_params(d, w.seed, rank, b_std=0.05))
+    P = {n: (synth.round_bf16(t) if t.dim() == 2 else t) for n, t in P.items()}
+    kw = dict(accum_m=2, lora_rank=rank, lora_scale=1.0)   # the term is about a third of the layer's output
+    eng = engine_for(w, **kw)
+    eng.load(P)
+    ids, labels = synth.make_batch(w, 0)
+    monkeypatch.setenv("ZL_GEMM_TILE", tile)
+    loss = eng.step(ids.cuda(), labels.cuda())[0]
+    h = eng.embed(ids.cuda())
+    y = eng.forward_chunk(1, h, None, batch, seq)
+    monkeypatch.delenv("ZL_GEMM_TILE")
+    orc = oracle_for(w, P, dtype=torch.float32, **kw)
+    h = h.float().cpu().view(batch, seq, -1)
+    L, g, ref = orc.local_grad(1, h, labels)
+    # about ten roundings to bf16 (2^-8 / sqrt(3) of a value in the mean, at most half of it on average) lie before each gradient,
+    # four before each output: 7e-3 and 5e-3; a wrong or missing term is 0.1 to 1
+    assert rel(loss, L) <= 1e-3
+    assert fro_rel(y.float().cpu().view(batch, seq, -1) - h, ref - h) <= 1e-2
+    for n in orc.chunk_names(1):
+        assert fro_rel(eng.get(n, 1), g[n]) <= 1.5e-2, n
+    eng.close()
