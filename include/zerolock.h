@@ -202,7 +202,9 @@ zl_status zl_read_losses(zl_ctx* ctx, float* losses_out, int n);
 /* Make the stream given to zl_set_stream wait for all queued work (no host wait). */
 zl_status zl_join(zl_ctx* ctx);
 
-/* Wait for all queued work, polling; ZL_ERR_TIMEOUT after timeout_ms (< 0: no limit).
+/* Wait for all queued work; ZL_ERR_TIMEOUT after timeout_ms, polled every 50 us (< 0: no limit; the
+ * CUDA runtime then waits, as in every call that returns a loss or a tensor, which keeps the calling
+ * thread's core busy unless the process has set cudaDeviceScheduleBlockingSync).
  * Also reports device-side argument errors (ids or labels out of range) of that work. */
 zl_status zl_synchronize(zl_ctx* ctx, int timeout_ms);
 

@@ -128,16 +128,18 @@ __device__ __forceinline__ void store_rows(uint32_t t, float f, uint8_t* st, con
 // a move. At the end O / l is the softmax-weighted sum and m + log2 l the row's log-sum-exp.
 // The first maximum is taken over two blocks, so that the largest of a row's first 128 probabilities is 1, which
 // bf16 holds without rounding: the maximum of 64 keys alone makes the result's error against 64 bits 0.75% larger
-// (2.045e-3 -> 2.060e-3 at B 2, S 1024, 32 heads of 128; 2.072e-3 -> 2.087e-3 at S 2048), for 0.9, 1.0 and 3 us less
-// at the shapes of GPT-2 (forward and backward 43.5 us), 7B (94.9) and B 4, S 2048 (379). l gathers a sum per block.
+// (2.045e-3 -> 2.060e-3 at B 2, S 1024, 32 heads of 128; 2.072e-3 -> 2.087e-3 at S 2048) and the forward 0.7 us
+// faster at the shapes of GPT-2 (10.8 of 11.5) and 7B (20.5 of 21.2), 2.4 at B 4, S 2048 (92.3 of 94.7): the second
+// block's product and reading are waited for before the first exponential. The first block kept in registers beside
+// the second (168 registers) 94.9 and 21.8, K loaded a block ahead of V 94.3 and 21.2. l gathers a sum per block.
 //
 // Two score buffers: S of the next block is formed under this block's softmax, and two CTAs per SM (256 TMEM
 // columns and at most 113 KB of shared memory each) fill each other's gaps. What bounds it: the softmax warps, two
 // an SM quarter, whose block (about 1,450 cycles, of which 256 are the exponentials) is a chain of TMEM read,
 // maximum, exponentials, TMEM write and hand-off. Measured against one score buffer of 128 keys and two softmax warps
-// per quadrant (which fit beside it): B 4, S 2048, 32 / 4 heads of 64 103 -> 92 us (743 TFLOP/s); B 2, S 1024, 32
-// heads of 128 22.7 -> 20.8 us (827 TFLOP/s); B 1, S 4096 1,250 -> 1,260 TFLOP/s. On the same blocks: three buffers
-// at head dim 64 93 us; two warps per quadrant, half a row each, 100 us; two groups of warps on alternate
+// per quadrant (which fit beside it), all with the maximum of the first block alone: B 4, S 2048, 32 / 4 heads of 64
+// 103 -> 92 us; B 2, S 1024, 32 heads of 128 22.7 -> 20.5 us; as it is 94.7 (726 TFLOP/s) and 21.2 (810), B 1, S 4096
+// 110 us (1,245). On the same blocks: three buffers at head dim 64 93 us; two warps per quadrant, half a row each, 100 us; two groups of warps on alternate
 // blocks, each with an O of its own, 98 us; one buffer and three CTAs 95 us.
 // ==============================================================================================
 template <int HD>

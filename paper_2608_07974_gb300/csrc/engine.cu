@@ -1008,7 +1008,7 @@ zl_status sync_all(zl_ctx* c, int timeout_ms) {
   CK(cudaMemcpyAsync(c->h_err, c->d_err, 4, cudaMemcpyDeviceToHost, c->user));
   rec(c->ev_sync, c->user);
   // without a limit the runtime waits (and sees the end at once: polling with a sleep cost 50-120 us a call, which
-  // every read of a loss or a tensor paid); with one, polling
+  // every read of a loss or a tensor paid; by the device's flags, so by default it spins); with one, polling
   if (timeout_ms < 0) CK(cudaEventSynchronize(c->ev_sync));
   const auto t0 = std::chrono::steady_clock::now();
   while (timeout_ms >= 0) {
