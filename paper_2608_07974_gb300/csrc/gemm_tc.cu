@@ -859,11 +859,13 @@ struct Plan {
 // share of the block's bytes that it has; pairs, which copy half as much of B, lose least. Forward, dX and dW of a
 // linear in one sequence, us: 282 tokens, 2400 -> 1624 40.4 -> 32.3 (the term and the 3 us for a split; 4 us, fitted
 // where the host's launches were the bound, kept such products whole), 312, 1768 -> 928 32.5 -> 26.8, 375, 1576 -> 1336
-// 36.8 -> 35.7, 1498, 840 -> 2144 49.7 -> 48.6; 70, 2384 -> 1016, whose launches are the bound, 25.9 -> 29.3; 130
-// linears and heads 0.6% faster. mode 4 (fused update):
+// 36.7 -> 35.7, 1498, 840 -> 2144 49.7 -> 48.6; 70, 2384 -> 1016, whose launches are the bound, 24.0 -> 27.3; 210 drawn
+// linears 1.2% faster in the mean, for terms of 0.2 to 0.4 and splits of 3 to 4 us alike. mode 4 (fused update):
 // a unit's epilogue streams its optimizer state, which is its time when the products are short. Its split count is
 // mode 2's, so the fused and the unfused update sum the gradient in the same order (the tile does not matter).
-Plan choose(int mode, int M, int N, int K) {
+// rotates: tiles of whole heads, one split (a plan among splits that it may not have took 73 us instead of 61 for
+// 142 tokens, 6496 -> 1920).
+Plan choose(int mode, int M, int N, int K, bool rotates = false) {
   const int same_splits = mode == 4 ? choose(2, M, N, K).splits : 0;
   struct Kind {
     int bn, pair;
@@ -879,7 +881,7 @@ Plan choose(int mode, int M, int N, int K) {
   double best = 1e30;
   Plan p{128, 1, 0};
   for (const Kind& c : kinds) {
-    if (mode == 4 && c.bn == 64) continue;
+    if ((mode == 4 || rotates) && c.bn == 64) continue;
     if (c.pair && M <= BM) continue;   // nothing to pair
     const long tm = (M + BM - 1) / BM, tn = (N + c.bn - 1) / c.bn;
     const long tiles = c.pair ? (tm + 1) / 2 * tn : tm * tn;
@@ -889,7 +891,7 @@ Plan choose(int mode, int M, int N, int K) {
     const double kb = c.kb * (dw ? 1.06 : 1.0) * (1.0 + 0.3 * (BM * off_a + nb * off_b) / (BM + nb));
     const double epi = c.epi + (mode == 4 ? 26.0 * BM * c.bn / 85e3 : 0.0);
     for (int sp : {1, 2, 3, 4, 6, 8}) {
-      if (sp > 1 && nk / sp < 4) continue;
+      if (sp > 1 && (nk / sp < 4 || rotates)) continue;
       if (same_splits && sp != same_splits) continue;
       const int kps = (nk + sp - 1) / sp;
       const long waves = (tiles * sp + slots - 1) / slots;
@@ -931,7 +933,7 @@ bool run_tc(int mode, int M, int N, int K, const void* A, const void* B, void* C
   if (mode >= 2 && M % 8 != 0) return false;
   if (ext && (mode > 1 || ext->K2 < 16 || ext->K2 % 8 != 0 || !ext->A2 || !ext->B2 || !al16(ext->A2) || !al16(ext->B2)))
     return false;
-  const tc::Plan plan = tc::choose(mode, M, N, K);
+  const tc::Plan plan = tc::choose(mode, M, N, K, rope != nullptr);
   int bn = plan.bn, splits = plan.splits, pair = plan.pair;
   if (const char* force = std::getenv("ZL_GEMM_TILE")) {   // test hook "BN:SPLITS[:PAIR]": forces the plan
     int fb = 0, fs = 0, fp = -1;
@@ -943,7 +945,7 @@ bool run_tc(int mode, int M, int N, int K, const void* A, const void* B, void* C
       if (nf == 3 && (fp == 0 || fp == 1)) pair = fp && bn >= 128 ? 1 : 0;
     }
   }
-  if (rope) {   // one split (the reduction does not rotate); tiles of 128 or 256 columns (heads never straddle)
+  if (rope) {   // also of a forced plan: one split (the reduction does not rotate), tiles of 128 or 256 columns (heads never straddle)
     splits = 1;
     if (bn < 128) bn = 128;
   }
