@@ -131,9 +131,9 @@ def roofline_of(prof, workload="llama7b"):
 GEMM_SOURCES = ["gemm_tc.cu", "tcgen05.cuh"]
 TRAFFIC = {
     "llama7b": {
-        "gemm_layer": {"sources": GEMM_SOURCES, "sha256": "59cb3733891c1c4d", "bytes_per_launch": 182912416.0},
-        "gemm_head": {"sources": GEMM_SOURCES, "sha256": "59cb3733891c1c4d", "bytes_per_launch": 471975047.5},
-        "gemm_update": {"sources": GEMM_SOURCES, "sha256": "59cb3733891c1c4d", "bytes_per_launch": 1397520192.0},
+        "gemm_layer": {"sources": GEMM_SOURCES, "sha256": "b438f0c733eabf21", "bytes_per_launch": 182084608.0},
+        "gemm_head": {"sources": GEMM_SOURCES, "sha256": "b438f0c733eabf21", "bytes_per_launch": 469645342.1},
+        "gemm_update": {"sources": GEMM_SOURCES, "sha256": "b438f0c733eabf21", "bytes_per_launch": 1397478656.0},
     },
 }
 
