@@ -21,7 +21,11 @@
 
 namespace zl {
 static std::atomic<unsigned long long> g_launches{0};
-void note_launch(int n) { g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed); }
+static thread_local long t_launches = 0;   // this thread's, for the profile
+void note_launch(int n) {
+  g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed);
+  t_launches += n;
+}
 unsigned long long launches_so_far() { return g_launches.load(std::memory_order_relaxed); }
 }  // namespace zl
 
@@ -383,13 +387,17 @@ const float* attn_rope(const zl_ctx* c) { return c->llama && attn_rotates(c->dt,
 void AF(zl_ctx* c, cudaStream_t s, const void* qkv, void* out, float* lse, int B, int S) {
   const double e = (double)esz(c), N = (double)B * S;
   ProfScope p(c, s, PC_ATTN_F, 2.0 * B * c->H * (double)S * S * c->hd, e * N * (c->qkvw + c->ad));
+  const long n0 = t_launches;
   attn_fwd(c->dt, qkv, out, lse, B, S, c->H, c->Hkv, c->hd, s, c->d_err, c->pool, attn_rope(c));
+  p.launches = (double)(t_launches - n0);
 }
 void AB(zl_ctx* c, cudaStream_t s, const void* qkv, const void* out, const void* dout, const float* lse, float* D,
         void* dqkv, int B, int S) {
   const double e = (double)esz(c), N = (double)B * S;
-  ProfScope p(c, s, PC_ATTN_B, 4.0 * B * c->H * (double)S * S * c->hd, e * N * (2.0 * c->qkvw + 2.0 * c->ad), 3);
+  ProfScope p(c, s, PC_ATTN_B, 4.0 * B * c->H * (double)S * S * c->hd, e * N * (2.0 * c->qkvw + 2.0 * c->ad));
+  const long n0 = t_launches;
   attn_bwd(c->dt, qkv, out, dout, lse, D, dqkv, B, S, c->H, c->Hkv, c->hd, s, c->pool, c->d_err, attn_rope(c));
+  p.launches = (double)(t_launches - n0);
 }
 void NF(zl_ctx* c, cudaStream_t s, const void* x, const float* g, const float* b, void* y, float* rstd, float* mean,
         int N) {

@@ -118,3 +118,21 @@ def test_attention_launch_count(B, dt, Bb, S, H, Hkv, hd, fwd, bwd):
     B.zl_op_attention_bwd(dt, qkv, out, torch.randn_like(out), lse, torch.empty_like(qkv), Bb, S, H, Hkv, hd)
     torch.cuda.synchronize()
     assert (n1 - n0, B.zl_kernel_launches() - n1) == (fwd, bwd)
+
+
+@pytest.mark.parametrize("hd,fwd,bwd", [(64, 1, 2), (50, 3, 6)])
+def test_attention_profile_count(B, hd, fwd, bwd):
+    """The step's profile counts the same launches."""
+    import synth
+    from tests.gpu_common import engine_for
+    d = synth.ModelDims(synth.ARCH_GPT2, 1, 4 * hd, 4, 4, 256, 300, 64)
+    w = synth.Workload("attn-profile", d, "bf16", batch=2, seq=64, K=1, steps=1, seed=3)
+    eng = engine_for(w)
+    eng.load(synth.make_params(d, w.seed))
+    ids, labels = (t.cuda() for t in synth.make_batch(w, 0))
+    eng.step(ids, labels)
+    B.zl_profile(eng.ctx, True)
+    eng.step(ids, labels)
+    p = B.zl_profile_read(eng.ctx)
+    eng.close()
+    assert (p["attn_fwd"]["launches"], p["attn_bwd"]["launches"]) == (fwd, bwd)
